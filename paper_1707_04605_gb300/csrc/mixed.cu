@@ -552,9 +552,13 @@ struct Chunk {
   }
 };
 
+// whole_groups: pad the shots so that the float4s of a node (ld4) are a power
+// of two up to 32 or a multiple of 32.  The node adjoint sums them with warp
+// shuffles over such groups; any other count would put lanes of two nodes
+// into one group and lanes outside the shuffle's mask (ld4 = 3 for 10 shots).
 int flux_setup(mg_mesh* M, const double* eps, const mg_shots* shots, const double* wavelet,
                double dt, int nt, const double* xi, const double* zeta, int flags,
-               cudaStream_t st, Scratch& X, Flux& F) {
+               cudaStream_t st, Scratch& X, Flux& F, bool whole_groups = false) {
   if (!M || !eps || !shots || !wavelet || nt < 1 || !(dt > 0.0)) return MG_ERR_ARG;
   const HostMesh* hm = host_mesh(M);
   const int d = hm->dim, k1 = d + 1;
@@ -643,6 +647,12 @@ int flux_setup(mg_mesh* M, const double* eps, const mg_shots* shots, const doubl
   }
   F.ld = S <= 4 ? 4 : ((S + 3) / 4) * 4;
   F.ld4 = F.ld / 4;
+  if (whole_groups) {
+    int g = 1;
+    while (g < F.ld4 && g < 32) g <<= 1;
+    F.ld4 = (F.ld4 + g - 1) / g * g;
+    F.ld = 4 * F.ld4;
+  }
   std::vector<int32_t> sp(n + 1, 0), ss(S), rp(n + 1, 0), rs(R), rt(R);
   const std::vector<int32_t>& perm = hm->perm;
   for (int s = 0; s < S; ++s) sp[perm[shots->src[s]] + 1]++;
@@ -872,7 +882,7 @@ extern "C" int mg_jacobian_T_apply_pml(mg_mesh* M, int level, const double* eps,
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   Scratch X(st);
   Flux F;
-  MG_FX(flux_setup(M, eps, shots, wavelet, dt, nt, xi, zeta, flags, st, X, F));
+  MG_FX(flux_setup(M, eps, shots, wavelet, dt, nt, xi, zeta, flags, st, X, F, true));
   const int64_t n = F.n, m = F.m, R = F.R, nc = hm->n_cells_level[level];
   const int K = std::min(ckpt_every, nt);
   const int nck = (nt + K - 1) / K;
