@@ -17,6 +17,7 @@
 #include "kernels.cuh"
 #include "mg_internal.h"
 #include "mesh_view.h"
+#include "resident.h"
 
 namespace {
 
@@ -123,6 +124,7 @@ struct mg_mesh {
     int stream = 0;       // row kernels: once-read loads bypass L1 allocation
     int prefetch = 0;     // capped row kernels: prefetch of late-loaded rows (1 L1, 2 L2)
     int wide = 1;         // capped forward: 8 consecutive shots per lane (256-bit loads)
+    int shaped = 0;       // a launch shape was asked for: no resident kernel in its place
   } tune[3];
   int dep_launch = 1;                     // row kernels launched as programmatic dependents
   Buf ellu;                               // ELL with every slice padded to wu columns
@@ -145,6 +147,19 @@ struct mg_mesh {
   };
   std::map<int, TileTables> tiles;        // by rows per tile
   int smem_optin = 0;
+  int n_sm = 0;
+  // partitions of the resident kernels by patch count, their row groups by rows
+  // per warp
+  struct PatchTables {
+    mg::HostPatches host;
+    struct Groups {
+      Buf grp_off, border, pair_off, halo_off, x_off, hdr, row, halo, halo_x, diag, pair;
+      mg::DevPatches dev{};
+    };
+    std::map<int, Groups> groups;
+  };
+  std::map<int, PatchTables> patches;
+  Buf xbuf;                               // resident kernels: exchange of border rows
   // autotuned choices by (n_shots padded), so repeated calls skip the search
   std::map<int, std::array<Tuning, 3>> tuned;
   cudaStream_t cap = nullptr;             // private capture stream
@@ -595,12 +610,151 @@ int persist_status(mg_mesh* M, cudaStream_t st) {
   return MG_ERR_TIMEOUT;
 }
 
+// Device tables of the partition into B patches with rpw rows per warp,
+// built on first use.
+int patch_tables(mg_mesh* M, int B, int rpw, mg::DevPatches& D) {
+  auto it = M->patches.find(B);
+  if (it == M->patches.end()) {
+    mg::HostPatches H;
+    MG_TRY(mg::build_patches(M->hm, B, H));
+    it = M->patches.emplace(B, mg_mesh::PatchTables()).first;
+    it->second.host = std::move(H);
+  }
+  mg_mesh::PatchTables& T = it->second;
+  auto ig = T.groups.find(rpw);
+  if (ig == T.groups.end()) {
+    mg::HostGroups G;
+    mg::group_rows(M->hm, T.host, rpw, G);
+    mg_mesh::PatchTables::Groups& R = T.groups[rpw];
+    MG_TRY(upload(R.grp_off, G.grp_off));
+    MG_TRY(upload(R.border, G.border));
+    MG_TRY(upload(R.pair_off, G.pair_off));
+    MG_TRY(upload(R.halo_off, G.halo_off));
+    MG_TRY(upload(R.x_off, G.x_off));
+    MG_TRY(upload(R.hdr, G.hdr));
+    MG_TRY(upload(R.row, G.row));
+    MG_TRY(upload(R.halo, G.halo));
+    MG_TRY(upload(R.halo_x, G.halo_x));
+    MG_TRY(upload(R.diag, G.diag));
+    MG_TRY(upload(R.pair, G.pair));
+    mg::DevPatches& d = R.dev;
+    d.n_x = G.x_off[B];
+    d.max_pairs = G.max_pairs;
+    d.max_groups = G.max_groups;
+    d.uniform = G.uniform;
+    d.max_halo = G.max_halo;
+    d.max_slots = G.max_slots;
+    d.grp_off = P_<const int32_t>(R.grp_off);
+    d.border = P_<const int32_t>(R.border);
+    d.pair_off = P_<const int32_t>(R.pair_off);
+    d.halo_off = P_<const int32_t>(R.halo_off);
+    d.x_off = P_<const int32_t>(R.x_off);
+    d.hdr = P_<const int32_t>(R.hdr);
+    d.row = P_<const int32_t>(R.row);
+    d.halo = P_<const int32_t>(R.halo);
+    d.halo_x = P_<const int32_t>(R.halo_x);
+    d.diag = P_<const float>(R.diag);
+    d.pair = P_<const int4>(R.pair);
+    d.B = B;   // set last: the tables are complete
+    ig = T.groups.find(rpw);
+  }
+  D = ig->second.dev;
+  return D.B ? MG_OK : MG_ERR_OOM;
+}
+
+// Resident launch shape of a call that advances S_pad columns for `steps`
+// steps: the widest column group whose patches fit.  shape.lpr = 0: the row
+// kernels are the path.
+int resident_shape(mg_mesh* M, int kind, int S_pad, int steps, mg::DevPatches& D,
+                   mg::ResidentShape& shape) {
+  shape = mg::ResidentShape();
+  const mg_mesh::Tuning& t = M->tune[kind];
+  if (t.shaped || steps < 16) return MG_OK;
+  if (!M->n_sm)
+    MG_CU(cudaDeviceGetAttribute(&M->n_sm, cudaDevAttrMultiProcessorCount, M->device));
+  const int B = (int)std::min<int64_t>(M->n_sm, std::max<int64_t>(1, M->hm.n / 32));
+  if (M->hm.max_row_nnz > 256) return MG_OK;
+  for (int lpr = std::min(S_pad, 128) / 4; lpr >= 1; lpr >>= 1) {
+    // the states alone too large: no tables needed to see it
+    if (M->hm.n / B * (int64_t)lpr * 32 > M->smem_optin) continue;
+    MG_TRY(patch_tables(M, B, 32 / lpr, D));
+    if (mg::resident_fit(D, lpr, M->smem_optin - 1024, shape) == MG_OK) return MG_OK;
+    shape = mg::ResidentShape();
+  }
+  return MG_OK;
+}
+
+// Exchange buffer and status word of resident launches.
+int resident_buffers(mg_mesh* M, const mg::DevPatches& D, int lpr, cudaStream_t st,
+                     mg::ResidentArgs& r) {
+  MG_TRY(ensure(M->xbuf, (size_t)2 * D.n_x * lpr * 2 * sizeof(uint4)));
+  r.status = err_word(M);
+  if (!r.status) return MG_ERR_OOM;
+  MG_CU(cudaMemsetAsync(r.status, 0, sizeof(int), st));
+  r.xbuf = P<uint4>(M->xbuf);
+  r.budget = M->persist_budget;
+  return MG_OK;
+}
+
+// Steps [0, nt) with the resident kernel, one launch per column group and
+// checkpoint interval.  Checkpoints as run_forward's; hist: slot j of it
+// receives p_{j-1} (slots 0 and 1 zero).  MG_ERR_UNSUPPORTED before anything
+// has run when the device cannot hold the launch.
+int run_forward_resident(mg_mesh* M, const Prep& pp, int nt, float* traces, int ckpt_every,
+                         float* ckpt, float* hist, const mg::DevPatches& D,
+                         const mg::ResidentShape& shape, cudaStream_t st) {
+  const size_t state = (size_t)M->hm.n * pp.S_pad;
+  mg::ResidentArgs r{};
+  r.P = D;
+  r.ev = pp.ev;
+  r.coef = P<const float4>(M->coef);
+  r.wavelet = P<const float>(M->wavf);
+  r.traces = traces;
+  r.nt = nt;
+  r.ld = pp.S_pad;
+  r.state = (int64_t)state;
+  MG_TRY(resident_buffers(M, D, shape.lpr, st, r));
+  if (hist) MG_CU(cudaMemsetAsync(hist, 0, 2 * state * sizeof(float), st));
+  if (ckpt) MG_CU(cudaMemsetAsync(ckpt, 0, 2 * state * sizeof(float), st));
+  const int len = ckpt ? ckpt_every : nt;
+  for (int l = 0; l < nt; l += len) {
+    r.step0 = l;
+    r.steps = std::min(len, nt - l);
+    float* slot = ckpt && l ? ckpt + (size_t)(l / len) * 2 * state : nullptr;
+    float* next = ckpt && l + len < nt ? ckpt + (size_t)(l / len + 1) * 2 * state : nullptr;
+    r.p = slot;
+    r.pm = slot ? slot + state : nullptr;
+    r.out_p = next;
+    r.out_pm = next ? next + state : nullptr;
+    r.hist = hist ? hist + (size_t)(l + 2) * state : nullptr;
+    for (r.col0 = 0; r.col0 < pp.S_pad; r.col0 += 4 * shape.lpr) {
+      MG_TRY(mg::launch_resident_step(r, shape, st));
+      M->launches += 1;
+    }
+  }
+  if (traces) {
+    MG_TRY(mg::launch_poison(traces, pp.R * nt, r.status, st));
+    M->launches += 1;
+  }
+  return MG_OK;
+}
+
 // Batched forward loop over steps [0, nt); optional traces and checkpoints.
 // Whole chunks of M->chunk steps run as one graph launch each.
 int run_forward(mg_mesh* M, const Prep& pp, int nt, float* traces, int ckpt_every,
                 float* ckpt, cudaStream_t st, int flags) {
   const int64_t n = M->hm.n;
   const size_t state = (size_t)n * pp.S_pad;
+  if (!(flags & MG_PERSISTENT)) {
+    mg::DevPatches D;
+    mg::ResidentShape shape;
+    MG_TRY(resident_shape(M, 0, pp.S_pad, ckpt ? std::min(ckpt_every, nt) : nt, D, shape));
+    if (shape.lpr) {
+      const int rc =
+          run_forward_resident(M, pp, nt, traces, ckpt_every, ckpt, nullptr, D, shape, st);
+      if (rc != MG_ERR_UNSUPPORTED) return rc;
+    }
+  }
   MG_TRY(ensure(M->stA, state * sizeof(float)));
   MG_TRY(ensure(M->stB, state * sizeof(float)));
   float* p = P<float>(M->stA);
@@ -696,6 +850,13 @@ int run_forward(mg_mesh* M, const Prep& pp, int nt, float* traces, int ckpt_ever
 int run_forward_states(mg_mesh* M, const Prep& pp, int nt, float* traces, float* seg,
                        cudaStream_t st, int flags) {
   const size_t state = (size_t)M->hm.n * pp.S_pad;
+  mg::DevPatches D;
+  mg::ResidentShape shape;
+  MG_TRY(resident_shape(M, 0, pp.S_pad, nt, D, shape));
+  if (shape.lpr) {
+    const int rc = run_forward_resident(M, pp, nt, traces, 0, nullptr, seg, D, shape, st);
+    if (rc != MG_ERR_UNSUPPORTED) return rc;
+  }
   MG_CU(cudaMemsetAsync(seg, 0, 2 * state * sizeof(float), st));
   mg::StepArgs a = step_args(M, pp, pp.S_pad, nt);
   a.traces = traces;
@@ -856,6 +1017,14 @@ void mg_mesh_destroy(mg_mesh* M) {
     for (Buf* b : {&D.ell_off, &D.ell_idx, &D.ell_val, &D.sinfo, &D.halo_off, &D.halo_cnt, &D.halo})
       if (b->p) cudaFree(b->p);
   }
+  for (auto& kv : M->patches) {
+    for (auto& g : kv.second.groups) {
+      mg_mesh::PatchTables::Groups& R = g.second;
+      for (Buf* b : {&R.grp_off, &R.border, &R.pair_off, &R.halo_off, &R.x_off, &R.hdr, &R.row,
+                     &R.halo, &R.halo_x, &R.diag, &R.pair})
+        if (b->p) cudaFree(b->p);
+    }
+  }
   mg_mesh_trim(M);
   if (M->cap) cudaStreamDestroy(M->cap);
   delete M;
@@ -870,7 +1039,7 @@ int mg_mesh_trim(mg_mesh* M) {
   Buf* all[] = {&M->eps_h, &M->wav_h, &M->wavf, &M->coef, &M->tcoef, &M->mass, &M->scal,
                 &M->stA, &M->stB, &M->stC, &M->stD, &M->out_h, &M->w_h, &M->v_h, &M->g_h,
                 &M->ev, &M->G, &M->ckpt, &M->seg, &M->gfine, &M->step_base, &M->tr,
-                &M->trf, &M->tune_scratch};
+                &M->trf, &M->tune_scratch, &M->xbuf};
   for (Buf* b : all) {
     if (b->p) cudaFree(b->p);
     b->p = nullptr;
@@ -947,6 +1116,7 @@ static void drop_graphs(mg_mesh* M) {
 }
 
 static void apply_tuning(mg_mesh::Tuning& t, int batch, int tile_rows, int src_tile) {
+  if (batch != -1 || tile_rows != -1 || src_tile != -1) t.shaped = 1;
   if (batch != -1) t.batch = batch;
   if (tile_rows != -1) t.tile_rows = tile_rows;
   if (src_tile != -1) t.src_tile = src_tile;
@@ -974,7 +1144,10 @@ int mg_mesh_set_shot_groups(mg_mesh* M, int kind, int groups) {
     return MG_ERR_ARG;
   drop_graphs(M);
   for (int k = 0; k < 3; ++k)
-    if (kind == -1 || kind == k) M->tune[k].groups = groups;
+    if (kind == -1 || kind == k) {
+      M->tune[k].groups = groups;
+      M->tune[k].shaped = 1;
+    }
   return MG_OK;
 }
 
@@ -1084,6 +1257,7 @@ int mg_mesh_set_bulk_copies(mg_mesh* M, int on) {
   if (!M || (on != 0 && on != 1)) return MG_ERR_ARG;
   drop_graphs(M);
   M->tune[0].bulk = on;
+  M->tune[0].shaped = 1;
   return MG_OK;
 }
 
@@ -1103,7 +1277,10 @@ int mg_mesh_set_gather_ring(mg_mesh* M, int kind, int depth) {
   if (!M || kind < -1 || kind > 2 || (depth != 0 && depth != 4 && depth != 8)) return MG_ERR_ARG;
   drop_graphs(M);
   for (int k = 0; k < 3; ++k)
-    if (kind == -1 || kind == k) M->tune[k].ring = depth;
+    if (kind == -1 || kind == k) {
+      M->tune[k].ring = depth;
+      M->tune[k].shaped = 1;
+    }
   return MG_OK;
 }
 
@@ -1111,6 +1288,7 @@ int mg_mesh_set_row_sweep(mg_mesh* M, int blocks) {
   if (!M || blocks < 0 || blocks > 65536) return MG_ERR_ARG;
   drop_graphs(M);
   M->tune[0].sweep = blocks;
+  M->tune[0].shaped = 1;
   return MG_OK;
 }
 
@@ -1158,6 +1336,7 @@ int mg_mesh_set_tma_tiles(mg_mesh* M, int rows) {
   if (!M || rows < 0 || rows > 1024 || rows % mg::kSliceH) return MG_ERR_ARG;
   drop_graphs(M);
   M->tune[0].tma = rows;
+  M->tune[0].shaped = 1;
   return MG_OK;
 }
 
@@ -1185,6 +1364,7 @@ int mg_mesh_set_min_blocks(mg_mesh* M, int min_blocks) {
   if (!M || (min_blocks != 0 && min_blocks != 5)) return MG_ERR_ARG;
   drop_graphs(M);
   M->tune[0].min_blocks = min_blocks;
+  M->tune[0].shaped = 1;
   return MG_OK;
 }
 
@@ -1194,6 +1374,7 @@ int mg_mesh_set_kernel_min_blocks(mg_mesh* M, int kind, int min_blocks) {
     return MG_ERR_ARG;
   drop_graphs(M);
   M->tune[kind].min_blocks = min_blocks;
+  M->tune[kind].shaped = 1;
   return MG_OK;
 }
 
@@ -1889,9 +2070,10 @@ int mg_autotune(mg_mesh* M, const double* eps, const mg_shots* shots, const doub
   if (rc == MG_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = MG_ERR_CUDA;
   // the L1 policy is the caller's setting, not a candidate
   const int l1[3] = {M->tune[0].stream, M->tune[1].stream, M->tune[2].stream};
-  auto time_of = [&](int kind, mg_mesh::Tuning c, float* out) -> int {
+  auto time_of = [&](int kind, mg_mesh::Tuning c, float* out, int shaped = 1) -> int {
     drop_graphs(M);
     c.stream = l1[kind];
+    c.shaped = shaped;
     M->tune[kind] = c;
     int r = run(kind);  // warm-up: tile tables, buffers, graphs
     float cand = 1e30f;
@@ -1950,6 +2132,17 @@ int mg_autotune(mg_mesh* M, const double* eps, const mg_shots* shots, const doub
         if (rc != MG_OK) break;
         if (t < best * 0.99f) { best = t; pick = c; }   // groups must win by more than 1%
       }
+    }
+    pick.shaped = 1;
+    // the resident kernel, where the problem fits it, against the best of these
+    mg::DevPatches D;
+    mg::ResidentShape shape;
+    M->tune[kind] = mg_mesh::Tuning();
+    if (rc == MG_OK) rc = resident_shape(M, kind, S_pad, steps, D, shape);
+    if (rc == MG_OK && shape.lpr && kind == 0) {
+      float t = 0.0f;
+      rc = time_of(kind, pick, &t, 0);
+      if (t < best) pick.shaped = 0;
     }
     M->tune[kind] = pick;
   }

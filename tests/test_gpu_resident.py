@@ -1,0 +1,90 @@
+"""The resident kernels (states on chip for many steps, patches exchanging their
+border rows) against the row kernels, which an explicit launch shape selects:
+the same bits over meshes, boundary conditions, row orders, shot counts from one
+to several column groups, odd step counts, checkpoints and the kept history; and
+a wait that runs out shows as NaN results and MG_ERR_TIMEOUT."""
+import numpy as np
+import pytest
+
+from helpers import oracle_dt
+from workloads import configs, shots as shots_mod
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def mg(cuda_device):
+    import paper_1707_04605_gb300 as mg
+
+    return mg
+
+
+def _dev(x, dtype=torch.float64):
+    return torch.as_tensor(np.ascontiguousarray(x), dtype=dtype, device="cuda")
+
+
+def _pair(mg, w, order="morton", bc=None):
+    """The handle as created (resident kernels) and one with a row shape."""
+    a, b = (mg.mesh_from_workload(w, order=order, bc=bc) for _ in range(2))
+    b.set_tuning(-1, 1, 0, 32)
+    return a, b
+
+
+CASES = [
+    (configs.tiny_2d, dict(nt=41), "none", "dirichlet"),
+    (configs.tiny_3d, dict(nt=40), "rcm", "neumann"),
+    (configs.square_disc_2d, dict(nt=333), "rcm", "abc"),
+    (configs.asteroid_2d, dict(n_refine=1, S=6, nt=64), "none", "abc"),
+    (configs.asteroid_2d, dict(n_refine=2, S=37, nt=101), "morton", "abc"),
+    (configs.asteroid_2d, dict(n_refine=2, S=300, nt=33), "rcm", "neumann"),
+    (configs.asteroid_2d, dict(n_refine=3, S=200, nt=50), "morton", "abc"),
+    (configs.asteroid_2d, dict(n_refine=4, S=20, nt=40), "morton", "abc"),
+    (configs.ellipsoid_3d, dict(n_refine=1, S=24, nt=50), "morton", "abc"),
+]
+
+
+@pytest.mark.parametrize("make,kw,order,bc", CASES)
+def test_forward_carries_the_row_kernels_bits(mg, make, kw, order, bc):
+    w = make(**kw)
+    a, b = _pair(mg, w, order, bc)
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    s = _dev(w.wavelet(dt))
+    run = lambda m, **k: mg.forward(m, eps, w.shots, s, dt, **k)
+    ref = run(b)
+    n0 = a.launch_count()
+    assert torch.equal(run(a), ref)
+    assert a.launch_count() - n0 < w.nt          # several steps per launch
+    assert torch.equal(run(a, keep_checkpoints=True, ckpt_every=17), ref)
+    assert torch.equal(run(a, keep_states=True), ref)
+    assert a.device_status() == 0
+
+
+def test_many_sources_and_receivers_per_row(mg):
+    """Every shot on the same node, receivers on shared nodes, some repeated."""
+    w = configs.asteroid_2d(n_refine=1, S=5, nt=60)
+    n = w.mesh.coords.shape[0]
+    src = np.array([7, 7, 7, 1200, 7], np.int32)
+    rec = np.array([7, 7, 5, 1200, 5, 5, 9, n - 1, 0, 7], np.int32)
+    w.shots = shots_mod.Shots(src, np.array([0, 3, 3, 6, 8, 10], np.int64), rec)
+    a, b = _pair(mg, w)
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    s = _dev(w.wavelet(dt))
+    assert torch.equal(mg.forward(a, eps, w.shots, s, dt), mg.forward(b, eps, w.shots, s, dt))
+
+
+def test_a_wait_that_runs_out_is_loud(mg):
+    from paper_1707_04605_gb300 import _lib as L
+
+    w = configs.asteroid_2d(n_refine=2, S=37, nt=200)
+    a, b = _pair(mg, w)
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    s = _dev(w.wavelet(dt))
+    a.set_persistent(wait_cycles=1000)           # below one exchange of border rows
+    y = mg.forward(a, eps, w.shots, s, dt)
+    assert bool(torch.isnan(y).all())
+    assert a.device_status() == L.MG_ERR_TIMEOUT
+    a.set_persistent()
+    assert torch.equal(mg.forward(a, eps, w.shots, s, dt), mg.forward(b, eps, w.shots, s, dt))
+    assert a.device_status() == 0
