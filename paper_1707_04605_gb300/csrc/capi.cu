@@ -160,6 +160,7 @@ struct mg_mesh {
   };
   std::map<int, PatchTables> patches;
   Buf xbuf;                               // resident kernels: exchange of border rows
+  bool status_clear = false;              // the running call cleared the status word for them
   // autotuned choices by (n_shots padded), so repeated calls skip the search
   std::map<int, std::array<Tuning, 3>> tuned;
   cudaStream_t cap = nullptr;             // private capture stream
@@ -345,6 +346,7 @@ int* err_word(mg_mesh* M);
 int prepare(mg_mesh* M, const double* eps, const mg_shots* shots, const double* wavelet,
             double dt, int nt, int flags, cudaStream_t st, Prep& pp) {
   if (!eps || !wavelet || nt < 1 || !(dt > 0.0) || !std::isfinite(dt)) return MG_ERR_ARG;
+  M->status_clear = false;
   MG_TRY(validate_shots(M, shots));
   pp.S = shots->n_shots;
   pp.S_pad = round_pad(pp.S);
@@ -663,36 +665,97 @@ int patch_tables(mg_mesh* M, int B, int rpw, mg::DevPatches& D) {
 }
 
 // Resident launch shape of a call that advances S_pad columns for `steps`
-// steps: the widest column group whose patches fit.  shape.lpr = 0: the row
-// kernels are the path.
+// steps (launch, tables and exchange buffer cost about 10 us: at least 16 of
+// them).  Forward: the widest column group whose patches fit; tangent: the
+// same with p and dp as columns (2 lpr shots per launch); adjoint: whole source
+// tiles of the row kernel only, for the same sums over the shots.
+// shape.lpr = 0: the row kernels are the path (nothing fits, or a launch shape
+// of theirs was asked for).
 int resident_shape(mg_mesh* M, int kind, int S_pad, int steps, mg::DevPatches& D,
                    mg::ResidentShape& shape) {
   shape = mg::ResidentShape();
-  const mg_mesh::Tuning& t = M->tune[kind];
-  if (t.shaped || steps < 16) return MG_OK;
+  if (M->tune[kind].shaped || steps < 16 || M->hm.max_row_nnz > 256) return MG_OK;
   if (!M->n_sm)
     MG_CU(cudaDeviceGetAttribute(&M->n_sm, cudaDevAttrMultiProcessorCount, M->device));
   const int B = (int)std::min<int64_t>(M->n_sm, std::max<int64_t>(1, M->hm.n / 32));
-  if (M->hm.max_row_nnz > 256) return MG_OK;
-  for (int lpr = std::min(S_pad, 128) / 4; lpr >= 1; lpr >>= 1) {
-    // the states alone too large: no tables needed to see it
-    if (M->hm.n / B * (int64_t)lpr * 32 > M->smem_optin) continue;
-    MG_TRY(patch_tables(M, B, 32 / lpr, D));
-    if (mg::resident_fit(D, lpr, M->smem_optin - 1024, shape) == MG_OK) return MG_OK;
-    shape = mg::ResidentShape();
+  const int widest = kind == 1 ? std::min(32, S_pad / 2) : std::min(S_pad, 128) / 4;
+  const int row_bytes = kind == 1 ? 8 : kind == 2 ? 16 : 0;
+  for (int lpr = widest; lpr >= (kind == 1 ? 2 : 1); lpr >>= 1) {
+    // where the states alone are too large no tables are needed to see it
+    if (M->hm.n / B * (int64_t)lpr * 32 <= M->smem_optin) {
+      MG_TRY(patch_tables(M, B, 32 / lpr, D));
+      if (mg::resident_fit(D, lpr, row_bytes, M->smem_optin - 1024, shape) == MG_OK) return MG_OK;
+      shape = mg::ResidentShape();
+    }
+    if (kind == 2) return MG_OK;
   }
   return MG_OK;
 }
 
-// Exchange buffer and status word of resident launches.
-int resident_buffers(mg_mesh* M, const mg::DevPatches& D, int lpr, cudaStream_t st,
-                     mg::ResidentArgs& r) {
+// Exchange buffer and status word (cleared once per call) of resident launches.
+template <class A>
+int resident_buffers(mg_mesh* M, const mg::DevPatches& D, int lpr, cudaStream_t st, A& r) {
   MG_TRY(ensure(M->xbuf, (size_t)2 * D.n_x * lpr * 2 * sizeof(uint4)));
   r.status = err_word(M);
   if (!r.status) return MG_ERR_OOM;
-  MG_CU(cudaMemsetAsync(r.status, 0, sizeof(int), st));
+  if (!M->status_clear) MG_CU(cudaMemsetAsync(r.status, 0, sizeof(int), st));
+  M->status_clear = true;
   r.xbuf = P<uint4>(M->xbuf);
   r.budget = M->persist_budget;
+  return MG_OK;
+}
+
+mg::ResidentArgs resident_args(mg_mesh* M, const Prep& pp, int nt, const mg::DevPatches& D) {
+  mg::ResidentArgs r{};
+  r.P = D;
+  r.ev = pp.ev;
+  r.coef = P<const float4>(M->coef);
+  r.wavelet = P<const float>(M->wavf);
+  r.nt = nt;
+  r.steps = nt;
+  r.ld = pp.S_pad;
+  r.state = (int64_t)M->hm.n * pp.S_pad;
+  return r;
+}
+
+// p_{l+1} .. p_{l+steps} of the states p_l, p_{l-1} into hist (state floats
+// apart), every column group.
+int run_recompute_resident(mg_mesh* M, const Prep& pp, int nt, int l, int steps, const float* p,
+                           const float* pm, float* hist, const mg::DevPatches& D,
+                           const mg::ResidentShape& shape, cudaStream_t st) {
+  mg::ResidentArgs r = resident_args(M, pp, nt, D);
+  MG_TRY(resident_buffers(M, D, shape.lpr, st, r));
+  r.step0 = l;
+  r.steps = steps;
+  r.p = p;
+  r.pm = pm;
+  r.hist = hist;
+  for (r.col0 = 0; r.col0 < pp.S_pad; r.col0 += 4 * shape.lpr) {
+    MG_TRY(mg::launch_resident_step(r, shape, st));
+    M->launches += 1;
+  }
+  return MG_OK;
+}
+
+// The tangent (and with traces or hist the forward it rides on) from rest.
+int run_tangent_resident(mg_mesh* M, const Prep& pp, int nt, float* traces, float* dtraces,
+                         float* hist, const mg::DevPatches& D, const mg::ResidentShape& shape,
+                         cudaStream_t st) {
+  mg::ResidentArgs r = resident_args(M, pp, nt, D);
+  MG_TRY(resident_buffers(M, D, shape.lpr, st, r));
+  r.tcoef = P<const float2>(M->tcoef);
+  r.traces = traces;
+  r.dtraces = dtraces;
+  r.hist = hist;
+  for (r.col0 = 0; r.col0 < pp.S_pad; r.col0 += 2 * shape.lpr) {
+    MG_TRY(mg::launch_resident_tangent(r, shape, st));
+    M->launches += 1;
+  }
+  for (float* x : {traces, dtraces})
+    if (x) {
+      MG_TRY(mg::launch_poison(x, pp.R * nt, r.status, st));
+      M->launches += 1;
+    }
   return MG_OK;
 }
 
@@ -704,15 +767,8 @@ int run_forward_resident(mg_mesh* M, const Prep& pp, int nt, float* traces, int 
                          float* ckpt, float* hist, const mg::DevPatches& D,
                          const mg::ResidentShape& shape, cudaStream_t st) {
   const size_t state = (size_t)M->hm.n * pp.S_pad;
-  mg::ResidentArgs r{};
-  r.P = D;
-  r.ev = pp.ev;
-  r.coef = P<const float4>(M->coef);
-  r.wavelet = P<const float>(M->wavf);
+  mg::ResidentArgs r = resident_args(M, pp, nt, D);
   r.traces = traces;
-  r.nt = nt;
-  r.ld = pp.S_pad;
-  r.state = (int64_t)state;
   MG_TRY(resident_buffers(M, D, shape.lpr, st, r));
   if (hist) MG_CU(cudaMemsetAsync(hist, 0, 2 * state * sizeof(float), st));
   if (ckpt) MG_CU(cudaMemsetAsync(ckpt, 0, 2 * state * sizeof(float), st));
@@ -1526,6 +1582,16 @@ int mg_jacobian_apply(mg_mesh* M, int level, const double* eps, const mg_shots* 
   float* tr = P<float>(M->tr);
   const int64_t n = M->hm.n;
   const size_t state = (size_t)n * pp.S_pad;
+  if (!(flags & MG_REUSE_CHECKPOINTS)) {
+    mg::DevPatches D;
+    mg::ResidentShape shape;
+    MG_TRY(resident_shape(M, 1, pp.S_pad, nt, D, shape));
+    if (shape.lpr) {
+      const int rc = run_tangent_resident(M, pp, nt, nullptr, tr, nullptr, D, shape, st);
+      if (rc == MG_OK) return deliver(M->tr, jv, tbytes, flags, st);
+      if (rc != MG_ERR_UNSUPPORTED) return rc;
+    }
+  }
   Buf* bufs[] = {&M->stA, &M->stB, &M->stC, &M->stD};
   for (Buf* b : bufs) {
     MG_TRY(ensure(*b, state * sizeof(float)));
@@ -1678,7 +1744,33 @@ int mg_forward_jacobian_apply(mg_mesh* M, int level, const double* eps, const mg
     MG_TRY(ensure(M->seg, (size_t)(nt + 2) * state * sizeof(float)));
     seg = P<float>(M->seg);
     MG_CU(cudaMemsetAsync(seg, 0, 2 * state * sizeof(float), st));
-  } else {
+  }
+  auto finish = [&]() -> int {
+    if (keep) {
+      M->ck_valid = true;  M->ck_gen++;
+      M->seg_full = true;
+      M->ck_every = nt;
+      M->ck_nt = nt;
+      M->ck_S_pad = pp.S_pad;
+      M->ck_nshots = pp.S;
+      M->ck_dt = dt;
+      M->ck_ev_gen = M->ev_gen;
+    }
+    MG_TRY(deliver(M->trf, traces, tbytes, flags, st));
+    return deliver(M->tr, jv, tbytes, flags, st);
+  };
+  if (!(flags & MG_PERSISTENT)) {
+    mg::DevPatches D;
+    mg::ResidentShape shape;
+    MG_TRY(resident_shape(M, 1, pp.S_pad, nt, D, shape));
+    if (shape.lpr) {
+      const int rc = run_tangent_resident(M, pp, nt, trf, tr, keep ? seg + 2 * state : nullptr, D,
+                                          shape, st);
+      if (rc == MG_OK) return finish();
+      if (rc != MG_ERR_UNSUPPORTED) return rc;
+    }
+  }
+  if (!keep) {
     for (Buf* b : {&M->stA, &M->stB}) {
       MG_TRY(ensure(*b, state * sizeof(float)));
       MG_CU(cudaMemsetAsync(b->p, 0, state * sizeof(float), st));
@@ -1771,18 +1863,7 @@ int mg_forward_jacobian_apply(mg_mesh* M, int level, const double* eps, const mg
     MG_TRY(record(st));
     M->launches += (int64_t)NG * nt;
   }
-  if (keep) {
-    M->ck_valid = true;  M->ck_gen++;
-    M->seg_full = true;
-    M->ck_every = nt;
-    M->ck_nt = nt;
-    M->ck_S_pad = pp.S_pad;
-    M->ck_nshots = pp.S;
-    M->ck_dt = dt;
-    M->ck_ev_gen = M->ev_gen;
-  }
-  MG_TRY(deliver(M->trf, traces, tbytes, flags, st));
-  return deliver(M->tr, jv, tbytes, flags, st);
+  return finish();
 }
 
 int mg_jacobian_T_apply(mg_mesh* M, int level, const double* eps, const mg_shots* shots,
@@ -1873,10 +1954,66 @@ int mg_jacobian_T_apply(mg_mesh* M, int level, const double* eps, const mg_shots
     MG_TRY(ensure(M->step_base, 16));
     base = P<int32_t>(M->step_base);
   }
+  // resident kernels for the recompute and the reverse steps of a segment (not
+  // for one too short; MG_PERSISTENT asks for its own kernels)
+  mg::DevPatches Df, Da;
+  mg::ResidentShape shf, sha;
+  if (!(flags & MG_PERSISTENT)) {
+    MG_TRY(resident_shape(M, 0, pp.S_pad, std::min(ckpt_every, nt), Df, shf));
+    MG_TRY(resident_shape(M, 2, pp.S_pad, std::min(ckpt_every, nt), Da, sha));
+  }
+  mg::ResidentAdjArgs ra{};
+  if (sha.lpr) {
+    ra.P = Da;
+    ra.ev = pp.ev;
+    ra.coef = aa.coef;
+    ra.w = wd;
+    ra.nt = nt;
+    ra.ld = pp.S_pad;
+    ra.state = (int64_t)state;
+  }
+  // false: not on the resident kernel (rc says whether something failed)
+  auto resident_recompute = [&](int a, int l0, int l1, int& rc) {
+    rc = MG_OK;
+    if (!shf.lpr || l1 - l0 < 16) return false;
+    const float* slot = ck + (size_t)a * 2 * state;
+    rc = run_recompute_resident(M, pp, nt, l0, l1 - l0, slot, slot + state, seg + 2 * state, Df,
+                                shf, st);
+    if (rc != MG_ERR_UNSUPPORTED) return true;
+    rc = MG_OK;
+    shf.lpr = 0;
+    return false;
+  };
+  auto resident_reverse = [&](int l0, int l1, int& rc) {
+    rc = MG_OK;
+    if (!sha.lpr || l1 - l0 < 16) return false;
+    rc = resident_buffers(M, Da, sha.lpr, st, ra);
+    ra.mu = mu;
+    ra.mu1 = mu1;
+    ra.k = l1;
+    ra.steps = l1 - l0;
+    ra.pk = seg + (size_t)(l1 - l0 + 1) * state;
+    for (int set = 0; rc == MG_OK && set * 4 * sha.lpr < pp.S_pad; ++set) {
+      ra.col0 = set * 4 * sha.lpr;
+      ra.G = aa.G + (size_t)set * n;
+      ra.Gc = aa.Gc + (size_t)set * n;
+      ra.H = aa.H + (size_t)set * n;
+      ra.Hc = aa.Hc + (size_t)set * n;
+      rc = mg::launch_resident_adjoint(ra, sha, st);
+      M->launches += 1;
+    }
+    if (rc != MG_ERR_UNSUPPORTED) return true;   // refused before its first launch only
+    rc = MG_OK;
+    sha.lpr = 0;
+    return false;
+  };
   for (int a = nck - 1; a >= 0; --a) {
     const int l0 = a * ckpt_every;
     const int l1 = std::min(nt, l0 + ckpt_every);
-    if (!states) {
+    int rc = MG_OK;
+    const bool recomputed = !states && resident_recompute(a, l0, l1, rc);
+    MG_TRY(rc);
+    if (!states && !recomputed) {
       MG_TRY(mg::launch_copy_f4(ck + (size_t)a * 2 * state, seg + state, (int64_t)state, st));
       MG_TRY(mg::launch_copy_f4(ck + (size_t)a * 2 * state + state, seg, (int64_t)state, st));
       M->launches += 2;
@@ -1912,7 +2049,7 @@ int mg_jacobian_T_apply(mg_mesh* M, int level, const double* eps, const mg_shots
       M->launches += 1;
       const std::string kr = key_of("rec", {seg, fa.wavelet, fa.coef, fa.ev.src_ptr, base},
                                     {pp.S_pad, pp.S, pp.R, nt, ckpt_every, n, Wf});
-      if (!states) MG_TRY(run_graph(M, kr, NGf * ckpt_every, st, [&](cudaStream_t cs) {
+      if (!states && !recomputed) MG_TRY(run_graph(M, kr, NGf * ckpt_every, st, [&](cudaStream_t cs) {
         mg::StepArgs b = fa;
         b.step_base = base;
         b.cols = Wf;
@@ -1928,6 +2065,10 @@ int mg_jacobian_T_apply(mg_mesh* M, int level, const double* eps, const mg_shots
         }
         return MG_OK;
       }));
+      if (resident_reverse(l0, l1, rc)) {
+        MG_TRY(rc);
+        continue;
+      }
       const std::string ka = key_of("adj", {seg, mu, mu1, wd, aa.coef, aa.ev.rec_ptr, G, base},
                                     {pp.S_pad, pp.S, pp.R, nt, ckpt_every, n, Wa});
       MG_TRY(run_graph(M, ka, NGa * ckpt_every, st, [&](cudaStream_t cs) {
@@ -1951,7 +2092,7 @@ int mg_jacobian_T_apply(mg_mesh* M, int level, const double* eps, const mg_shots
       }));
       continue;   // even segment length: mu / mu1 are back in place
     }
-    for (int l = l0; l < l1 && !states; ++l) {
+    for (int l = l0; l < l1 && !states && !recomputed; ++l) {
       const int j = l - l0 + 1;  // slot of p_l
       fa.p = seg + (size_t)j * state;
       fa.pm = seg + (size_t)(j - 1) * state;
@@ -1959,6 +2100,10 @@ int mg_jacobian_T_apply(mg_mesh* M, int level, const double* eps, const mg_shots
       fa.step = l;
       MG_TRY(do_step(M, fa, pp.S_pad, st));
       M->launches += 1;
+    }
+    if (resident_reverse(l0, l1, rc)) {
+      MG_TRY(rc);
+      continue;
     }
     for (int g = 0; g < NGa; ++g) {
       mg::AdjointArgs b = aa;
@@ -2003,6 +2148,10 @@ int mg_jacobian_T_apply(mg_mesh* M, int level, const double* eps, const mg_shots
   MG_TRY(mg::launch_restrict(nc, P<int64_t>(M->lvl_ptr[level]), P<int32_t>(M->lvl_idx[level]),
                              ga.g_fine, P<double>(M->g_h), st));
   M->launches += 2;
+  if (M->status_clear) {   // resident launches ran: NaN if one of their waits ran out
+    MG_TRY(mg::launch_poison(P<float>(M->g_h), 2 * nc, err_word(M), st));
+    M->launches += 1;
+  }
   return deliver(M->g_h, g, nc * sizeof(double), flags, st);
 }
 
@@ -2139,7 +2288,7 @@ int mg_autotune(mg_mesh* M, const double* eps, const mg_shots* shots, const doub
     mg::ResidentShape shape;
     M->tune[kind] = mg_mesh::Tuning();
     if (rc == MG_OK) rc = resident_shape(M, kind, S_pad, steps, D, shape);
-    if (rc == MG_OK && shape.lpr && kind == 0) {
+    if (rc == MG_OK && shape.lpr) {
       float t = 0.0f;
       rc = time_of(kind, pick, &t, 0);
       if (t < best) pick.shaped = 0;

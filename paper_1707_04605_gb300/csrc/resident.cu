@@ -35,11 +35,11 @@ int resident_smem_limit(const void* kern, int smem) {
   return MG_OK;
 }
 
-int resident_fit(const DevPatches& D, int lpr, int smem_max, ResidentShape& s) {
+int resident_fit(const DevPatches& D, int lpr, int row_bytes, int smem_max, ResidentShape& s) {
   const int rpw = 32 / lpr;
   s.lpr = lpr;
-  s.smem = 2 * D.max_slots * 16 * lpr + 16 * (D.max_pairs + D.max_groups * rpw) +
-           4 * (D.max_groups * rpw + D.max_halo + D.max_groups);
+  s.smem = 2 * D.max_slots * 16 * lpr + 16 * D.max_pairs +
+           (16 + 4 + row_bytes) * D.max_groups * rpw + 4 * (D.max_halo + D.max_groups + 4);
   if (s.smem > smem_max) return MG_ERR_UNSUPPORTED;
   // a warp for each group, and at least one of each kind
   s.warps = std::min(kResidentThreads / 32, D.max_groups + 1);
@@ -48,12 +48,12 @@ int resident_fit(const DevPatches& D, int lpr, int smem_max, ResidentShape& s) {
 
 int launch_resident_step(const ResidentArgs& a, const ResidentShape& s, cudaStream_t st) {
   switch (s.lpr) {
-    case 1: return launch_lpr<1>(a, s, st);
-    case 2: return launch_lpr<2>(a, s, st);
-    case 4: return launch_lpr<4>(a, s, st);
-    case 8: return launch_lpr<8>(a, s, st);
-    case 16: return launch_lpr<16>(a, s, st);
-    case 32: return launch_lpr<32>(a, s, st);
+    case 1: return launch_lpr<1, false>(a, s, st);
+    case 2: return launch_lpr<2, false>(a, s, st);
+    case 4: return launch_lpr<4, false>(a, s, st);
+    case 8: return launch_lpr<8, false>(a, s, st);
+    case 16: return launch_lpr<16, false>(a, s, st);
+    case 32: return launch_lpr<32, false>(a, s, st);
   }
   return MG_ERR_ARG;
 }

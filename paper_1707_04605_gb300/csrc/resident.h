@@ -70,6 +70,8 @@ struct ResidentArgs {
   const float4* coef;
   const float* wavelet;
   float* traces;            // [n_traces][nt] or null
+  const float2* tcoef;      // tangent: its coefficients and the traces of dp
+  float* dtraces;
   int32_t nt, step0, steps; // steps step0 .. step0 + steps - 1
   int32_t ld, col0;         // shot columns [col0, col0 + 4 lpr) of rows of ld floats
   const float *p, *pm;      // p_l, p_{l-1} at step0, or null: zero
@@ -81,12 +83,32 @@ struct ResidentArgs {
   long long budget;         // SM clock cycles one wait may take
 };
 
-// Shape of lpr lanes per row; MG_ERR_UNSUPPORTED when a patch does not fit
-// smem_max bytes of shared memory.
-int resident_fit(const DevPatches& D, int lpr, int smem_max, ResidentShape& s);
+// Reverse steps k, k - 1, ... (`steps` of them) on the source tile of shot
+// columns [col0, col0 + 4 lpr).
+struct ResidentAdjArgs {
+  DevPatches P;
+  DevEvents ev;
+  const float4* coef;
+  const float* w;           // [n_traces][nt] trace weights
+  int32_t nt, k, steps, ld, col0;
+  float *mu, *mu1;          // mu_k, mu_{k+1}; then those after the last step
+  const float* pk;          // p_k; p_{k-j} is j * state floats before it
+  int64_t state;
+  float *G, *Gc, *H, *Hc;   // [n] sums of the tile
+  uint4* xbuf;
+  int* status;
+  long long budget;
+};
+
+// Shape of lpr lanes per row with row_bytes more bytes of shared memory per
+// own row; MG_ERR_UNSUPPORTED when a patch does not fit smem_max bytes.
+int resident_fit(const DevPatches& D, int lpr, int row_bytes, int smem_max, ResidentShape& s);
 // Raises the dynamic shared memory limit of a kernel on the current device.
 int resident_smem_limit(const void* kern, int smem);
 int launch_resident_step(const ResidentArgs& a, const ResidentShape& s, cudaStream_t st);
+// p and dp of 2 lpr shots, from rest.
+int launch_resident_tangent(const ResidentArgs& a, const ResidentShape& s, cudaStream_t st);
+int launch_resident_adjoint(const ResidentAdjArgs& a, const ResidentShape& s, cudaStream_t st);
 // x[0..n) <- NaN if *status != 0: results of a launch whose wait ran out.
 int launch_poison(float* x, int64_t n, const int* status, cudaStream_t st);
 

@@ -233,25 +233,60 @@ __device__ __forceinline__ float4 row_product(unsigned st, unsigned q, int pairs
   return acc;
 }
 
-// Sources and receivers of row r (-1: none) at step l; c0: the lane's first
-// shot column.
-__device__ __forceinline__ void resident_events(const ResidentArgs& a, int r, int c0, int l,
+// Sources of row r (-1: none) at step l; c0: the lane's first shot column.
+__device__ __forceinline__ void resident_source(const ResidentArgs& a, int r, int c0, int l,
                                                 float gamma, float4& o) {
   if (r < 0) return;
   const int q0 = __ldg(a.ev.src_ptr + r), q1 = __ldg(a.ev.src_ptr + r + 1);
-  if (q0 != q1) {
-    const float sv = gamma * __ldg(a.wavelet + l);
-    for (int q = q0; q < q1; ++q) {
-      const int d = __ldg(a.ev.src_shot + q) - c0;
-      if (d >= 0 && d < 4) add_comp(o, d, sv);
-    }
+  if (q0 == q1) return;
+  const float sv = gamma * __ldg(a.wavelet + l);
+  for (int q = q0; q < q1; ++q) {
+    const int d = __ldg(a.ev.src_shot + q) - c0;
+    if (d >= 0 && d < 4) add_comp(o, d, sv);
   }
-  if (a.traces)
-    for (int q = __ldg(a.ev.rec_ptr + r); q < __ldg(a.ev.rec_ptr + r + 1); ++q) {
-      const int d = __ldg(a.ev.rec_shot + q) - c0;
-      if (d >= 0 && d < 4)
-        a.traces[(size_t)__ldg(a.ev.rec_trace + q) * a.nt + l] = get_comp(o, d);
-    }
+}
+// Receivers of row r: sample l of their traces.
+__device__ __forceinline__ void resident_record(const ResidentArgs& a, float* traces, int r,
+                                                int c0, int l, const float4& o) {
+  if (r < 0 || !traces) return;
+  for (int q = __ldg(a.ev.rec_ptr + r); q < __ldg(a.ev.rec_ptr + r + 1); ++q) {
+    const int d = __ldg(a.ev.rec_shot + q) - c0;
+    if (d >= 0 && d < 4) traces[(size_t)__ldg(a.ev.rec_trace + q) * a.nt + l] = get_comp(o, d);
+  }
+}
+// What tangent_fix subtracts.
+__device__ __forceinline__ float4 tangent_term(float4 pn, float4 ps, float4 pold, float2 tc) {
+  return make_float4(
+      __fmaf_rn(tc.x, d2t(pn.x, ps.x, pold.x), __fmul_rn(tc.y, d1t(pn.x, pold.x))),
+      __fmaf_rn(tc.x, d2t(pn.y, ps.y, pold.y), __fmul_rn(tc.y, d1t(pn.y, pold.y))),
+      __fmaf_rn(tc.x, d2t(pn.z, ps.z, pold.z), __fmul_rn(tc.y, d1t(pn.z, pold.z))),
+      __fmaf_rn(tc.x, d2t(pn.w, ps.w, pold.w), __fmul_rn(tc.y, d1t(pn.w, pold.w))));
+}
+
+// Cooperative launch (patches wait for one another: all resident), the
+// exchange buffer's step numbers cleared first.  MG_ERR_UNSUPPORTED when the
+// device cannot hold it.
+template <class A>
+int launch_resident(void (*kern)(A), const A& a, const ResidentShape& s, cudaStream_t st) {
+  const int rc = resident_smem_limit(reinterpret_cast<const void*>(kern), s.smem);
+  if (rc != MG_OK) return rc;
+  if (a.P.n_x && cudaMemsetAsync(a.xbuf, 0, (size_t)2 * a.P.n_x * s.lpr * 2 * sizeof(uint4),
+                                 st) != cudaSuccess)
+    return MG_ERR_CUDA;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(a.P.B);
+  cfg.blockDim = dim3(32 * s.warps);
+  cfg.dynamicSmemBytes = s.smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a);
+  if (e == cudaSuccess) return MG_OK;
+  cudaGetLastError();
+  return e == cudaErrorCooperativeLaunchTooLarge ? MG_ERR_UNSUPPORTED : MG_ERR_CUDA;
 }
 
 }  // namespace

@@ -1,7 +1,13 @@
 #pragma once
 
-// Resident forward kernel: one cooperative launch advances a group of shots
-// by many leapfrog steps with the states on chip (resident_common.cuh).
+// Resident forward kernel and forward + tangent kernel: one cooperative launch
+// advances a group of shots by many leapfrog steps with the states on chip
+// (resident_common.cuh).
+//
+// TAN: p and dp of 2 LPR shots share the rows, the first half of a row's lanes
+// holding p and the second dp: both are columns of the same product, and the
+// lanes of dp take the correction of tangent_fix from their partner by
+// shuffles (four values).
 //
 // Bound by shared memory bandwidth: a float4 of a row takes 41 reads and writes
 // of 16 bytes per 4 columns (6 neighbours, self, p_{l-1}, result, entries,
@@ -24,8 +30,8 @@ namespace mg {
 namespace {
 
 // U: pairs of every row are 3 (straight code), else as the group headers say.
-// HIST: every state goes to the history.
-template <int LPR, bool U, bool HIST>
+// HIST: every state p goes to the history.
+template <int LPR, bool U, bool HIST, bool TAN>
 __global__ void __launch_bounds__(kResidentThreads, 1) k_resident_step(ResidentArgs a) {
   constexpr int RPW = 32 / LPR, SLOT = 16 * LPR;
   extern __shared__ __align__(16) unsigned char sm[];
@@ -34,16 +40,23 @@ __global__ void __launch_bounds__(kResidentThreads, 1) k_resident_step(ResidentA
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
   const DevPatches& D = a.P;
   const unsigned buf = (unsigned)D.max_slots * SLOT;
-  const Patch t = patch_tables<RPW>(D, sm + 2 * (size_t)buf, b);
+  float2* const tc = reinterpret_cast<float2*>(sm + 2 * (size_t)buf);   // TAN, per own slot
+  const Patch t = patch_tables<RPW>(
+      D, sm + 2 * (size_t)buf + (TAN ? (D.max_groups * RPW + 1) / 2 * 16 : 0), b);
   fill_patch<LPR>(D, a.ev, t, a.coef, b, tid, threads);
   if (tid < 2) failed[tid] = 0;
+  if (TAN)
+    for (int i = tid; i < t.ng * RPW; i += threads) {
+      const int r = __ldg(D.row + t.g0 * RPW + i);
+      tc[i] = r < 0 ? make_float2(0.f, 0.f) : __ldg(a.tcoef + r);
+    }
   const unsigned s0 = smem_u32(sm);
   const int own = t.ng * RPW;
   for (int i = tid; i < (own + t.halo) * LPR; i += threads) {
     const int s = i / LPR;   // p_l of every slot, p_{l-1} of the own ones
     const int r = s < own ? __ldg(D.row + t.g0 * RPW + s) : __ldg(D.halo + t.h0 + s - own);
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f), u = v;
-    if (a.p && r >= 0) {
+    if (!TAN && a.p && r >= 0) {   // the tangent starts at rest
       const size_t o = (size_t)r * a.ld + a.col0;
       v = __ldg(reinterpret_cast<const float4*>(a.p + o) + i % LPR);
       if (s < own) u = __ldg(reinterpret_cast<const float4*>(a.pm + o) + i % LPR);
@@ -63,9 +76,13 @@ __global__ void __launch_bounds__(kResidentThreads, 1) k_resident_step(ResidentA
   unsigned mine = s0 + lane * 16, st = s0 + lane % LPR * 16,
            pair0 = smem_u32(t.pair + lane / LPR), coef0 = smem_u32(t.coef + lane / LPR),
            row0 = smem_u32(t.row + lane / LPR), hdr0 = smem_u32(t.hdr);
-  int c0 = a.col0 + lane % LPR * 4;
+  constexpr int COLS = TAN ? LPR / 2 : LPR;   // lanes of a row with different shots
+  const bool is_q = TAN && lane % LPR >= COLS;
+  int c0 = a.col0 + lane % COLS * 4;
+  unsigned tc0 = smem_u32(tc + lane / LPR);
   asm volatile("" : "+r"(mine), "+r"(st), "+r"(pair0), "+r"(coef0), "+r"(row0), "+r"(hdr0),
-               "+r"(c0));
+               "+r"(c0), "+r"(tc0));
+  float* const traces = is_q ? a.dtraces : a.traces;
   uint4* const xmine = a.xbuf + ((size_t)t.x0 * LPR + lane) * 2;   // border group g: + 64 g
   for (int j = 0; j < a.steps; ++j) {
     const unsigned in = (j & 1) * buf, out = ((j & 1) ^ 1) * buf;
@@ -87,19 +104,32 @@ __global__ void __launch_bounds__(kResidentThreads, 1) k_resident_step(ResidentA
             : row_product<RPW>(st + in, pair0 + (h & ((1 << kPairShift) - 1)) * 16,
                                (h >> kPairShift) & kPairMask, c.w, self);
       float4 o = leap(c, self, old, acc);
-      if (h < 0) resident_events(a, lds1(row0 + g * (RPW * 4)), c0, a.step0 + j, c.z, o);
+      if (h < 0) resident_source(a, is_q ? -1 : lds1(row0 + g * (RPW * 4)), c0, a.step0 + j, c.z, o);
+      if (TAN) {   // dp -= cm (p+ - 2 p + p-) + cd (p+ - p-)
+        const int2 v = lds2(tc0 + g * (RPW * 8));
+        const float4 f = tangent_term(o, self, old, make_float2(__int_as_float(v.x),
+                                                                __int_as_float(v.y)));
+        const float4 e = make_float4(__shfl_xor_sync(0xffffffffu, f.x, COLS),
+                                     __shfl_xor_sync(0xffffffffu, f.y, COLS),
+                                     __shfl_xor_sync(0xffffffffu, f.z, COLS),
+                                     __shfl_xor_sync(0xffffffffu, f.w, COLS));
+        if (is_q)
+          o = make_float4(__fsub_rn(o.x, e.x), __fsub_rn(o.y, e.y), __fsub_rn(o.z, e.z),
+                          __fsub_rn(o.w, e.w));
+      }
+      if (h < 0) resident_record(a, traces, lds1(row0 + g * (RPW * 4)), c0, a.step0 + j, o);
       if (border) xstore(xo + g * 64, o, (unsigned)(j + 1));
       sts4(mine + out + g * 512, o);
       if (HIST) {
         const int r = lds1(row0 + g * (RPW * 4));
-        if (r >= 0)
+        if (r >= 0 && !is_q)
           *reinterpret_cast<float4*>(a.hist + (size_t)j * a.state + (size_t)r * a.ld + c0) = o;
       }
     }
     __syncthreads();
     if (failed[j & 1]) return;
   }
-  if (a.out_p) {
+  if (!TAN && a.out_p) {
     const unsigned in = (a.steps & 1) * buf, out = ((a.steps & 1) ^ 1) * buf;
     for (int g = g_first; g < g_end; g += nw) {
       const int r = lds1(row0 + g * (RPW * 4));
@@ -111,35 +141,18 @@ __global__ void __launch_bounds__(kResidentThreads, 1) k_resident_step(ResidentA
   }
 }
 
-template <int LPR, bool U, bool HIST>
+template <int LPR, bool U, bool HIST, bool TAN>
 int launch_one(const ResidentArgs& a, const ResidentShape& s, cudaStream_t st) {
-  auto kern = k_resident_step<LPR, U, HIST>;
-  const int rc = resident_smem_limit(reinterpret_cast<const void*>(kern), s.smem);
-  if (rc != MG_OK) return rc;
-  if (a.P.n_x && cudaMemsetAsync(a.xbuf, 0, (size_t)2 * a.P.n_x * LPR * 2 * sizeof(uint4), st) !=
-                     cudaSuccess)
-    return MG_ERR_CUDA;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(a.P.B);
-  cfg.blockDim = dim3(32 * s.warps);
-  cfg.dynamicSmemBytes = s.smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeCooperative;   // patches wait for one another: all resident
-  at[0].val.cooperative = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, a);
-  if (e == cudaSuccess) return MG_OK;
-  cudaGetLastError();
-  return e == cudaErrorCooperativeLaunchTooLarge ? MG_ERR_UNSUPPORTED : MG_ERR_CUDA;
+  return launch_resident(k_resident_step<LPR, U, HIST, TAN>, a, s, st);
 }
 
-template <int LPR>
+template <int LPR, bool TAN>
 int launch_lpr(const ResidentArgs& a, const ResidentShape& s, cudaStream_t st) {
   if (a.P.uniform == 3)
-    return a.hist ? launch_one<LPR, true, true>(a, s, st) : launch_one<LPR, true, false>(a, s, st);
-  return a.hist ? launch_one<LPR, false, true>(a, s, st) : launch_one<LPR, false, false>(a, s, st);
+    return a.hist ? launch_one<LPR, true, true, TAN>(a, s, st)
+                  : launch_one<LPR, true, false, TAN>(a, s, st);
+  return a.hist ? launch_one<LPR, false, true, TAN>(a, s, st)
+                : launch_one<LPR, false, false, TAN>(a, s, st);
 }
 
 }  // namespace

@@ -61,6 +61,35 @@ def test_forward_carries_the_row_kernels_bits(mg, make, kw, order, bc):
     assert a.device_status() == 0
 
 
+@pytest.mark.parametrize("make,kw,order,bc", CASES)
+def test_jacobians_carry_the_row_kernels_bits(mg, make, kw, order, bc):
+    """J v alone and in the fused pass, J^T w from checkpoints (a last segment of
+    any length) and on the kept history."""
+    w = make(**kw)
+    a, b = _pair(mg, w, order, bc)
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    s = _dev(w.wavelet(dt))
+    rng = np.random.default_rng(2)
+    level = w.mesh.n_levels - 1
+    v = _dev(rng.standard_normal(w.mesh.n_cells[level]))
+    W = _dev(rng.standard_normal((w.shots.n_traces, w.nt)), torch.float32)
+
+    def run(m):
+        jv = mg.jacobian_apply(m, level, eps, w.shots, s, dt, v)
+        y0, j0 = mg.forward_jacobian_apply(m, level, eps, w.shots, s, dt, v)
+        y1, j1 = mg.forward_jacobian_apply(m, level, eps, w.shots, s, dt, v, keep_states=True)
+        gk = mg.jacobian_T_apply(m, level, eps, w.shots, s, dt, W, ckpt_every=w.nt,
+                                 reuse_checkpoints=True)
+        jk = mg.jacobian_apply(m, level, eps, w.shots, s, dt, v, reuse_states=True)
+        gs = [mg.jacobian_T_apply(m, level, eps, w.shots, s, dt, W, ckpt_every=c)
+              for c in (16, 17, 32, w.nt)]
+        return [jv, y0, j0, y1, j1, gk, jk] + gs
+
+    for x, y in zip(run(a), run(b)):
+        assert torch.equal(x, y)
+    assert a.device_status() == 0
+
+
 def test_many_sources_and_receivers_per_row(mg):
     """Every shot on the same node, receivers on shared nodes, some repeated."""
     w = configs.asteroid_2d(n_refine=1, S=5, nt=60)
@@ -71,7 +100,10 @@ def test_many_sources_and_receivers_per_row(mg):
     a, b = _pair(mg, w)
     dt, eps = oracle_dt(w), _dev(w.eps)
     s = _dev(w.wavelet(dt))
-    assert torch.equal(mg.forward(a, eps, w.shots, s, dt), mg.forward(b, eps, w.shots, s, dt))
+    W = _dev(np.random.default_rng(3).standard_normal((10, w.nt)), torch.float32)
+    for run in (lambda m: mg.forward(m, eps, w.shots, s, dt),
+                lambda m: mg.jacobian_T_apply(m, 1, eps, w.shots, s, dt, W, ckpt_every=20)):
+        assert torch.equal(run(a), run(b))
 
 
 def test_a_wait_that_runs_out_is_loud(mg):
@@ -85,6 +117,8 @@ def test_a_wait_that_runs_out_is_loud(mg):
     y = mg.forward(a, eps, w.shots, s, dt)
     assert bool(torch.isnan(y).all())
     assert a.device_status() == L.MG_ERR_TIMEOUT
+    W = _dev(np.ones(tuple(y.shape)), torch.float32)
+    assert bool(torch.isnan(mg.jacobian_T_apply(a, 1, eps, w.shots, s, dt, W)).all())
     a.set_persistent()
     assert torch.equal(mg.forward(a, eps, w.shots, s, dt), mg.forward(b, eps, w.shots, s, dt))
     assert a.device_status() == 0
