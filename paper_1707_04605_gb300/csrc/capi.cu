@@ -132,6 +132,7 @@ struct mg_mesh {
   int cchunk = 0;                         // its chunk (0: none)
   int64_t cstride = 0;                    // entries per slice in it
   bool chunked_ell = false;
+  std::map<int, Buf> auto_ellc;           // the same for the default launch shapes, by chunk
   int wu = 0;
   bool uniform_ell = false;
   int cache_hints = 1;                    // kept history: L2 evict-first on last reads
@@ -470,12 +471,62 @@ int* err_word(mg_mesh* M) {
   return P<int>(M->errbuf);
 }
 
+// Launch shape of a kind on `cols` columns: the one that was asked for, or by
+// default (from 16 columns on) two float4 per lane under the register cap with
+// chunk-major entries, for the tangent one float4 per lane under the cap (it
+// gathers two states).  Measured against one float4 without the cap and by
+// column, us per step: forward, 232,505 nodes of tetrahedra, 128 shots 190.9 ->
+// 114.8, 32 shots 60.2 -> 38.4, 8 shots 18.9 -> 18.5; reverse steps, 62,641
+// nodes, 128 shots 39.0 -> 26.4, 256 shots 85.2 -> 59.6; tangent, 62,641 nodes,
+// 128 shots 55.3 -> 49.2, 30,525 nodes of tetrahedra, 256 shots 71.7 -> 65.1.
+// The source tiles of the adjoint stay 128 columns wide: the same sums.
+struct RowShape {
+  int batch, min_blocks, most_cols;
+  bool chunked;   // from M->auto_ellc
+};
+RowShape row_shape(const mg_mesh* M, int kind, int cols) {
+  const mg_mesh::Tuning& t = M->tune[kind];
+  if (t.shaped || cols < 16) return {t.batch, t.min_blocks, 512, false};
+  return {kind == 1 ? 1 : 2, 5, 128, !M->chunked_ell};
+}
+
+// Chunk-major entries for the default shape of a kind, built on the device on
+// first use (before any graph capture).
+int ensure_auto_entries(mg_mesh* M, int kind, int cols, cudaStream_t st) {
+  const RowShape r = row_shape(M, kind, cols);
+  const int chunk = mg::rows_lanes(cols, r.batch, kind == 2 ? r.most_cols : 512);
+  if (!r.chunked || chunk < 2 || chunk > 16) return MG_OK;
+  Buf& b = M->auto_ellc[chunk];
+  if (b.p) return MG_OK;
+  int w = 0;
+  for (int32_t x : M->hm.slice_w) w = std::max(w, (int)x);
+  const int64_t stride = (int64_t)(w + chunk - 1) / chunk * mg::kSliceH * chunk;
+  MG_TRY(ensure(b, (size_t)M->hm.n_slices * stride * sizeof(int2)));
+  M->launches += 1;
+  return mg::launch_chunk_entries(dev_ell(M), chunk, stride, P<int2>(b), st);
+}
+
+void use_auto_entries(mg_mesh* M, const RowShape& r, int kind, int cols, mg::DevEll& K) {
+  if (!r.chunked) return;
+  const int chunk = mg::rows_lanes(cols, r.batch, kind == 2 ? r.most_cols : 512);
+  auto it = M->auto_ellc.find(chunk);
+  if (it == M->auto_ellc.end() || !it->second.p) return;
+  int w = 0;
+  for (int32_t x : M->hm.slice_w) w = std::max(w, (int)x);
+  K.ellc = P<const int2>(it->second);
+  K.cchunk = chunk;
+  K.cstride = (int64_t)(w + chunk - 1) / chunk * mg::kSliceH * chunk;
+}
+
 int do_step(mg_mesh* M, const mg::StepArgs& a, int S_pad, cudaStream_t st) {
-  const mg::DevTiles T = dev_tiles(M, a.cols ? a.cols : S_pad, 0);
+  const int cols = a.cols ? a.cols : S_pad;
+  const mg::DevTiles T = dev_tiles(M, cols, 0);
   if (T.n_tiles) return mg::launch_step_tiled(a, T, st);
   mg::StepArgs b = a;
-  b.batch = M->tune[0].batch;
-  b.min_blocks = M->tune[0].min_blocks;
+  const RowShape rs = row_shape(M, 0, cols);
+  b.batch = rs.batch;
+  b.min_blocks = rs.min_blocks;
+  use_auto_entries(M, rs, 0, cols, b.K);
   b.ring = M->tune[0].ring;
   b.sweep = M->tune[0].sweep;
   b.stream = M->tune[0].stream;
@@ -497,16 +548,22 @@ int do_step(mg_mesh* M, const mg::StepArgs& a, int S_pad, cudaStream_t st) {
   return mg::launch_step(b, S_pad, st);
 }
 
+void row_tangent_args(mg_mesh* M, int cols, mg::TangentArgs& b) {
+  const RowShape rs = row_shape(M, 1, cols);
+  b.f.batch = rs.batch;
+  b.f.min_blocks = rs.min_blocks;
+  use_auto_entries(M, rs, 1, cols, b.f.K);
+  b.f.ring = M->tune[1].ring;
+  b.f.stream = M->tune[1].stream;
+  b.f.prefetch = M->tune[1].prefetch;
+  b.f.pdl = M->dep_launch;
+}
+
 int do_tangent(mg_mesh* M, const mg::TangentArgs& a, int S_pad, cudaStream_t st) {
   const mg::DevTiles T = dev_tiles(M, a.f.cols ? a.f.cols : S_pad, 1);
   if (T.n_tiles) return mg::launch_tangent_tiled(a, T, st);
   mg::TangentArgs b = a;
-  b.f.batch = M->tune[1].batch;
-  b.f.ring = M->tune[1].ring;
-  b.f.stream = M->tune[1].stream;
-  b.f.prefetch = M->tune[1].prefetch;
-  b.f.min_blocks = M->tune[1].min_blocks;
-  b.f.pdl = M->dep_launch;
+  row_tangent_args(M, a.f.cols ? a.f.cols : S_pad, b);
   return mg::launch_tangent(b, S_pad, st);
 }
 
@@ -514,11 +571,15 @@ int do_adjoint(mg_mesh* M, const mg::AdjointArgs& a, int S_pad, cudaStream_t st)
   const mg::DevTiles T = dev_tiles(M, a.cols ? a.cols : S_pad, 2);
   if (T.n_tiles) return mg::launch_adjoint_tiled(a, T, st);
   mg::AdjointArgs b = a;
-  b.batch = M->tune[2].batch;
+  const int cols = a.cols ? a.cols : S_pad;
+  const RowShape rs = row_shape(M, 2, cols);
+  b.batch = rs.batch;
+  b.min_blocks = rs.min_blocks;
+  b.most_cols = rs.most_cols;
+  use_auto_entries(M, rs, 2, cols, b.K);
   b.ring = M->tune[2].ring;
   b.stream = M->tune[2].stream;
   b.prefetch = M->tune[2].prefetch;
-  b.min_blocks = M->tune[2].min_blocks;
   b.pdl = M->dep_launch;
   return mg::launch_adjoint(b, S_pad, st);
 }
@@ -528,7 +589,8 @@ int do_adjoint(mg_mesh* M, const mg::AdjointArgs& a, int S_pad, cudaStream_t st)
 // one after another), else one per source tile of the whole shot range.
 int adjoint_sets(mg_mesh* M, int S_pad, int cols) {
   if (dev_tiles(M, cols, 2).n_tiles) return 1;
-  return (S_pad / cols) * mg::rows_tiles(cols, M->tune[2].batch);
+  const RowShape rs = row_shape(M, 2, cols);
+  return (S_pad / cols) * mg::rows_tiles(cols, rs.batch, rs.most_cols);
 }
 
 mg::StepArgs step_args(mg_mesh* M, const Prep& pp, int ld, int nt) {
@@ -664,13 +726,36 @@ int patch_tables(mg_mesh* M, int B, int rpw, mg::DevPatches& D) {
   return D.B ? MG_OK : MG_ERR_OOM;
 }
 
+// Estimates of a step's time on the two paths, in us, from measurements at 2, 8,
+// 16, 64, 128 and 256 columns on triangles (3,997 to 249,697 nodes) and
+// tetrahedra (30,525), most within 15% of them.  Resident: a launch per column
+// group, each the exchange of border rows, the patch's shared memory accesses
+// (a row read by fewer than 8 lanes conflicts with others) and its halo's.  Row
+// kernels: launch and tail, then the gathers, or the states' traffic when they
+// exceed L2.
+double resident_us(const mg::DevPatches& D, const mg::ResidentShape& s, int kind, int S_pad) {
+  const double conflicts = s.lpr >= 8 ? 1.0 : s.lpr == 4 ? 1.5 : s.lpr == 2 ? 2.4 : 1.6;
+  const double pairs = (double)D.max_pairs / (D.max_groups * (32 / s.lpr));
+  const double group = 14.0 + pairs * (1.0 + 8.0 * conflicts) + (kind == 1 ? 6.0 : kind == 2 ? 12.0 : 0.0);
+  const int launches = S_pad / (kind == 1 ? 2 * s.lpr : 4 * s.lpr);
+  return launches * (0.9 + 0.65e-3 * group * D.max_groups + 0.3e-3 * D.max_halo * 2 * s.lpr);
+}
+double rows_us(const mg_mesh* M, int kind, int S_pad) {
+  const double work = (double)M->hm.rowptr.back() * S_pad, cols = (double)M->hm.n * S_pad;
+  const double gathers = 4.0 + (kind == 0 ? 0.27e-6 : kind == 1 ? 0.5e-6 : 0.38e-6) * work;
+  const double held = (kind == 1 ? 16.0 : 8.0) * cols;   // bytes of the states of a step
+  const double moved = (kind == 0 ? 12.0 : kind == 1 ? 24.0 : 16.0) * cols;
+  if (held < 100e6) return gathers;
+  return std::max(gathers, moved / (held < 200e6 ? 3.9e6 : 3.4e6));
+}
+
 // Resident launch shape of a call that advances S_pad columns for `steps`
 // steps (launch, tables and exchange buffer cost about 10 us: at least 16 of
 // them).  Forward: the widest column group whose patches fit; tangent: the
 // same with p and dp as columns (2 lpr shots per launch); adjoint: whole source
 // tiles of the row kernel only, for the same sums over the shots.
-// shape.lpr = 0: the row kernels are the path (nothing fits, or a launch shape
-// of theirs was asked for).
+// shape.lpr = 0: the row kernels are the path (nothing fits, they are estimated
+// to be faster, or a launch shape of theirs was asked for).
 int resident_shape(mg_mesh* M, int kind, int S_pad, int steps, mg::DevPatches& D,
                    mg::ResidentShape& shape) {
   shape = mg::ResidentShape();
@@ -681,14 +766,16 @@ int resident_shape(mg_mesh* M, int kind, int S_pad, int steps, mg::DevPatches& D
   const int widest = kind == 1 ? std::min(32, S_pad / 2) : std::min(S_pad, 128) / 4;
   const int row_bytes = kind == 1 ? 8 : kind == 2 ? 16 : 0;
   for (int lpr = widest; lpr >= (kind == 1 ? 2 : 1); lpr >>= 1) {
-    // where the states alone are too large no tables are needed to see it
-    if (M->hm.n / B * (int64_t)lpr * 32 <= M->smem_optin) {
+    // where rows and entries alone are too large no tables are needed to see it
+    const int64_t rows = M->hm.n / B, entries = (M->hm.rowptr.back() - M->hm.n) / B;
+    if (rows * (32 * lpr + 20 + row_bytes) + entries * 8 <= M->smem_optin) {
       MG_TRY(patch_tables(M, B, 32 / lpr, D));
-      if (mg::resident_fit(D, lpr, row_bytes, M->smem_optin - 1024, shape) == MG_OK) return MG_OK;
+      if (mg::resident_fit(D, lpr, row_bytes, M->smem_optin - 1024, shape) == MG_OK) break;
       shape = mg::ResidentShape();
     }
-    if (kind == 2) return MG_OK;
+    if (kind == 2) break;
   }
+  if (shape.lpr && resident_us(D, shape, kind, S_pad) > rows_us(M, kind, S_pad)) shape.lpr = 0;
   return MG_OK;
 }
 
@@ -810,6 +897,7 @@ int run_forward(mg_mesh* M, const Prep& pp, int nt, float* traces, int ckpt_ever
           run_forward_resident(M, pp, nt, traces, ckpt_every, ckpt, nullptr, D, shape, st);
       if (rc != MG_ERR_UNSUPPORTED) return rc;
     }
+    MG_TRY(ensure_auto_entries(M, 0, group_cols(M, 0, pp.S_pad), st));
   }
   MG_TRY(ensure(M->stA, state * sizeof(float)));
   MG_TRY(ensure(M->stB, state * sizeof(float)));
@@ -918,6 +1006,7 @@ int run_forward_states(mg_mesh* M, const Prep& pp, int nt, float* traces, float*
   a.traces = traces;
   a.hint = M->cache_hints;
   const int W = group_cols(M, 0, pp.S_pad), NG = pp.S_pad / W;
+  MG_TRY(ensure_auto_entries(M, 0, W, st));
   if (graphs_on(M, flags) && nt % 2 == 0) {
     MG_TRY(ensure(M->step_base, 16));
     int32_t* base = P<int32_t>(M->step_base);
@@ -1068,6 +1157,8 @@ void mg_mesh_destroy(mg_mesh* M) {
   for (auto* v : {&M->anc, &M->lvl_ptr, &M->lvl_idx})
     for (Buf& b : *v)
       if (b.p) cudaFree(b.p);
+  for (auto& kv : M->auto_ellc)
+    if (kv.second.p) cudaFree(kv.second.p);
   for (auto& kv : M->tiles) {
     mg_mesh::TileTables& D = kv.second;
     for (Buf* b : {&D.ell_off, &D.ell_idx, &D.ell_val, &D.sinfo, &D.halo_off, &D.halo_cnt, &D.halo})
@@ -1592,6 +1683,7 @@ int mg_jacobian_apply(mg_mesh* M, int level, const double* eps, const mg_shots* 
       if (rc != MG_ERR_UNSUPPORTED) return rc;
     }
   }
+  MG_TRY(ensure_auto_entries(M, 1, group_cols(M, 1, pp.S_pad), st));
   Buf* bufs[] = {&M->stA, &M->stB, &M->stC, &M->stD};
   for (Buf* b : bufs) {
     MG_TRY(ensure(*b, state * sizeof(float)));
@@ -1770,6 +1862,7 @@ int mg_forward_jacobian_apply(mg_mesh* M, int level, const double* eps, const mg
       if (rc != MG_ERR_UNSUPPORTED) return rc;
     }
   }
+  MG_TRY(ensure_auto_entries(M, 1, group_cols(M, 1, pp.S_pad), st));
   if (!keep) {
     for (Buf* b : {&M->stA, &M->stB}) {
       MG_TRY(ensure(*b, state * sizeof(float)));
@@ -1786,12 +1879,7 @@ int mg_forward_jacobian_apply(mg_mesh* M, int level, const double* eps, const mg
   mg::TangentArgs a{};
   a.f = step_args(M, pp, pp.S_pad, nt);
   a.f.traces = trf;
-  a.f.batch = M->tune[1].batch;
-  a.f.ring = M->tune[1].ring;
-  a.f.stream = M->tune[1].stream;
-  a.f.prefetch = M->tune[1].prefetch;
-  a.f.min_blocks = M->tune[1].min_blocks;
-  a.f.pdl = M->dep_launch;
+  a.f.batch = M->tune[1].batch;   // MG_PERSISTENT
   a.f.hint = keep ? M->cache_hints : 0;   // p_{l-1} is last read here only when kept
   a.tcoef = P<const float2>(M->tcoef);
   a.dtraces = tr;
@@ -1825,6 +1913,7 @@ int mg_forward_jacobian_apply(mg_mesh* M, int level, const double* eps, const mg
         b.q = u;
         b.qm = z;
         b.f.step = j;
+        row_tangent_args(M, W, b);
         MG_TRY(mg::launch_tangent(b, pp.S_pad, cs));
         std::swap(u, z);
       }
@@ -1962,6 +2051,8 @@ int mg_jacobian_T_apply(mg_mesh* M, int level, const double* eps, const mg_shots
     MG_TRY(resident_shape(M, 0, pp.S_pad, std::min(ckpt_every, nt), Df, shf));
     MG_TRY(resident_shape(M, 2, pp.S_pad, std::min(ckpt_every, nt), Da, sha));
   }
+  if (!shf.lpr && !states) MG_TRY(ensure_auto_entries(M, 0, Wf, st));
+  if (!sha.lpr) MG_TRY(ensure_auto_entries(M, 2, Wa, st));
   mg::ResidentAdjArgs ra{};
   if (sha.lpr) {
     ra.P = Da;

@@ -181,6 +181,17 @@ __global__ void k_copy_f4(const float4* __restrict__ src, float4* __restrict__ d
 }
 
 
+// One thread per slot of the copy: entry k of slice row r at
+// (k / chunk * 32 + r) chunk + k % chunk of its slice, zero past the width.
+__global__ void k_chunk_entries(DevEll K, int chunk, int64_t stride, int64_t total, int2* out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= total) return;
+  const int64_t s = i / stride;
+  const int o = (int)(i - s * stride), r = o / chunk % kSliceH;
+  const int k = o / (chunk * kSliceH) * chunk + o % chunk;
+  out[i] = k < K.slice_w[s] ? K.ell[K.slice_off[s] + (int64_t)k * kSliceH + r] : make_int2(0, 0);
+}
+
 }  // namespace
 
 namespace {
@@ -194,6 +205,12 @@ __global__ void k_prolong(int64_t m, const int32_t* anc, const double* v, const 
 int launch_prolong(int64_t m, const int32_t* anc, const double* v, const double* base,
                    double* out, cudaStream_t st) {
   k_prolong<<<(unsigned)((m + 255) / 256), 256, 0, st>>>(m, anc, v, base, out);
+  return check_launch();
+}
+
+int launch_chunk_entries(const DevEll& K, int chunk, int64_t stride, int2* out, cudaStream_t st) {
+  const int64_t total = (K.n + kSliceH - 1) / kSliceH * stride;
+  k_chunk_entries<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(K, chunk, stride, total, out);
   return check_launch();
 }
 

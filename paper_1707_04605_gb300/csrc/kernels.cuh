@@ -95,6 +95,7 @@ struct AdjointArgs {
   int32_t stream = 0;       // row kernel: once-read loads without L1 allocation
   int32_t min_blocks = 0;   // row kernel: 0, or 5 or 6 resident CTAs per SM (register cap)
   int32_t prefetch = 0;     // as in StepArgs
+  int32_t most_cols = 512;  // row kernel: widest source tile
   float* G;                 // [tiles][n] sums; row kernels: set = absolute source tile
   float* Gc;                // compensations
   float* H;
@@ -133,7 +134,12 @@ int launch_adjoint_tiled(const AdjointArgs& a, const DevTiles& T, cudaStream_t s
 // launch and `nv` float4 per lane; the adjoint keeps one accumulator set per
 // source tile of the whole padded shot range (S_pad / cols launches of
 // rows_tiles(cols, nv) tiles each).
-int rows_tiles(int cols, int nv);
+int rows_tiles(int cols, int nv, int most_cols = 512);
+// Lanes per row of the row kernels for that launch.
+int rows_lanes(int cols, int nv, int most_cols = 512);
+// The chunk-major copy of the entries (DevEll::ellc) for `chunk` lanes per row,
+// from the sliced ones; `stride` entries per slice.
+int launch_chunk_entries(const DevEll& K, int chunk, int64_t stride, int2* out, cudaStream_t st);
 
 int launch_step(const StepArgs& a, int S_pad, cudaStream_t st);
 // Forward step with neighbour rows staged by bulk asynchronous copies

@@ -156,7 +156,10 @@ bool persist_ok(const PersistArgs& pa) {
 
 }  // namespace
 
-int rows_tiles(int cols, int nv) { return (int)shape_of(1, cols, nv).grid.y; }
+int rows_tiles(int cols, int nv, int most_cols) {
+  return (int)shape_of(1, cols, nv, most_cols).grid.y;
+}
+int rows_lanes(int cols, int nv, int most_cols) { return shape_of(1, cols, nv, most_cols).lpr; }
 
 #define MG_PERSIST_SWITCH(KERN, ARGS)                                                    \
   switch (sh.lpr * 8 + sh.nv) {                                                        \
@@ -307,7 +310,7 @@ int launch_tangent_kept(const TangentArgs& a, int S_pad, cudaStream_t st) {
 int launch_adjoint(const AdjointArgs& a, int S_pad, cudaStream_t st) {
   if (a.ring) return launch_adjoint_ring(a, S_pad, st);
   const int cols = a.cols ? a.cols : S_pad;
-  const Shape sh = shape_of(a.K.n, cols, a.batch);
+  const Shape sh = shape_of(a.K.n, cols, a.batch, a.most_cols);
   if (!range_ok(sh, a.col0, cols, a.ld)) return MG_ERR_ARG;
   cudaError_t err = cudaSuccess;
   if (a.min_blocks == 6) {

@@ -14,6 +14,7 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <mutex>
 #include <set>
 #include <utility>
@@ -882,11 +883,25 @@ __device__ __forceinline__ void adjoint_rows_block(const AdjointArgs& a, int blk
       if (j >= 0)
         add_to<NV>(out, j, d, c.w * __ldg(a.w + (size_t)__ldg(a.ev.rec_trace + q) * a.nt + (k - 1)));
     }
+    // The row's sums over the shots in the order of one float4 per lane on
+    // NV LPR lanes: a term per float4, then the upper stages of that shuffle
+    // tree inside the lane, so the bits do not depend on NV.
+    float u1[NV], u2[NV];
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
       st4(a.mu1 + ro + 4 * LPR * j, out[j]);
-      adj_terms(pk[j], out[j], self[j], old[j], t1, t2);
+      u1[j] = u2[j] = 0.0f;
+      adj_terms(pk[j], out[j], self[j], old[j], u1[j], u2[j]);
     }
+#pragma unroll
+    for (int half = NV / 2; half > 0; half >>= 1)
+#pragma unroll
+      for (int j = 0; j < half; ++j) {
+        u1[j] += u1[j + half];
+        u2[j] += u2[j + half];
+      }
+    t1 = u1[0];
+    t2 = u2[0];
   }
 #pragma unroll
   for (int off = LPR / 2; off > 0; off >>= 1) {
@@ -920,11 +935,13 @@ struct Shape {
   dim3 grid;
 };
 
-Shape shape_of(int n, int cols, int nv) {
+// most_cols: widest source tile (the adjoint keeps one accumulator per row and
+// tile, so its tiling is part of its result).
+Shape shape_of(int n, int cols, int nv, int most_cols = 512) {
   Shape s;
   for (;; nv >>= 1) {
     s.nv = nv;
-    s.lpr = cols / (4 * nv) >= 32 ? 32 : cols / (4 * nv);
+    s.lpr = std::min({32, cols / (4 * nv), most_cols / (4 * nv)});
     // LPR must be a power of two (lanes of a row inside a warp)
     if (nv == 1 || (s.lpr >= 1 && (s.lpr & (s.lpr - 1)) == 0 && cols % (4 * nv * s.lpr) == 0))
       break;

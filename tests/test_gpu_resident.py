@@ -40,7 +40,7 @@ CASES = [
     (configs.asteroid_2d, dict(n_refine=2, S=37, nt=101), "morton", "abc"),
     (configs.asteroid_2d, dict(n_refine=2, S=300, nt=33), "rcm", "neumann"),
     (configs.asteroid_2d, dict(n_refine=3, S=200, nt=50), "morton", "abc"),
-    (configs.asteroid_2d, dict(n_refine=4, S=20, nt=40), "morton", "abc"),
+    (configs.asteroid_2d, dict(n_refine=4, S=8, nt=40), "morton", "abc"),
     (configs.ellipsoid_3d, dict(n_refine=1, S=24, nt=50), "morton", "abc"),
 ]
 
@@ -122,3 +122,32 @@ def test_a_wait_that_runs_out_is_loud(mg):
     a.set_persistent()
     assert torch.equal(mg.forward(a, eps, w.shots, s, dt), mg.forward(b, eps, w.shots, s, dt))
     assert a.device_status() == 0
+
+
+@pytest.mark.parametrize("make,kw", [
+    (configs.asteroid_2d, dict(n_refine=4, S=40, nt=24)),
+    (configs.ellipsoid_3d, dict(n_refine=1, S=300, nt=24)),
+    (configs.ellipsoid_3d, dict(n_refine=2, S=20, nt=12))])
+def test_default_row_shapes_carry_the_plain_shape_bits(mg, make, kw):
+    """Meshes and batches that stay with the row kernels run two float4 per lane
+    under the register cap with chunk-major entries (source tiles of the adjoint
+    128 columns wide) by default: the bits of one float4 per lane."""
+    w = make(**kw)
+    a, b = _pair(mg, w)
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    s = _dev(w.wavelet(dt))
+    rng = np.random.default_rng(4)
+    v = _dev(rng.standard_normal(w.mesh.n_cells[0]))
+    W = _dev(rng.standard_normal((w.shots.n_traces, w.nt)), torch.float32)
+
+    def run(m):
+        y = mg.forward(m, eps, w.shots, s, dt, keep_states=True)
+        return (y, mg.jacobian_T_apply(m, 0, eps, w.shots, s, dt, W, ckpt_every=w.nt,
+                                       reuse_checkpoints=True),
+                mg.jacobian_apply(m, 0, eps, w.shots, s, dt, v, reuse_states=True),
+                mg.jacobian_apply(m, 0, eps, w.shots, s, dt, v),
+                *mg.forward_jacobian_apply(m, 0, eps, w.shots, s, dt, v),
+                mg.jacobian_T_apply(m, 0, eps, w.shots, s, dt, W, ckpt_every=8))
+
+    for x, y in zip(run(a), run(b)):
+        assert torch.equal(x, y)
