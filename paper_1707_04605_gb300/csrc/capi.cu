@@ -10,6 +10,7 @@
 #include <cstring>
 #include <initializer_list>
 #include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -171,6 +172,9 @@ struct mg_mesh {
   Buf tr;                                 // internal trace buffer [R][nt]
   Buf trf;                                // forward traces of the fused forward + tangent
   Buf tune_scratch;                       // autotuner inputs/outputs
+  std::vector<mg::FluxBuffer> flux_scratch;   // work buffers of the flux path's calls
+  std::mutex flux_mu;                     // guards them and the packed geometry
+  Buf flux_cell, flux_ptr, flux_inc;      // its packed geometry
 };
 
 namespace {
@@ -1151,7 +1155,7 @@ void mg_mesh_destroy(mg_mesh* M) {
   Buf* all[] = {&M->ell, &M->slice_off, &M->slice_w, &M->nc_ptr, &M->nc_cell, &M->nc_w,
                 &M->nf_ptr, &M->nf_cell, &M->nf_w, &M->is_bnd, &M->row_abs, &M->cells,
                 &M->vol, &M->cf_ptr, &M->cf_facet, &M->bnd, &M->bnd_meas, &M->ellu,
-                &M->ellc};
+                &M->ellc, &M->flux_cell, &M->flux_ptr, &M->flux_inc};
   for (Buf* b : all)
     if (b->p) cudaFree(b->p);
   for (auto* v : {&M->anc, &M->lvl_ptr, &M->lvl_idx})
@@ -1192,6 +1196,8 @@ int mg_mesh_trim(mg_mesh* M) {
     b->p = nullptr;
     b->bytes = 0;
   }
+  for (mg::FluxBuffer& b : M->flux_scratch) cudaFree(b.p);
+  M->flux_scratch.clear();
   M->ev_valid = false;
   M->ck_valid = false;  M->ck_gen++;
   M->seg_full = false;
@@ -2403,6 +2409,40 @@ const HostMesh* host_mesh(const mg_mesh* M) { return M ? &M->hm : nullptr; }
 int mesh_device(const mg_mesh* M) { return M->device; }
 int mesh_graph_chunk(const mg_mesh* M) { return M->chunk; }
 void add_launches(mg_mesh* M, int64_t n) { M->launches += n; }
+
+void mesh_take_scratch(mg_mesh* M, std::vector<FluxBuffer>& bufs) {
+  std::lock_guard<std::mutex> lock(M->flux_mu);
+  bufs.clear();
+  bufs.swap(M->flux_scratch);
+}
+
+bool mesh_keep_scratch(mg_mesh* M, std::vector<FluxBuffer>& bufs) {
+  std::lock_guard<std::mutex> lock(M->flux_mu);
+  if (!M->flux_scratch.empty()) return false;
+  bufs.swap(M->flux_scratch);
+  return true;
+}
+
+std::mutex& mesh_flux_mutex(mg_mesh* M) { return M->flux_mu; }
+
+bool mesh_flux_geometry(mg_mesh* M, FluxGeometry* g) {
+  if (!M->flux_inc.p) return false;
+  g->cell = P<const float4>(M->flux_cell);
+  g->inc_ptr = P<const int32_t>(M->flux_ptr);
+  g->inc = P<const int4>(M->flux_inc);
+  g->cells = P<const int32_t>(M->cells);
+  return true;
+}
+
+int mesh_set_flux_geometry(mg_mesh* M, const std::vector<float>& cell,
+                           const std::vector<int32_t>& ptr, const std::vector<int4>& inc,
+                           FluxGeometry* g) {
+  MG_TRY(upload(M->flux_cell, cell));
+  MG_TRY(upload(M->flux_ptr, ptr));
+  MG_TRY(upload(M->flux_inc, inc));   // last: its presence marks the set
+  mesh_flux_geometry(M, g);
+  return MG_OK;
+}
 
 int mesh_view(mg_mesh* M, MeshView* v) {
   if (!M || !v) return MG_ERR_ARG;

@@ -3,6 +3,8 @@
 #pragma once
 
 #include <cstdint>
+#include <mutex>
+#include <vector>
 
 #include "../../include/mgwave.h"
 #include "kernels.cuh"
@@ -38,6 +40,28 @@ const HostMesh* host_mesh(const mg_mesh* mesh);
 int mesh_device(const mg_mesh* mesh);
 int mesh_graph_chunk(const mg_mesh* mesh);   // steps per CUDA-graph chunk (0: off)
 void add_launches(mg_mesh* mesh, int64_t n);
+
+// Work buffers of the flux path's calls: taken from the handle for a call, and
+// left on it again (false: it holds a set already).
+struct FluxBuffer {
+  void* p;
+  size_t bytes;
+};
+void mesh_take_scratch(mg_mesh* mesh, std::vector<FluxBuffer>& bufs);
+bool mesh_keep_scratch(mg_mesh* mesh, std::vector<FluxBuffer>& bufs);
+
+// Packed geometry of the flux path, kept on the handle.
+struct FluxGeometry {
+  const float4* cell = nullptr;      // per cell: rows, gradients
+  const int32_t* inc_ptr = nullptr;  // [n + 1]
+  const int4* inc = nullptr;         // per node and incident cell: {cell, weights}
+  const int32_t* cells = nullptr;    // [m][d + 1] rows
+};
+std::mutex& mesh_flux_mutex(mg_mesh* mesh);   // held around the next two
+bool mesh_flux_geometry(mg_mesh* mesh, FluxGeometry* out);   // false: not built yet
+int mesh_set_flux_geometry(mg_mesh* mesh, const std::vector<float>& cell,
+                           const std::vector<int32_t>& inc_ptr, const std::vector<int4>& inc,
+                           FluxGeometry* out);
 
 // One problem of a multi-instance batch, prepared on its own handle: device
 // inputs staged, coefficients and FP32 wavelet computed, event lists built,

@@ -28,6 +28,8 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "../../include/mgwave.h"
@@ -84,38 +86,147 @@ __global__ void k_flux_coefs(CoefArgs c, const double* __restrict__ xi, double d
   out[r] = make_float2((float)(dt / C), (float)RS);
 }
 
-// q^(k) <- (1 - dt zeta_k) q^(k) + dt sum_a grad[a][k] p[v_a]
+__device__ __forceinline__ float4 fma4f(float a, float4 x, float4 y) {
+  return make_float4(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y), fmaf(a, x.z, y.z), fmaf(a, x.w, y.w));
+}
+__device__ __forceinline__ void add_source(const DevEvents& ev, int s0, int s1, int c4, float f,
+                                           float4& rhs) {
+  for (int s = s0; s < s1; ++s) {
+    const int d = __ldg(ev.src_shot + s) - 4 * c4;
+    if (d == 0) rhs.x += f;
+    if (d == 1) rhs.y += f;
+    if (d == 2) rhs.z += f;
+    if (d == 3) rhs.w += f;
+  }
+}
+__device__ __forceinline__ void record(const DevEvents& ev, int r0, int r1, int c4, float* traces,
+                                       int nt, int l, const float4& pv) {
+  for (int r = r0; r < r1; ++r) {
+    const int d = __ldg(ev.rec_shot + r) - 4 * c4;
+    if (d < 0 || d > 3) continue;
+    const float v = d == 0 ? pv.x : d == 1 ? pv.y : d == 2 ? pv.z : pv.w;
+    traces[(int64_t)__ldg(ev.rec_trace + r) * nt + l] = v;
+  }
+}
+
+// Damping factors 1 - dt zeta of the cells; *bad is set when a value is
+// negative or not finite.
+__global__ void k_flux_keep(int64_t count, const double* __restrict__ zeta, float dt,
+                            float* __restrict__ keep, int* bad) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= count) return;
+  const double z = zeta ? zeta[i] : 0.0;
+  if (!(z >= 0.0) || !isfinite(z)) *bad = 1;
+  keep[i] = 1.0f - dt * (float)z;
+}
+
+// Geometry packed so that a warp reads a cell's (an incidence's) constants with
+// a few 16-byte loads instead of one load per value, which took more of the
+// load pipe than the states: cell e, kCellW<D> float4: its D + 1 rows, then the
+// gradients [a][k]; incidence: {cell, |e| dphi_i/dx_k}.
 template <int D>
-__global__ void k_flux_q(int64_t m, int ld4, const int32_t* __restrict__ cells,
-                         const float* __restrict__ grad, const float* __restrict__ damp,
-                         const float4* __restrict__ p, float4* __restrict__ q, float dt,
-                         StepRef sr, Slots sl) {
+constexpr int kCellW = ((D + 1) * (D + 1) + 3) / 4;
+
+template <int D>
+struct Cell {
+  int v[D + 1];
+  float g[D + 1][D];
+};
+template <int D>
+__device__ __forceinline__ Cell<D> load_cell(const float4* __restrict__ cell, int64_t e) {
+  float w[4 * kCellW<D>];
+#pragma unroll
+  for (int i = 0; i < kCellW<D>; ++i) {
+    const float4 x = __ldg(cell + e * kCellW<D> + i);
+    w[4 * i] = x.x;
+    w[4 * i + 1] = x.y;
+    w[4 * i + 2] = x.z;
+    w[4 * i + 3] = x.w;
+  }
+  Cell<D> c;
+#pragma unroll
+  for (int a = 0; a <= D; ++a) {
+    c.v[a] = __float_as_int(w[a]);
+#pragma unroll
+    for (int k = 0; k < D; ++k) c.g[a][k] = w[D + 1 + a * D + k];
+  }
+  return c;
+}
+
+// One thread per float4 of shots (threadIdx.x) of one cell or node
+// (threadIdx.y): see item_block.
+struct Item {
+  int64_t i;
+  int c4;
+  bool ok;
+};
+__device__ __forceinline__ Item item_of(int64_t count, int ld4) {
+  Item t;
+  t.i = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
+  t.c4 = blockIdx.y * blockDim.x + threadIdx.x;
+  t.ok = t.i < count && t.c4 < ld4;
+  return t;
+}
+
+// q^(k) <- keep_k q^(k) + dt sum_a grad[a][k] p[v_a]; SIGN < 0, dt = 1: the
+// adjoint's Qt^(k) <- keep_k Qt^(k) - sum_a grad[a][k] r[v_a].
+//
+// Bound by the states' traffic through L2: a step gathers and writes 900 MB at
+// 62,641 nodes, 124,416 cells and 128 shots in its two kernels, 98 us (with one
+// load per constant and 64-bit divisions 103).
+// Advancing 32 shots at a time, with states that fit L2, takes 88 us there, 16
+// shots at a time 142.
+template <int D, int SIGN>
+__global__ void __launch_bounds__(256) k_flux_q(int64_t m, int ld4,
+                                                const float4* __restrict__ cell,
+                                                const float* __restrict__ keep,
+                                                const float4* __restrict__ p,
+                                                float4* __restrict__ q, float dt, StepRef sr,
+                                                Slots sl) {
+  const Item t = item_of(m, ld4);
+  if (!t.ok) return;
+  const Cell<D> c = load_cell<D>(cell, t.i);
+  float kp[D];
+#pragma unroll
+  for (int k = 0; k < D; ++k) kp[k] = __ldg(keep + t.i * D + k);
+  // the constants are complete before the call's first step
   pdl_sync();
   if (sl.seg) p = slot_of(sl, step_of(sr));
-  const int64_t total = m * ld4;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = t / ld4;
-    const int c4 = (int)(t - e * ld4);
-    float4 pv[D + 1];
+  float4 pv[D + 1], o[D];
 #pragma unroll
-    for (int a = 0; a <= D; ++a) pv[a] = __ldg(p + (int64_t)__ldg(cells + e * (D + 1) + a) * ld4 + c4);
+  for (int k = 0; k < D; ++k) o[k] = q[((int64_t)k * m + t.i) * ld4 + t.c4];
+#pragma unroll
+  for (int a = 0; a <= D; ++a) pv[a] = __ldg(p + (int64_t)c.v[a] * ld4 + t.c4);
+#pragma unroll
+  for (int k = 0; k < D; ++k) {
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int a = 0; a <= D; ++a) acc = fma4f(c.g[a][k], pv[a], acc);
+    float4* qp = q + ((int64_t)k * m + t.i) * ld4 + t.c4;
+    *qp = SIGN > 0 ? make_float4(fmaf(kp[k], o[k].x, dt * acc.x), fmaf(kp[k], o[k].y, dt * acc.y),
+                                 fmaf(kp[k], o[k].z, dt * acc.z), fmaf(kp[k], o[k].w, dt * acc.w))
+                   : make_float4(fmaf(kp[k], o[k].x, -acc.x), fmaf(kp[k], o[k].y, -acc.y),
+                                 fmaf(kp[k], o[k].z, -acc.z), fmaf(kp[k], o[k].w, -acc.w));
+  }
+}
+
+// bt_n += sum_{e ni i} sum_k w[e,i,k] q_n^(k)_e for NQ flux fields, in the order
+// of the incidences.  One incidence at a time: with two, three or four of them
+// in flight the registers cost more warps than the loads gain (62,641 nodes,
+// 128 shots, forward step 98, 112, 114, 128 us).
+template <int D, int NQ>
+__device__ __forceinline__ void gather_flux(int s0, int s1, const int4* __restrict__ inc,
+                                            int64_t m, int ld4, int c4,
+                                            const float4* const (&q)[NQ], float4 (&bt)[NQ]) {
+#pragma unroll 1
+  for (int s = s0; s < s1; ++s) {
+    const int4 w = __ldg(inc + s);
 #pragma unroll
     for (int k = 0; k < D; ++k) {
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      const float wk = __int_as_float(k == 0 ? w.y : k == 1 ? w.z : w.w);
 #pragma unroll
-      for (int a = 0; a <= D; ++a) {
-        const float g = __ldg(grad + (e * (D + 1) + a) * D + k);
-        acc.x = fmaf(g, pv[a].x, acc.x);
-        acc.y = fmaf(g, pv[a].y, acc.y);
-        acc.z = fmaf(g, pv[a].z, acc.z);
-        acc.w = fmaf(g, pv[a].w, acc.w);
-      }
-      const float keep = 1.0f - dt * __ldg(damp + e * D + k);
-      float4* qp = q + ((int64_t)k * m + e) * ld4 + c4;
-      const float4 o = *qp;
-      *qp = make_float4(fmaf(keep, o.x, dt * acc.x), fmaf(keep, o.y, dt * acc.y),
-                        fmaf(keep, o.z, dt * acc.z), fmaf(keep, o.w, dt * acc.w));
+      for (int n = 0; n < NQ; ++n)
+        bt[n] = fma4f(wk, __ldg(q[n] + ((int64_t)k * m + w.x) * ld4 + c4), bt[n]);
     }
   }
 }
@@ -123,64 +234,37 @@ __global__ void k_flux_q(int64_t m, int ld4, const int32_t* __restrict__ cells,
 // pout <- p + dt/C (f delta_src - (R+S) p - sum_{e ni i} sum_k w[e,i,k] q^(k)_e)
 // (pout may be p); sources and traces of the row's shots
 template <int D>
-__global__ void k_flux_p(int64_t n, int64_t m, int ld4, const int64_t* __restrict__ nc_ptr,
-                         const int32_t* __restrict__ nc_cell, const float* __restrict__ w,
-                         const float2* __restrict__ coef, const float4* __restrict__ q,
-                         const float4* p, float4* pout, const int32_t* __restrict__ src_ptr,
-                         const int32_t* __restrict__ src_shot, const int32_t* __restrict__ rec_ptr,
-                         const int32_t* __restrict__ rec_shot,
-                         const int32_t* __restrict__ rec_trace, const float* __restrict__ fl,
-                         float* __restrict__ traces, int nt, StepRef sr, Slots sl) {
+__global__ void __launch_bounds__(256) k_flux_p(
+    int64_t n, int64_t m, int ld4, const int32_t* __restrict__ inc_ptr,
+    const int4* __restrict__ inc, const float2* __restrict__ coef, const float4* __restrict__ q,
+    const float4* p, float4* pout, DevEvents ev, const float* __restrict__ fl,
+    float* __restrict__ traces, int nt, StepRef sr, Slots sl) {
   pdl_sync();
   const int l = step_of(sr);
-  const float f = __ldg(fl + l);
   if (sl.seg) {   // p_l in slot l, p_{l+1} into the next slot
     pout = slot_of(sl, l);
     p = pout;
     pout += sl.ns4;
   }
-  const int64_t total = n * ld4;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = t / ld4;
-    const int c4 = (int)(t - i * ld4);
-    float4 bt = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int64_t s = __ldg(nc_ptr + i); s < __ldg(nc_ptr + i + 1); ++s) {
-      const int64_t e = __ldg(nc_cell + s);
-#pragma unroll
-      for (int k = 0; k < D; ++k) {
-        const float wk = __ldg(w + s * D + k);
-        const float4 qv = __ldg(q + ((int64_t)k * m + e) * ld4 + c4);
-        bt.x = fmaf(wk, qv.x, bt.x);
-        bt.y = fmaf(wk, qv.y, bt.y);
-        bt.z = fmaf(wk, qv.z, bt.z);
-        bt.w = fmaf(wk, qv.w, bt.w);
-      }
-    }
-    const float2 c = __ldg(coef + i);
-    float4 rhs = make_float4(-bt.x, -bt.y, -bt.z, -bt.w);
-    const int s0 = __ldg(src_ptr + i), s1 = __ldg(src_ptr + i + 1);
-    for (int s = s0; s < s1; ++s) {
-      const int d = __ldg(src_shot + s) - 4 * c4;
-      if (d == 0) rhs.x += f;
-      if (d == 1) rhs.y += f;
-      if (d == 2) rhs.z += f;
-      if (d == 3) rhs.w += f;
-    }
-    float4 pv = p[t];
-    pv.x = fmaf(c.x, fmaf(-c.y, pv.x, rhs.x), pv.x);
-    pv.y = fmaf(c.x, fmaf(-c.y, pv.y, rhs.y), pv.y);
-    pv.z = fmaf(c.x, fmaf(-c.y, pv.z, rhs.z), pv.z);
-    pv.w = fmaf(c.x, fmaf(-c.y, pv.w, rhs.w), pv.w);
-    pout[t] = pv;
-    const int r0 = __ldg(rec_ptr + i), r1 = __ldg(rec_ptr + i + 1);
-    for (int r = r0; r < r1; ++r) {
-      const int d = __ldg(rec_shot + r) - 4 * c4;
-      if (d < 0 || d > 3) continue;
-      const float v = d == 0 ? pv.x : d == 1 ? pv.y : d == 2 ? pv.z : pv.w;
-      traces[(int64_t)__ldg(rec_trace + r) * nt + l] = v;
-    }
-  }
+  const Item it = item_of(n, ld4);
+  if (!it.ok) return;
+  const int64_t i = it.i, t = i * ld4 + it.c4;
+  const int c4 = it.c4;
+  float4 pv = p[t];
+  const float2 c = __ldg(coef + i);
+  const int s0 = __ldg(ev.src_ptr + i), s1 = __ldg(ev.src_ptr + i + 1);
+  const int r0 = __ldg(ev.rec_ptr + i), r1 = __ldg(ev.rec_ptr + i + 1);
+  float4 bt[1] = {make_float4(0.f, 0.f, 0.f, 0.f)};
+  const float4* const qs[1] = {q};
+  gather_flux<D, 1>(__ldg(inc_ptr + i), __ldg(inc_ptr + i + 1), inc, m, ld4, c4, qs, bt);
+  float4 rhs = make_float4(-bt[0].x, -bt[0].y, -bt[0].z, -bt[0].w);
+  if (s0 != s1) add_source(ev, s0, s1, c4, __ldg(fl + l), rhs);
+  pv.x = fmaf(c.x, fmaf(-c.y, pv.x, rhs.x), pv.x);
+  pv.y = fmaf(c.x, fmaf(-c.y, pv.y, rhs.y), pv.y);
+  pv.z = fmaf(c.x, fmaf(-c.y, pv.z, rhs.z), pv.z);
+  pv.w = fmaf(c.x, fmaf(-c.y, pv.w, rhs.w), pv.w);
+  pout[t] = pv;
+  if (r0 != r1) record(ev, r0, r1, c4, traces, nt, l, pv);
 }
 
 // C_i = sum_{e ni i} x[e] |e| / (d+1) in FP64 (x = eps, or a direction)
@@ -201,76 +285,42 @@ __global__ void k_flux_ratio(int64_t n, const double* __restrict__ dC, const dou
 // Tangent node update: p as in k_flux_p, and
 // dp <- dp + dt/C (-(R+S) dp - sum B^T dq) - ratio (p_new - p_old); traces of dp.
 template <int D>
-__global__ void k_flux_p_tan(int64_t n, int64_t m, int ld4, const int64_t* __restrict__ nc_ptr,
-                             const int32_t* __restrict__ nc_cell, const float* __restrict__ w,
-                             const float2* __restrict__ coef, const float* __restrict__ ratio,
-                             const float4* __restrict__ q, const float4* __restrict__ dq,
-                             float4* __restrict__ p, float4* __restrict__ dp,
-                             const int32_t* __restrict__ src_ptr,
-                             const int32_t* __restrict__ src_shot,
-                             const int32_t* __restrict__ rec_ptr,
-                             const int32_t* __restrict__ rec_shot,
-                             const int32_t* __restrict__ rec_trace,
-                             const float* __restrict__ fl, float* __restrict__ traces, int nt,
-                             StepRef sr) {
+__global__ void __launch_bounds__(256) k_flux_p_tan(
+    int64_t n, int64_t m, int ld4, const int32_t* __restrict__ inc_ptr,
+    const int4* __restrict__ inc, const float2* __restrict__ coef,
+    const float* __restrict__ ratio, const float4* __restrict__ q,
+    const float4* __restrict__ dq, float4* __restrict__ p, float4* __restrict__ dp, DevEvents ev,
+    const float* __restrict__ fl, float* __restrict__ traces, int nt, StepRef sr) {
   pdl_sync();
   const int l = step_of(sr);
-  const float f = __ldg(fl + l);
-  const int64_t total = n * ld4;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = t / ld4;
-    const int c4 = (int)(t - i * ld4);
-    float4 bt = make_float4(0.f, 0.f, 0.f, 0.f), dbt = bt;
-    for (int64_t s = __ldg(nc_ptr + i); s < __ldg(nc_ptr + i + 1); ++s) {
-      const int64_t e = __ldg(nc_cell + s);
-#pragma unroll
-      for (int k = 0; k < D; ++k) {
-        const float wk = __ldg(w + s * D + k);
-        const int64_t at = ((int64_t)k * m + e) * ld4 + c4;
-        const float4 qv = __ldg(q + at), dv = __ldg(dq + at);
-        bt.x = fmaf(wk, qv.x, bt.x);
-        bt.y = fmaf(wk, qv.y, bt.y);
-        bt.z = fmaf(wk, qv.z, bt.z);
-        bt.w = fmaf(wk, qv.w, bt.w);
-        dbt.x = fmaf(wk, dv.x, dbt.x);
-        dbt.y = fmaf(wk, dv.y, dbt.y);
-        dbt.z = fmaf(wk, dv.z, dbt.z);
-        dbt.w = fmaf(wk, dv.w, dbt.w);
-      }
-    }
-    const float2 c = __ldg(coef + i);
-    const float rt = __ldg(ratio + i);
-    float4 rhs = make_float4(-bt.x, -bt.y, -bt.z, -bt.w);
-    const int s0 = __ldg(src_ptr + i), s1 = __ldg(src_ptr + i + 1);
-    for (int s = s0; s < s1; ++s) {
-      const int d = __ldg(src_shot + s) - 4 * c4;
-      if (d == 0) rhs.x += f;
-      if (d == 1) rhs.y += f;
-      if (d == 2) rhs.z += f;
-      if (d == 3) rhs.w += f;
-    }
-    float4 pv = p[t], dv = dp[t];
-    const float4 inc = make_float4(fmaf(-c.y, pv.x, rhs.x), fmaf(-c.y, pv.y, rhs.y),
-                                   fmaf(-c.y, pv.z, rhs.z), fmaf(-c.y, pv.w, rhs.w));
-    dv.x = fmaf(-rt, c.x * inc.x, fmaf(c.x, fmaf(-c.y, dv.x, -dbt.x), dv.x));
-    dv.y = fmaf(-rt, c.x * inc.y, fmaf(c.x, fmaf(-c.y, dv.y, -dbt.y), dv.y));
-    dv.z = fmaf(-rt, c.x * inc.z, fmaf(c.x, fmaf(-c.y, dv.z, -dbt.z), dv.z));
-    dv.w = fmaf(-rt, c.x * inc.w, fmaf(c.x, fmaf(-c.y, dv.w, -dbt.w), dv.w));
-    pv.x = fmaf(c.x, inc.x, pv.x);
-    pv.y = fmaf(c.x, inc.y, pv.y);
-    pv.z = fmaf(c.x, inc.z, pv.z);
-    pv.w = fmaf(c.x, inc.w, pv.w);
-    p[t] = pv;
-    dp[t] = dv;
-    const int r0 = __ldg(rec_ptr + i), r1 = __ldg(rec_ptr + i + 1);
-    for (int r = r0; r < r1; ++r) {
-      const int d = __ldg(rec_shot + r) - 4 * c4;
-      if (d < 0 || d > 3) continue;
-      const float v = d == 0 ? dv.x : d == 1 ? dv.y : d == 2 ? dv.z : dv.w;
-      traces[(int64_t)__ldg(rec_trace + r) * nt + l] = v;
-    }
-  }
+  const Item it = item_of(n, ld4);
+  if (!it.ok) return;
+  const int64_t i = it.i, t = i * ld4 + it.c4;
+  const int c4 = it.c4;
+  float4 pv = p[t], dv = dp[t];
+  const float2 c = __ldg(coef + i);
+  const float rt = __ldg(ratio + i);
+  const int s0 = __ldg(ev.src_ptr + i), s1 = __ldg(ev.src_ptr + i + 1);
+  const int r0 = __ldg(ev.rec_ptr + i), r1 = __ldg(ev.rec_ptr + i + 1);
+  float4 b2[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+  const float4* const qs[2] = {q, dq};
+  gather_flux<D, 2>(__ldg(inc_ptr + i), __ldg(inc_ptr + i + 1), inc, m, ld4, c4, qs, b2);
+  const float4 dbt = b2[1];
+  float4 rhs = make_float4(-b2[0].x, -b2[0].y, -b2[0].z, -b2[0].w);
+  if (s0 != s1) add_source(ev, s0, s1, c4, __ldg(fl + l), rhs);
+  const float4 inc4 = make_float4(fmaf(-c.y, pv.x, rhs.x), fmaf(-c.y, pv.y, rhs.y),
+                                  fmaf(-c.y, pv.z, rhs.z), fmaf(-c.y, pv.w, rhs.w));
+  dv.x = fmaf(-rt, c.x * inc4.x, fmaf(c.x, fmaf(-c.y, dv.x, -dbt.x), dv.x));
+  dv.y = fmaf(-rt, c.x * inc4.y, fmaf(c.x, fmaf(-c.y, dv.y, -dbt.y), dv.y));
+  dv.z = fmaf(-rt, c.x * inc4.z, fmaf(c.x, fmaf(-c.y, dv.z, -dbt.z), dv.z));
+  dv.w = fmaf(-rt, c.x * inc4.w, fmaf(c.x, fmaf(-c.y, dv.w, -dbt.w), dv.w));
+  pv.x = fmaf(c.x, inc4.x, pv.x);
+  pv.y = fmaf(c.x, inc4.y, pv.y);
+  pv.z = fmaf(c.x, inc4.z, pv.z);
+  pv.w = fmaf(c.x, inc4.w, pv.w);
+  p[t] = pv;
+  dp[t] = dv;
+  if (r0 != r1) record(ev, r0, r1, c4, traces, nt, l, dv);
 }
 
 // Adjoint node kernel of reverse step l (p_l in slot l mod K of sl, p_{l+1}
@@ -284,110 +334,59 @@ __global__ void k_flux_p_tan(int64_t n, int64_t m, int ld4, const int64_t* __res
 // its FP32 rate: one FP64 add per node and step), then stores r = a dt/C
 // and tp = a - (R+S) r.
 template <int D>
-__global__ void k_flux_adj_p(int64_t n, int64_t m, int ld4, const int64_t* __restrict__ nc_ptr,
-                             const int32_t* __restrict__ nc_cell, const float* __restrict__ w,
-                             const float2* __restrict__ coef, const float4* __restrict__ Qt,
-                             float4* __restrict__ tp, float4* __restrict__ rr, Slots sl,
-                             double* __restrict__ hacc, const int32_t* __restrict__ rec_ptr,
-                             const int32_t* __restrict__ rec_shot,
-                             const int32_t* __restrict__ rec_trace,
-                             const float* __restrict__ W, int nt, StepRef sr, float dt) {
+__global__ void __launch_bounds__(256) k_flux_adj_p(
+    int64_t n, int64_t m, int ld4, const int32_t* __restrict__ inc_ptr,
+    const int4* __restrict__ inc, const float2* __restrict__ coef,
+    const float4* __restrict__ Qt, float4* __restrict__ tp, float4* __restrict__ rr, Slots sl,
+    double* __restrict__ hacc, DevEvents ev, const float* __restrict__ W, int nt, StepRef sr,
+    float dt) {
   pdl_sync();
   const int l = step_of(sr);
   const bool first = l == nt - 1;
   const float4* __restrict__ p0 = slot_of(sl, l);   // p_l; p_{l+1} in the next slot
   const float4* __restrict__ p1 = p0 + sl.ns4;
-  const int64_t total = n * ld4;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = t / ld4;
-    const int c4 = (int)(t - i * ld4);
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (!first) {
-      float4 bt = a;
-      for (int64_t s = __ldg(nc_ptr + i); s < __ldg(nc_ptr + i + 1); ++s) {
-        const int64_t e = __ldg(nc_cell + s);
-#pragma unroll
-        for (int k = 0; k < D; ++k) {
-          const float wk = __ldg(w + s * D + k);
-          const float4 qv = __ldg(Qt + ((int64_t)k * m + e) * ld4 + c4);
-          bt.x = fmaf(wk, qv.x, bt.x);
-          bt.y = fmaf(wk, qv.y, bt.y);
-          bt.z = fmaf(wk, qv.z, bt.z);
-          bt.w = fmaf(wk, qv.w, bt.w);
-        }
-      }
-      const float4 tv = tp[t];
-      a = make_float4(fmaf(dt, bt.x, tv.x), fmaf(dt, bt.y, tv.y), fmaf(dt, bt.z, tv.z),
-                      fmaf(dt, bt.w, tv.w));
-    }
-    const int r0 = __ldg(rec_ptr + i), r1 = __ldg(rec_ptr + i + 1);
-    for (int r = r0; r < r1; ++r) {
-      const int d = __ldg(rec_shot + r) - 4 * c4;
-      if (d < 0 || d > 3) continue;
-      const float v = __ldg(W + (int64_t)__ldg(rec_trace + r) * nt + l);
-      if (d == 0) a.x += v;
-      if (d == 1) a.y += v;
-      if (d == 2) a.z += v;
-      if (d == 3) a.w += v;
-    }
-    const float4 x1 = __ldg(p1 + t), x0 = __ldg(p0 + t);
-    float h = a.x * (x1.x - x0.x);
-    h = fmaf(a.y, x1.y - x0.y, h);
-    h = fmaf(a.z, x1.z - x0.z, h);
-    h = fmaf(a.w, x1.w - x0.w, h);
-    // ld4 is a power of two or a multiple of 32, and t mod 32 is the lane:
-    // the gw lanes of a node's segment are active together
-    const int gw = ld4 < 32 ? ld4 : 32;
-    const int lane = threadIdx.x & 31;
-    const unsigned gmask =
-        gw == 32 ? 0xffffffffu : (((1u << gw) - 1u) << (lane & ~(gw - 1)));
-    for (int off = gw / 2; off > 0; off >>= 1) h += __shfl_xor_sync(gmask, h, off);
-    if ((c4 & (gw - 1)) == 0) {
-      const int nseg = ld4 < 32 ? 1 : ld4 / 32;
-      hacc[i * nseg + c4 / 32] += (double)h;
-    }
-    const float2 c = __ldg(coef + i);
-    const float4 r = make_float4(a.x * c.x, a.y * c.x, a.z * c.x, a.w * c.x);
-    rr[t] = r;
-    tp[t] = make_float4(fmaf(-c.y, r.x, a.x), fmaf(-c.y, r.y, a.y), fmaf(-c.y, r.z, a.z),
-                        fmaf(-c.y, r.w, a.w));
+  const Item it = item_of(n, ld4);
+  if (!it.ok) return;
+  const int64_t i = it.i, t = i * ld4 + it.c4;
+  const int c4 = it.c4;
+  const float4 x1 = __ldg(p1 + t), x0 = __ldg(p0 + t);
+  const float2 c = __ldg(coef + i);
+  const int r0 = __ldg(ev.rec_ptr + i), r1 = __ldg(ev.rec_ptr + i + 1);
+  float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (!first) {
+    const float4 tv = tp[t];
+    float4 bt[1] = {a};
+    const float4* const qs[1] = {Qt};
+    gather_flux<D, 1>(__ldg(inc_ptr + i), __ldg(inc_ptr + i + 1), inc, m, ld4, c4, qs, bt);
+    a = fma4f(dt, bt[0], tv);
   }
-}
-
-// Adjoint cell kernel: Qt^(k) <- (1 - dt zeta_k) Qt^(k) - sum_a dphi_a/dx_k r[v_a]
-template <int D>
-__global__ void k_flux_adj_q(int64_t m, int ld4, const int32_t* __restrict__ cells,
-                             const float* __restrict__ grad, const float* __restrict__ damp,
-                             const float4* __restrict__ rr, float4* __restrict__ Qt, float dt) {
-  pdl_sync();
-  const int64_t total = m * ld4;
-  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = t / ld4;
-    const int c4 = (int)(t - e * ld4);
-    float4 rv[D + 1];
-#pragma unroll
-    for (int a = 0; a <= D; ++a)
-      rv[a] = __ldg(rr + (int64_t)__ldg(cells + e * (D + 1) + a) * ld4 + c4);
-#pragma unroll
-    for (int k = 0; k < D; ++k) {
-      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int a = 0; a <= D; ++a) {
-        const float g = __ldg(grad + (e * (D + 1) + a) * D + k);
-        acc.x = fmaf(g, rv[a].x, acc.x);
-        acc.y = fmaf(g, rv[a].y, acc.y);
-        acc.z = fmaf(g, rv[a].z, acc.z);
-        acc.w = fmaf(g, rv[a].w, acc.w);
-      }
-      const float keep = 1.0f - dt * __ldg(damp + e * D + k);
-      float4* qp = Qt + ((int64_t)k * m + e) * ld4 + c4;
-      const float4 o = *qp;
-      *qp = make_float4(fmaf(keep, o.x, -acc.x), fmaf(keep, o.y, -acc.y),
-                        fmaf(keep, o.z, -acc.z), fmaf(keep, o.w, -acc.w));
-    }
+  for (int r = r0; r < r1; ++r) {
+    const int d = __ldg(ev.rec_shot + r) - 4 * c4;
+    if (d < 0 || d > 3) continue;
+    const float v = __ldg(W + (int64_t)__ldg(ev.rec_trace + r) * nt + l);
+    if (d == 0) a.x += v;
+    if (d == 1) a.y += v;
+    if (d == 2) a.z += v;
+    if (d == 3) a.w += v;
   }
+  float h = a.x * (x1.x - x0.x);
+  h = fmaf(a.y, x1.y - x0.y, h);
+  h = fmaf(a.z, x1.z - x0.z, h);
+  h = fmaf(a.w, x1.w - x0.w, h);
+  // ld4 is a power of two or a multiple of 32 and blockDim.x is ld4 or a multiple of 32:
+  // the gw lanes of a node's segment are consecutive and active together
+  const int gw = ld4 < 32 ? ld4 : 32;
+  const int lane = (threadIdx.y * blockDim.x + threadIdx.x) & 31;
+  const unsigned gmask = gw == 32 ? 0xffffffffu : (((1u << gw) - 1u) << (lane & ~(gw - 1)));
+  for (int off = gw / 2; off > 0; off >>= 1) h += __shfl_xor_sync(gmask, h, off);
+  if ((c4 & (gw - 1)) == 0) {
+    const int nseg = ld4 < 32 ? 1 : ld4 / 32;
+    hacc[i * nseg + c4 / 32] += (double)h;
+  }
+  const float4 r = make_float4(a.x * c.x, a.y * c.x, a.z * c.x, a.w * c.x);
+  rr[t] = r;
+  tp[t] = make_float4(fmaf(-c.y, r.x, a.x), fmaf(-c.y, r.y, a.y), fmaf(-c.y, r.z, a.z),
+                      fmaf(-c.y, r.w, a.w));
 }
 
 // gC_i = -sum_seg hacc[i][seg] / C_i (fixed order over the shot segments)
@@ -411,45 +410,74 @@ __global__ void k_flux_cell_grad(int64_t m, int k1, const int32_t* __restrict__ 
   g[e] = vol[e] / k1 * s;
 }
 
+// Work buffers of a call, left on the handle for the next one (in the order of
+// use, so the same call finds its sizes again).  A call takes them away from
+// the handle while it runs: a second thread's call finds none and allocates
+// its own.  More than kKeepBytes, or a second set, is freed at the end.  The
+// calls end with a stream synchronisation, on errors in the destructor: the
+// next call may use another stream.
+constexpr size_t kKeepBytes = (size_t)2 << 30;
 struct Scratch {
+  mg_mesh* M;
   cudaStream_t st;
-  std::vector<void*> p;
-  explicit Scratch(cudaStream_t s) : st(s) {}
+  size_t next = 0;
+  std::vector<FluxBuffer> own;
+  Scratch(mg_mesh* m, cudaStream_t s) : M(m), st(s) { mesh_take_scratch(M, own); }
   ~Scratch() {
-    for (void* x : p) cudaFreeAsync(x, st);
+    cudaStreamSynchronize(st);
+    size_t total = 0;
+    for (const FluxBuffer& b : own) total += b.bytes;
+    if (total > kKeepBytes || !mesh_keep_scratch(M, own))
+      for (const FluxBuffer& b : own) cudaFree(b.p);
   }
-  template <class T>
-  T* put(const std::vector<T>& v) {
-    void* x = nullptr;
-    if (cudaMallocAsync(&x, std::max<size_t>(v.size(), 1) * sizeof(T), st) != cudaSuccess)
-      return nullptr;
-    p.push_back(x);
-    if (!v.empty() &&
-        cudaMemcpyAsync(x, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, st) !=
-            cudaSuccess)
-      return nullptr;
-    return static_cast<T*>(x);
-  }
-  template <class T>
-  T* put(const T* src, size_t count) {  // host array
-    return put(std::vector<T>(src, src + count));
-  }
+  Scratch(const Scratch&) = delete;
+  Scratch& operator=(const Scratch&) = delete;
   template <class T>
   T* get(size_t count) {
-    void* x = nullptr;
-    if (cudaMallocAsync(&x, std::max<size_t>(count, 1) * sizeof(T), st) != cudaSuccess)
-      return nullptr;
-    p.push_back(x);
-    return static_cast<T*>(x);
+    const size_t bytes = std::max<size_t>(count, 1) * sizeof(T);
+    if (next == own.size()) own.push_back({nullptr, 0});
+    FluxBuffer& b = own[next++];
+    if (b.bytes < bytes) {
+      cudaFree(b.p);
+      b = {nullptr, 0};
+      if (cudaMalloc(&b.p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        b.p = nullptr;
+        return nullptr;
+      }
+      b.bytes = bytes;
+    }
+    return static_cast<T*>(b.p);
   }
+  template <class T>
+  T* put(const T* src, size_t count) {   // host array
+    T* x = get<T>(count);
+    if (x && count &&
+        cudaMemcpyAsync(x, src, count * sizeof(T), cudaMemcpyHostToDevice, st) != cudaSuccess)
+      return nullptr;
+    return x;
+  }
+  template <class T>
+  T* put(const std::vector<T>& v) { return put(v.data(), v.size()); }
 };
+
+// Block and grid of a kernel over `count` cells or nodes of ld4 float4 each
+// (item_of): rows of up to 256 float4, no division in the kernel.
+struct ItemGrid {
+  dim3 block, grid;
+};
+ItemGrid item_grid(int64_t count, int ld4) {
+  const int ny = (ld4 + 255) / 256;
+  const int bx = ny == 1 ? ld4 : ((ld4 + ny - 1) / ny + 31) / 32 * 32, by = 256 / bx;
+  return {dim3(bx, by), dim3((unsigned)((count + by - 1) / by), ny)};
+}
 
 // Launch of a step kernel as a programmatic dependent (see pdl_sync).
 template <class... KArgs, class... Args>
-void launch_pdl(void (*kern)(KArgs...), int grid, cudaStream_t st, Args... args) {
+void launch_pdl(void (*kern)(KArgs...), const ItemGrid& g, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(256);
+  cfg.gridDim = g.grid;
+  cfg.blockDim = g.block;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -457,10 +485,6 @@ void launch_pdl(void (*kern)(KArgs...), int grid, cudaStream_t st, Args... args)
   cfg.attrs = at;
   cfg.numAttrs = 1;
   cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
-}
-
-int grid_for(int64_t total) {
-  return (int)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, 152 * 16));
 }
 
 // Everything the three entry points share: geometry, layer damping, event
@@ -474,39 +498,27 @@ struct Flux {
   MeshView V;
   CoefArgs c;
   const double* eps_d = nullptr;
-  int32_t* cells = nullptr;
-  float *grad = nullptr, *w = nullptr, *damp = nullptr;
-  int32_t *sp = nullptr, *ss = nullptr, *rp = nullptr, *rs = nullptr, *rt = nullptr;
+  FluxGeometry geo;
+  float* keep = nullptr;    // 1 - dt zeta
+  DevEvents ev{};
   float* fl = nullptr;      // f_l (FP32) per step, device
   float2* coef = nullptr;
 
   // flux update from p (or, with sl.seg, from the slot of step sr)
   void step_q(float* p, float* q, cudaStream_t s, StepRef sr = {0, nullptr},
               Slots sl = {nullptr, 0, 1}) const {
-    const int g = grid_for(m * ld4);
-    if (d == 2)
-      launch_pdl(k_flux_q<2>, g, s, m, ld4, cells, grad, damp,
-                 reinterpret_cast<const float4*>(p), reinterpret_cast<float4*>(q), (float)dt, sr,
-                 sl);
-    else
-      launch_pdl(k_flux_q<3>, g, s, m, ld4, cells, grad, damp,
-                 reinterpret_cast<const float4*>(p), reinterpret_cast<float4*>(q), (float)dt, sr,
-                 sl);
+    launch_pdl(d == 2 ? k_flux_q<2, 1> : k_flux_q<3, 1>, item_grid(m, ld4), s, m, ld4, geo.cell,
+               keep, reinterpret_cast<const float4*>(p), reinterpret_cast<float4*>(q), (float)dt,
+               sr, sl);
   }
   // node update of step sr: p_{l+1} into pout (nullptr: in place over p),
   // or with sl.seg from the step's slot into the next one
   void step_p(const float* q, float* p, float* traces, StepRef sr, cudaStream_t s,
               float* pout = nullptr, Slots sl = {nullptr, 0, 1}) const {
-    const int g = grid_for(n * ld4);
-    float4* po = reinterpret_cast<float4*>(pout ? pout : p);
-    if (d == 2)
-      launch_pdl(k_flux_p<2>, g, s, n, m, ld4, c.nc_ptr, c.nc_cell, w, coef,
-                 reinterpret_cast<const float4*>(q), reinterpret_cast<const float4*>(p), po, sp,
-                 ss, rp, rs, rt, fl, traces, nt, sr, sl);
-    else
-      launch_pdl(k_flux_p<3>, g, s, n, m, ld4, c.nc_ptr, c.nc_cell, w, coef,
-                 reinterpret_cast<const float4*>(q), reinterpret_cast<const float4*>(p), po, sp,
-                 ss, rp, rs, rt, fl, traces, nt, sr, sl);
+    launch_pdl(d == 2 ? k_flux_p<2> : k_flux_p<3>, item_grid(n, ld4), s, n, m, ld4, geo.inc_ptr,
+               geo.inc, coef, reinterpret_cast<const float4*>(q),
+               reinterpret_cast<const float4*>(p), reinterpret_cast<float4*>(pout ? pout : p), ev,
+               fl, traces, nt, sr, sl);
   }
 };
 
@@ -552,6 +564,91 @@ struct Chunk {
   }
 };
 
+#define MG_FX(x)                  \
+  do {                            \
+    const int rc_ = (x);          \
+    if (rc_ != MG_OK) return rc_; \
+  } while (0)
+
+// The packed geometry of the handle's mesh, built on first use and kept with
+// it: gradients of the barycentric functions and incidence weights |e|
+// dphi_i/dx_k (FP64 -> FP32).
+int flux_geometry(mg_mesh* M, const HostMesh& hm, FluxGeometry& out) {
+  std::lock_guard<std::mutex> lock(mesh_flux_mutex(M));
+  if (mesh_flux_geometry(M, &out)) return MG_OK;
+  const int d = hm.dim, k1 = d + 1, cw = (k1 * k1 + 3) / 4;
+  const int64_t n = hm.n, m = hm.m;
+  std::vector<float> grad((size_t)m * k1 * d), cell((size_t)m * cw * 4, 0.0f);
+  int bad = 0;
+#pragma omp parallel for schedule(static) reduction(+ : bad)
+  for (int64_t e = 0; e < m; ++e) {
+    const int32_t* v = hm.cells.data() + (size_t)e * k1;
+    double E[kMaxDim][kMaxDim], inv[kMaxDim][kMaxDim];
+    for (int a = 0; a < d; ++a)
+      for (int b = 0; b < d; ++b)
+        E[a][b] = hm.coords[(size_t)v[b + 1] * d + a] - hm.coords[(size_t)v[0] * d + a];
+    // inverse of E (columns x_b - x_0); rows of inv are grad phi_1..phi_d
+    double det;
+    if (d == 2) {
+      det = E[0][0] * E[1][1] - E[0][1] * E[1][0];
+      inv[0][0] = E[1][1] / det; inv[0][1] = -E[0][1] / det;
+      inv[1][0] = -E[1][0] / det; inv[1][1] = E[0][0] / det;
+    } else {
+      det = E[0][0] * (E[1][1] * E[2][2] - E[1][2] * E[2][1]) -
+            E[0][1] * (E[1][0] * E[2][2] - E[1][2] * E[2][0]) +
+            E[0][2] * (E[1][0] * E[2][1] - E[1][1] * E[2][0]);
+      for (int a = 0; a < 3; ++a)
+        for (int b = 0; b < 3; ++b) {
+          const int a1 = (b + 1) % 3, a2 = (b + 2) % 3, b1 = (a + 1) % 3, b2 = (a + 2) % 3;
+          inv[a][b] = (E[a1][b1] * E[a2][b2] - E[a1][b2] * E[a2][b1]) / det;
+        }
+    }
+    if (!(det != 0.0) || !std::isfinite(det)) {
+      ++bad;
+      continue;
+    }
+    for (int k = 0; k < d; ++k) {
+      double g0 = 0.0;
+      for (int a = 1; a <= d; ++a) {
+        const double g = inv[a - 1][k];
+        grad[((size_t)e * k1 + a) * d + k] = (float)g;
+        g0 -= g;
+      }
+      grad[((size_t)e * k1) * d + k] = (float)g0;
+    }
+    float* c = cell.data() + (size_t)e * cw * 4;
+    for (int a = 0; a < k1; ++a) {
+      std::memcpy(c + a, v + a, sizeof(float));
+      for (int k = 0; k < d; ++k) c[k1 + a * d + k] = grad[((size_t)e * k1 + a) * d + k];
+    }
+  }
+  std::vector<int32_t> ptr(n + 1);
+  std::vector<int4> inc(hm.nc_cell.size());
+  if (hm.nc_cell.size() > 0x7fffffff) return MG_ERR_UNSUPPORTED;
+#pragma omp parallel for schedule(static) reduction(+ : bad)
+  for (int64_t i = 0; i < n; ++i) {
+    ptr[i] = (int32_t)hm.nc_ptr[i];
+    for (int64_t s = hm.nc_ptr[i]; s < hm.nc_ptr[i + 1]; ++s) {
+      const int32_t e = hm.nc_cell[s];
+      int a = 0;
+      while (a < k1 && hm.cells[(size_t)e * k1 + a] != i) ++a;
+      if (a == k1) {
+        ++bad;
+        continue;
+      }
+      float w[3] = {0.0f, 0.0f, 0.0f};
+      for (int k = 0; k < d; ++k)
+        w[k] = (float)(hm.cell_vol[e] * grad[((size_t)e * k1 + a) * d + k]);
+      int4 q = make_int4(e, 0, 0, 0);
+      std::memcpy(&q.y, w, 3 * sizeof(float));
+      inc[s] = q;
+    }
+  }
+  ptr[n] = (int32_t)hm.nc_ptr[n];
+  if (bad) return MG_ERR_ARG;
+  return mesh_set_flux_geometry(M, cell, ptr, inc, &out);
+}
+
 // whole_groups: pad the shots so that the float4s of a node (ld4) are a power
 // of two up to 32 or a multiple of 32.  The node adjoint sums them with warp
 // shuffles over such groups; any other count would put lanes of two nodes
@@ -586,65 +683,7 @@ int flux_setup(mg_mesh* M, const double* eps, const mg_shots* shots, const doubl
   F.host = host;
   F.st = st;
 
-  // per cell: gradients of the barycentric functions (FP64 -> FP32) and
-  // per node-cell incidence: |e| dphi_i/dx_k
-  std::vector<float> grad((size_t)m * k1 * d);
-  for (int64_t e = 0; e < m; ++e) {
-    const int32_t* v = hm->cells.data() + (size_t)e * k1;
-    double E[kMaxDim][kMaxDim], inv[kMaxDim][kMaxDim];
-    for (int a = 0; a < d; ++a)
-      for (int b = 0; b < d; ++b)
-        E[a][b] = hm->coords[(size_t)v[b + 1] * d + a] - hm->coords[(size_t)v[0] * d + a];
-    // inverse of E (columns x_b - x_0); rows of inv are grad phi_1..phi_d
-    double det;
-    if (d == 2) {
-      det = E[0][0] * E[1][1] - E[0][1] * E[1][0];
-      inv[0][0] = E[1][1] / det; inv[0][1] = -E[0][1] / det;
-      inv[1][0] = -E[1][0] / det; inv[1][1] = E[0][0] / det;
-    } else {
-      det = E[0][0] * (E[1][1] * E[2][2] - E[1][2] * E[2][1]) -
-            E[0][1] * (E[1][0] * E[2][2] - E[1][2] * E[2][0]) +
-            E[0][2] * (E[1][0] * E[2][1] - E[1][1] * E[2][0]);
-      for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) {
-          const int a1 = (b + 1) % 3, a2 = (b + 2) % 3, b1 = (a + 1) % 3, b2 = (a + 2) % 3;
-          inv[a][b] = (E[a1][b1] * E[a2][b2] - E[a1][b2] * E[a2][b1]) / det;
-        }
-    }
-    if (!(det != 0.0) || !std::isfinite(det)) return MG_ERR_ARG;
-    for (int k = 0; k < d; ++k) {
-      double g0 = 0.0;
-      for (int a = 1; a <= d; ++a) {
-        const double g = inv[a - 1][k];
-        grad[((size_t)e * k1 + a) * d + k] = (float)g;
-        g0 -= g;
-      }
-      grad[((size_t)e * k1) * d + k] = (float)g0;
-    }
-  }
-  std::vector<float> wnc(hm->nc_cell.size() * d);
-  for (int64_t i = 0; i < n; ++i)
-    for (int64_t s = hm->nc_ptr[i]; s < hm->nc_ptr[i + 1]; ++s) {
-      const int32_t e = hm->nc_cell[s];
-      int a = 0;
-      while (a < k1 && hm->cells[(size_t)e * k1 + a] != i) ++a;
-      if (a == k1) return MG_ERR_ARG;
-      for (int k = 0; k < d; ++k)
-        wnc[(size_t)s * d + k] = (float)(hm->cell_vol[e] * grad[((size_t)e * k1 + a) * d + k]);
-    }
-  // damping zeta per cell and direction (FP32), sources / receivers per row
-  std::vector<float> damp((size_t)m * d, 0.0f);
-  if (zeta) {
-    std::vector<double> zeta_h((size_t)m * d);
-    if (host) std::copy(zeta, zeta + (size_t)m * d, zeta_h.begin());
-    else if (cudaMemcpy(zeta_h.data(), zeta, zeta_h.size() * sizeof(double),
-                        cudaMemcpyDeviceToHost) != cudaSuccess)
-      return MG_ERR_CUDA;
-    for (size_t q = 0; q < zeta_h.size(); ++q) {
-      if (!(zeta_h[q] >= 0.0) || !std::isfinite(zeta_h[q])) return MG_ERR_ARG;
-      damp[q] = (float)zeta_h[q];
-    }
-  }
+  MG_FX(flux_geometry(M, *hm, F.geo));
   F.ld = S <= 4 ? 4 : ((S + 3) / 4) * 4;
   F.ld4 = F.ld / 4;
   if (whole_groups) {
@@ -692,24 +731,32 @@ int flux_setup(mg_mesh* M, const double* eps, const mg_shots* shots, const doubl
     if (xi) xi_d = X.put(xi, (size_t)m);
     if (!F.eps_d || (xi && !xi_d)) return MG_ERR_OOM;
   }
+  const double* zeta_d = zeta;
+  if (host && zeta) {
+    zeta_d = X.put(zeta, (size_t)m * d);
+    if (!zeta_d) return MG_ERR_OOM;
+  }
+  F.keep = X.get<float>((size_t)m * d);
+  int* bad = X.get<int>(1);
+  if (!F.keep || !bad) return MG_ERR_OOM;
+  if (cudaMemsetAsync(bad, 0, sizeof(int), st) != cudaSuccess) return MG_ERR_CUDA;
+  k_flux_keep<<<(unsigned)((m * d + 255) / 256), 256, 0, st>>>(m * d, zeta_d, (float)dt, F.keep,
+                                                               bad);
+  int bad_h = 0;
+  if (cudaMemcpyAsync(&bad_h, bad, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess)
+    return MG_ERR_CUDA;
+  if (bad_h) return MG_ERR_ARG;
   if (!(flags & MG_ALLOW_CFL)) {
     double dtc = 0.0;
     const int rc = mg_cfl_dt(M, F.eps_d, 0, st, &dtc);
     if (rc) return rc;
     if (dt > dtc * (1.0 + 1e-12)) return MG_ERR_CFL;
   }
-  F.cells = X.put(hm->cells);
-  F.grad = X.put(grad);
-  F.w = X.put(wnc);
-  F.damp = X.put(damp);
-  F.sp = X.put(sp);
-  F.ss = X.put(ss);
-  F.rp = X.put(rp);
-  F.rs = X.put(rs);
-  F.rt = X.put(rt);
+  F.ev = {X.put(sp), X.put(ss), X.put(rp), X.put(rs), X.put(rt)};
   F.fl = X.put(fl_h);
   F.coef = X.get<float2>(n);
-  if (!F.cells || !F.grad || !F.w || !F.damp || !F.sp || !F.ss || !F.rp || !F.rs || !F.rt ||
+  if (!F.ev.src_ptr || !F.ev.src_shot || !F.ev.rec_ptr || !F.ev.rec_shot || !F.ev.rec_trace ||
       !F.fl || !F.coef)
     return MG_ERR_OOM;
   F.c = F.V.coef_base;
@@ -727,11 +774,6 @@ struct DeviceScope {
   ~DeviceScope() { cudaSetDevice(prev); }
 };
 
-#define MG_FX(x)                  \
-  do {                            \
-    const int rc_ = (x);          \
-    if (rc_ != MG_OK) return rc_; \
-  } while (0)
 
 // Steps per CUDA-graph chunk for a call (0: plain launches): the handle's
 // chunk length, unless MG_NO_GRAPH.
@@ -752,7 +794,7 @@ extern "C" int mg_forward_pml(mg_mesh* M, const double* eps, const mg_shots* sho
   DeviceScope scope(mesh_device(M));
   if (!scope.ok) return MG_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  Scratch X(st);
+  Scratch X(M, st);
   Flux F;
   MG_FX(flux_setup(M, eps, shots, wavelet, dt, nt, xi, zeta, flags, st, X, F));
   const int64_t n = F.n, m = F.m, R = F.R;
@@ -802,7 +844,7 @@ extern "C" int mg_jacobian_apply_pml(mg_mesh* M, int level, const double* eps,
   DeviceScope scope(mesh_device(M));
   if (!scope.ok) return MG_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  Scratch X(st);
+  Scratch X(M, st);
   Flux F;
   MG_FX(flux_setup(M, eps, shots, wavelet, dt, nt, xi, zeta, flags, st, X, F));
   const int64_t n = F.n, m = F.m, R = F.R, nc = hm->n_cells_level[level];
@@ -831,20 +873,14 @@ extern "C" int mg_jacobian_apply_pml(mg_mesh* M, int level, const double* eps,
       cudaMemsetAsync(q, 0, qs * sizeof(float), st) ||
       cudaMemsetAsync(dq, 0, qs * sizeof(float), st))
     return MG_ERR_CUDA;
-  const int gp = grid_for(n * F.ld4);
+  const ItemGrid gp = item_grid(n, F.ld4);
   auto step = [&](StepRef sr, cudaStream_t s) {
     F.step_q(p, q, s);
     F.step_q(dp, dq, s);
-    if (F.d == 2)
-      launch_pdl(k_flux_p_tan<2>, gp, s, n, m, F.ld4, F.c.nc_ptr, F.c.nc_cell, F.w, F.coef,
-                 ratio, reinterpret_cast<const float4*>(q), reinterpret_cast<const float4*>(dq),
-                 reinterpret_cast<float4*>(p), reinterpret_cast<float4*>(dp), F.sp, F.ss, F.rp,
-                 F.rs, F.rt, F.fl, tr, nt, sr);
-    else
-      launch_pdl(k_flux_p_tan<3>, gp, s, n, m, F.ld4, F.c.nc_ptr, F.c.nc_cell, F.w, F.coef,
-                 ratio, reinterpret_cast<const float4*>(q), reinterpret_cast<const float4*>(dq),
-                 reinterpret_cast<float4*>(p), reinterpret_cast<float4*>(dp), F.sp, F.ss, F.rp,
-                 F.rs, F.rt, F.fl, tr, nt, sr);
+    launch_pdl(F.d == 2 ? k_flux_p_tan<2> : k_flux_p_tan<3>, gp, s, n, m, F.ld4, F.geo.inc_ptr,
+               F.geo.inc, F.coef, ratio, reinterpret_cast<const float4*>(q),
+               reinterpret_cast<const float4*>(dq), reinterpret_cast<float4*>(p),
+               reinterpret_cast<float4*>(dp), F.ev, F.fl, tr, nt, sr);
   };
   const int CL = chunk_len(M, flags);
   int l = 0;
@@ -880,7 +916,7 @@ extern "C" int mg_jacobian_T_apply_pml(mg_mesh* M, int level, const double* eps,
   DeviceScope scope(mesh_device(M));
   if (!scope.ok) return MG_ERR_CUDA;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  Scratch X(st);
+  Scratch X(M, st);
   Flux F;
   MG_FX(flux_setup(M, eps, shots, wavelet, dt, nt, xi, zeta, flags, st, X, F, true));
   const int64_t n = F.n, m = F.m, R = F.R, nc = hm->n_cells_level[level];
@@ -972,22 +1008,16 @@ extern "C" int mg_jacobian_T_apply_pml(mg_mesh* M, int level, const double* eps,
     launches += 2;
   }
   // reverse step l: p_l, p_{l+1} from their slots
-  const int gp = grid_for(n * F.ld4), gq = grid_for(m * F.ld4);
+  const ItemGrid gp = item_grid(n, F.ld4), gq = item_grid(m, F.ld4);
   const float fdt = (float)dt;
   auto rev = [&](StepRef sr, cudaStream_t s) {
-    if (F.d == 2) {
-      launch_pdl(k_flux_adj_p<2>, gp, s, n, m, F.ld4, F.c.nc_ptr, F.c.nc_cell, F.w, F.coef,
-                 reinterpret_cast<const float4*>(Qt), reinterpret_cast<float4*>(tp),
-                 reinterpret_cast<float4*>(rr), sl, hacc, F.rp, F.rs, F.rt, W, nt, sr, fdt);
-      launch_pdl(k_flux_adj_q<2>, gq, s, m, F.ld4, F.cells, F.grad, F.damp,
-                 reinterpret_cast<const float4*>(rr), reinterpret_cast<float4*>(Qt), fdt);
-    } else {
-      launch_pdl(k_flux_adj_p<3>, gp, s, n, m, F.ld4, F.c.nc_ptr, F.c.nc_cell, F.w, F.coef,
-                 reinterpret_cast<const float4*>(Qt), reinterpret_cast<float4*>(tp),
-                 reinterpret_cast<float4*>(rr), sl, hacc, F.rp, F.rs, F.rt, W, nt, sr, fdt);
-      launch_pdl(k_flux_adj_q<3>, gq, s, m, F.ld4, F.cells, F.grad, F.damp,
-                 reinterpret_cast<const float4*>(rr), reinterpret_cast<float4*>(Qt), fdt);
-    }
+    launch_pdl(F.d == 2 ? k_flux_adj_p<2> : k_flux_adj_p<3>, gp, s, n, m, F.ld4, F.geo.inc_ptr,
+               F.geo.inc, F.coef, reinterpret_cast<const float4*>(Qt),
+               reinterpret_cast<float4*>(tp), reinterpret_cast<float4*>(rr), sl, hacc, F.ev, W, nt,
+               sr, fdt);
+    launch_pdl(F.d == 2 ? k_flux_q<2, -1> : k_flux_q<3, -1>, gq, s, m, F.ld4, F.geo.cell, F.keep,
+               reinterpret_cast<const float4*>(rr), reinterpret_cast<float4*>(Qt), 1.0f,
+               StepRef{0, nullptr}, Slots{nullptr, 0, 1});
   };
   // segment [l0, l0 + len) with p_{l0} in slot 0 and q_{l0-1/2} in q: its
   // forward steps into slots 1..len (q in place), then the reverse steps
@@ -1050,7 +1080,7 @@ extern "C" int mg_jacobian_T_apply_pml(mg_mesh* M, int level, const double* eps,
   const unsigned gn = (unsigned)((n + 255) / 256), gm = (unsigned)((m + 255) / 256);
   k_flux_mass<<<gn, 256, 0, st>>>(F.c, F.eps_d, C);
   k_flux_hsum<<<gn, 256, 0, st>>>(n, nseg, hacc, C, gC);
-  k_flux_cell_grad<<<gm, 256, 0, st>>>(m, F.k1, F.cells, vol, gC, gf);
+  k_flux_cell_grad<<<gm, 256, 0, st>>>(m, F.k1, F.geo.cells, vol, gC, gf);
   if (cudaGetLastError() != cudaSuccess) return MG_ERR_CUDA;
   MG_FX(launch_restrict(nc, lp_d, li_d, gf, go, st));
   add_launches(M, launches + 5);
