@@ -174,7 +174,9 @@ struct mg_mesh {
   Buf tune_scratch;                       // autotuner inputs/outputs
   std::vector<mg::FluxBuffer> flux_scratch;   // work buffers of the flux path's calls
   std::mutex flux_mu;                     // guards them and the packed geometry
-  Buf flux_cell, flux_ptr, flux_inc;      // its packed geometry
+  Buf flux_cell, flux_ptr, flux_inc, flux_pinc;      // its packed geometry
+  std::array<Buf, 13> flux_tab;           // and patch tables
+  mg::DevFluxPatches flux_patches{};
 };
 
 namespace {
@@ -1155,7 +1157,7 @@ void mg_mesh_destroy(mg_mesh* M) {
   Buf* all[] = {&M->ell, &M->slice_off, &M->slice_w, &M->nc_ptr, &M->nc_cell, &M->nc_w,
                 &M->nf_ptr, &M->nf_cell, &M->nf_w, &M->is_bnd, &M->row_abs, &M->cells,
                 &M->vol, &M->cf_ptr, &M->cf_facet, &M->bnd, &M->bnd_meas, &M->ellu,
-                &M->ellc, &M->flux_cell, &M->flux_ptr, &M->flux_inc};
+                &M->ellc, &M->flux_cell, &M->flux_ptr, &M->flux_inc, &M->flux_pinc};
   for (Buf* b : all)
     if (b->p) cudaFree(b->p);
   for (auto* v : {&M->anc, &M->lvl_ptr, &M->lvl_idx})
@@ -1163,6 +1165,8 @@ void mg_mesh_destroy(mg_mesh* M) {
       if (b.p) cudaFree(b.p);
   for (auto& kv : M->auto_ellc)
     if (kv.second.p) cudaFree(kv.second.p);
+  for (Buf& b : M->flux_tab)
+    if (b.p) cudaFree(b.p);
   for (auto& kv : M->tiles) {
     mg_mesh::TileTables& D = kv.second;
     for (Buf* b : {&D.ell_off, &D.ell_idx, &D.ell_val, &D.sinfo, &D.halo_off, &D.halo_cnt, &D.halo})
@@ -2423,6 +2427,7 @@ bool mesh_keep_scratch(mg_mesh* M, std::vector<FluxBuffer>& bufs) {
   return true;
 }
 
+long long mesh_wait_budget(const mg_mesh* M) { return M->persist_budget; }
 std::mutex& mesh_flux_mutex(mg_mesh* M) { return M->flux_mu; }
 
 bool mesh_flux_geometry(mg_mesh* M, FluxGeometry* g) {
@@ -2431,12 +2436,46 @@ bool mesh_flux_geometry(mg_mesh* M, FluxGeometry* g) {
   g->inc_ptr = P<const int32_t>(M->flux_ptr);
   g->inc = P<const int4>(M->flux_inc);
   g->cells = P<const int32_t>(M->cells);
+  g->patches = M->flux_patches;
   return true;
 }
 
 int mesh_set_flux_geometry(mg_mesh* M, const std::vector<float>& cell,
                            const std::vector<int32_t>& ptr, const std::vector<int4>& inc,
-                           FluxGeometry* g) {
+                           const HostFluxPatches& H, FluxGeometry* g) {
+  if (H.B) {
+    DevFluxPatches D{};
+    int k = 0;
+    auto put = [&](const std::vector<int32_t>& v, const int32_t*& to) {
+      Buf& b = M->flux_tab[k++];
+      const int rc = upload(b, v);
+      to = P<const int32_t>(b);
+      return rc;
+    };
+    MG_TRY(put(H.own_off, D.own_off));
+    MG_TRY(put(H.border, D.border));
+    MG_TRY(put(H.halo_off, D.halo_off));
+    MG_TRY(put(H.x_off, D.x_off));
+    MG_TRY(put(H.cell_off, D.cell_off));
+    MG_TRY(put(H.inner, D.inner));
+    MG_TRY(put(H.inc_off, D.inc_off));
+    MG_TRY(put(H.row, D.row));
+    MG_TRY(put(H.row_inc, D.row_inc));
+    MG_TRY(put(H.halo, D.halo));
+    MG_TRY(put(H.halo_x, D.halo_x));
+    MG_TRY(put(H.cell, D.cell));
+    MG_TRY(put(H.cell_slot, D.cell_slot));
+    MG_TRY(upload(M->flux_pinc, H.inc));
+    D.inc = P<const int4>(M->flux_pinc);
+    D.n_x = H.x_off[H.B];
+    D.max_own = H.max_own;
+    D.max_halo = H.max_halo;
+    D.max_slots = H.max_slots;
+    D.max_cells = H.max_cells;
+    D.max_inc = H.max_inc;
+    D.B = H.B;
+    M->flux_patches = D;
+  }
   MG_TRY(upload(M->flux_cell, cell));
   MG_TRY(upload(M->flux_ptr, ptr));
   MG_TRY(upload(M->flux_inc, inc));   // last: its presence marks the set

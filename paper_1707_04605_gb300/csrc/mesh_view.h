@@ -8,6 +8,7 @@
 
 #include "../../include/mgwave.h"
 #include "kernels.cuh"
+#include "resident_flux.h"
 
 namespace mg {
 
@@ -56,12 +57,14 @@ struct FluxGeometry {
   const int32_t* inc_ptr = nullptr;  // [n + 1]
   const int4* inc = nullptr;         // per node and incident cell: {cell, weights}
   const int32_t* cells = nullptr;    // [m][d + 1] rows
+  DevFluxPatches patches{};          // B = 0: no resident kernel for this mesh
 };
 std::mutex& mesh_flux_mutex(mg_mesh* mesh);   // held around the next two
 bool mesh_flux_geometry(mg_mesh* mesh, FluxGeometry* out);   // false: not built yet
 int mesh_set_flux_geometry(mg_mesh* mesh, const std::vector<float>& cell,
                            const std::vector<int32_t>& inc_ptr, const std::vector<int4>& inc,
-                           FluxGeometry* out);
+                           const HostFluxPatches& patches, FluxGeometry* out);
+long long mesh_wait_budget(const mg_mesh* mesh);   // clock cycles of one device wait
 
 // One problem of a multi-instance batch, prepared on its own handle: device
 // inputs staged, coefficients and FP32 wavelet computed, event lists built,

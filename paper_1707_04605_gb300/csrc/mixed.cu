@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "../../include/mgwave.h"
+#include "flux_common.cuh"
 #include "kernels.cuh"
 #include "mesh_view.h"
 #include "mg_internal.h"
@@ -86,29 +87,6 @@ __global__ void k_flux_coefs(CoefArgs c, const double* __restrict__ xi, double d
   out[r] = make_float2((float)(dt / C), (float)RS);
 }
 
-__device__ __forceinline__ float4 fma4f(float a, float4 x, float4 y) {
-  return make_float4(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y), fmaf(a, x.z, y.z), fmaf(a, x.w, y.w));
-}
-__device__ __forceinline__ void add_source(const DevEvents& ev, int s0, int s1, int c4, float f,
-                                           float4& rhs) {
-  for (int s = s0; s < s1; ++s) {
-    const int d = __ldg(ev.src_shot + s) - 4 * c4;
-    if (d == 0) rhs.x += f;
-    if (d == 1) rhs.y += f;
-    if (d == 2) rhs.z += f;
-    if (d == 3) rhs.w += f;
-  }
-}
-__device__ __forceinline__ void record(const DevEvents& ev, int r0, int r1, int c4, float* traces,
-                                       int nt, int l, const float4& pv) {
-  for (int r = r0; r < r1; ++r) {
-    const int d = __ldg(ev.rec_shot + r) - 4 * c4;
-    if (d < 0 || d > 3) continue;
-    const float v = d == 0 ? pv.x : d == 1 ? pv.y : d == 2 ? pv.z : pv.w;
-    traces[(int64_t)__ldg(ev.rec_trace + r) * nt + l] = v;
-  }
-}
-
 // Damping factors 1 - dt zeta of the cells; *bad is set when a value is
 // negative or not finite.
 __global__ void k_flux_keep(int64_t count, const double* __restrict__ zeta, float dt,
@@ -120,13 +98,7 @@ __global__ void k_flux_keep(int64_t count, const double* __restrict__ zeta, floa
   keep[i] = 1.0f - dt * (float)z;
 }
 
-// Geometry packed so that a warp reads a cell's (an incidence's) constants with
-// a few 16-byte loads instead of one load per value, which took more of the
-// load pipe than the states: cell e, kCellW<D> float4: its D + 1 rows, then the
-// gradients [a][k]; incidence: {cell, |e| dphi_i/dx_k}.
-template <int D>
-constexpr int kCellW = ((D + 1) * (D + 1) + 3) / 4;
-
+// An incidence: {cell, |e| dphi_i/dx_k}, one 16-byte load.
 template <int D>
 struct Cell {
   int v[D + 1];
@@ -503,6 +475,40 @@ struct Flux {
   DevEvents ev{};
   float* fl = nullptr;      // f_l (FP32) per step, device
   float2* coef = nullptr;
+  ResidentShape shape;      // lpr = 0: launches per step
+  ResidentFluxArgs ra{};
+
+  // Steps [l, l + steps) with the resident kernel, from (p, q) (null: rest);
+  // the last states into (out_p, out_q), every new p into hist, `state` floats
+  // apart (each may be null).  MG_ERR_UNSUPPORTED before anything has run: the
+  // launches per step are the path then.
+  int advance(int l, int steps, const float* p, const float* q, float* out_p, float* out_q,
+              float* hist, float* traces) {
+    ResidentFluxArgs a = ra;
+    a.step0 = l;
+    a.steps = steps;
+    a.p = p;
+    a.q = q;
+    a.out_p = out_p;
+    a.out_q = out_q;
+    a.hist = hist;
+    a.traces = traces;
+    for (a.col0 = 0; a.col0 < ld; a.col0 += 4 * shape.lpr) {
+      const int rc = launch_resident_flux(a, d, shape, st);
+      if (rc == MG_ERR_UNSUPPORTED && l == 0 && a.col0 == 0) shape.lpr = 0;
+      if (rc != MG_OK) return rc;
+    }
+    return MG_OK;
+  }
+  // After the last launch: synchronises, and tells of a wait that ran out.
+  int finish() {
+    int word = 0;
+    if (ra.status && cudaMemcpyAsync(&word, ra.status, sizeof(int), cudaMemcpyDeviceToHost, st) !=
+                         cudaSuccess)
+      return MG_ERR_CUDA;
+    if (cudaStreamSynchronize(st) != cudaSuccess) return MG_ERR_CUDA;
+    return word ? MG_ERR_TIMEOUT : MG_OK;
+  }
 
   // flux update from p (or, with sl.seg, from the slot of step sr)
   void step_q(float* p, float* q, cudaStream_t s, StepRef sr = {0, nullptr},
@@ -646,7 +652,19 @@ int flux_geometry(mg_mesh* M, const HostMesh& hm, FluxGeometry& out) {
   }
   ptr[n] = (int32_t)hm.nc_ptr[n];
   if (bad) return MG_ERR_ARG;
-  return mesh_set_flux_geometry(M, cell, ptr, inc, &out);
+  // patches for the resident kernels, where one column of them can fit
+  int n_sm = 0, smem = 0;
+  if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, mesh_device(M)) ||
+      cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, mesh_device(M)))
+    return MG_ERR_CUDA;
+  const int B = (int)std::min<int64_t>(n_sm, std::max<int64_t>(1, n / 32));
+  HostFluxPatches H;
+  if ((n + (int64_t)m * d + m * (cw + 1) + (int64_t)inc.size()) * 16 / B < smem) {
+    const int rc = build_flux_patches(hm, B, inc, H);
+    if (rc == MG_ERR_UNSUPPORTED) H = HostFluxPatches();
+    else if (rc != MG_OK) return rc;
+  }
+  return mesh_set_flux_geometry(M, cell, ptr, inc, H, &out);
 }
 
 // whole_groups: pad the shots so that the float4s of a node (ld4) are a power
@@ -765,6 +783,41 @@ int flux_setup(mg_mesh* M, const double* eps, const mg_shots* shots, const doubl
   return cudaGetLastError() == cudaSuccess ? MG_OK : MG_ERR_CUDA;
 }
 
+// Chooses the path of a call's forward steps, `steps` of them at a time:
+// the resident kernel when its estimate is below that of two launches per step
+// (latency, then the gathers and states through L2).
+int flux_path(mg_mesh* M, int steps, Scratch& X, Flux& F) {
+  if (!F.geo.patches.B || steps < 16) return MG_OK;
+  int smem = 0;
+  if (cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, mesh_device(M)))
+    return MG_ERR_CUDA;
+  double us = 0.0;
+  resident_flux_shape(F.geo.patches, F.d, F.ld4, smem - 1024, F.shape, us);
+  // 16-byte accesses of a float4 column, at the measured rates: triangles 14 to
+  // 18 TB/s with states in L2 and 10 beyond it, tetrahedra 5 to 10
+  const double moved = ((double)F.m * (F.k1 * F.d + 3 * F.d + 1) + 2.0 * F.n) * F.ld4 * 16.0;
+  const double held = ((double)F.m * F.d + F.n) * F.ld4 * 16.0;
+  if (us > 5.0 + moved / (F.d == 2 && held < 100e6 ? 17e6 : 10e6)) F.shape.lpr = 0;
+  if (!F.shape.lpr) return MG_OK;
+  ResidentFluxArgs& a = F.ra;
+  a.P = F.geo.patches;
+  a.ev = F.ev;
+  a.coef = F.coef;
+  a.cell = F.geo.cell;
+  a.keep = F.keep;
+  a.fl = F.fl;
+  a.nt = F.nt;
+  a.ld = F.ld;
+  a.m = F.m;
+  a.dt = (float)F.dt;
+  a.state = F.n * F.ld;
+  a.budget = mesh_wait_budget(M);
+  a.xbuf = X.get<uint4>((size_t)2 * a.P.n_x * F.shape.lpr * 2);
+  a.status = X.get<int>(1);
+  if (!a.xbuf || !a.status) return MG_ERR_OOM;
+  return cudaMemsetAsync(a.status, 0, sizeof(int), F.st) == cudaSuccess ? MG_OK : MG_ERR_CUDA;
+}
+
 struct DeviceScope {
   int prev = 0;
   bool ok = false;
@@ -798,18 +851,30 @@ extern "C" int mg_forward_pml(mg_mesh* M, const double* eps, const mg_shots* sho
   Flux F;
   MG_FX(flux_setup(M, eps, shots, wavelet, dt, nt, xi, zeta, flags, st, X, F));
   const int64_t n = F.n, m = F.m, R = F.R;
-  float* p = X.get<float>((size_t)n * F.ld);
-  float* q = X.get<float>((size_t)F.d * m * F.ld);
   float* tr = F.host ? X.get<float>((size_t)R * nt) : traces;
-  int* base = X.get<int>(1);
-  if (!p || !q || !tr || !base) return MG_ERR_OOM;
-  if (cudaMemsetAsync(p, 0, (size_t)n * F.ld * sizeof(float), st) ||
-      cudaMemsetAsync(q, 0, (size_t)F.d * m * F.ld * sizeof(float), st))
-    return MG_ERR_CUDA;
+  if (!tr) return MG_ERR_OOM;
+  MG_FX(flux_path(M, nt, X, F));
+  int l = 0;   // steps done
+  if (F.shape.lpr) {
+    const int rc = F.advance(0, nt, nullptr, nullptr, nullptr, nullptr, nullptr, tr);
+    if (rc == MG_OK) l = nt;
+    else if (rc != MG_ERR_UNSUPPORTED) return rc;
+  }
+  float *p = nullptr, *q = nullptr;
+  int* base = nullptr;
+  if (l < nt) {
+    p = X.get<float>((size_t)n * F.ld);
+    q = X.get<float>((size_t)F.d * m * F.ld);
+    base = X.get<int>(1);
+    if (!p || !q || !base) return MG_ERR_OOM;
+    if (cudaMemsetAsync(p, 0, (size_t)n * F.ld * sizeof(float), st) ||
+        cudaMemsetAsync(q, 0, (size_t)F.d * m * F.ld * sizeof(float), st))
+      return MG_ERR_CUDA;
+  }
+  add_launches(M, 2 + (l ? (F.ld4 + F.shape.lpr - 1) / F.shape.lpr : 2 * (int64_t)nt));
   const int C = chunk_len(M, flags);
-  int l = 0;
   Chunk ch;
-  if (C && nt >= C) {   // whole chunks: one graph launch each
+  if (C && nt - l >= C) {   // whole chunks: one graph launch each
     MG_FX(launch_set_int(base, 0, st));
     MG_FX(ch.record([&](cudaStream_t cs) {
       for (int j = 0; j < C; ++j) {
@@ -825,11 +890,10 @@ extern "C" int mg_forward_pml(mg_mesh* M, const double* eps, const mg_shots* sho
     F.step_p(q, p, tr, {l, nullptr}, st);
   }
   if (cudaGetLastError() != cudaSuccess) return MG_ERR_CUDA;
-  add_launches(M, 1 + 2 * (int64_t)nt);
   if (F.host && cudaMemcpyAsync(traces, tr, (size_t)R * nt * sizeof(float),
                                 cudaMemcpyDeviceToHost, st) != cudaSuccess)
     return MG_ERR_CUDA;
-  return cudaStreamSynchronize(st) == cudaSuccess ? MG_OK : MG_ERR_CUDA;
+  return F.finish();
 }
 
 extern "C" int mg_jacobian_apply_pml(mg_mesh* M, int level, const double* eps,
@@ -964,6 +1028,23 @@ extern "C" int mg_jacobian_T_apply_pml(mg_mesh* M, int level, const double* eps,
   const Slots sl{reinterpret_cast<float4*>(seg), (int64_t)ns / 4, keep ? nt + 1 : K};
   // forward, keeping (p_l, q_{l-1/2}) at l = 0, K, 2K, ... (or every p_l)
   if (keep && cudaMemsetAsync(seg, 0, ns * sizeof(float), st)) return MG_ERR_CUDA;
+  // resident: the forward steps in intervals of K; the last one's only as the
+  // first segment's recompute
+  MG_FX(flux_path(M, K, X, F));
+  if (F.shape.lpr) {
+    int rc = MG_OK;
+    if (!keep && (cudaMemsetAsync(ck_p, 0, ns * sizeof(float), st) ||
+                  cudaMemsetAsync(ck_q, 0, qs * sizeof(float), st)))
+      return MG_ERR_CUDA;
+    for (int c = 0; c < (keep ? 1 : nck - 1) && rc == MG_OK; ++c) {
+      rc = keep ? F.advance(0, nt, nullptr, nullptr, nullptr, nullptr, seg + ns, nullptr)
+                : F.advance(c * K, K, c ? ck_p + ns * c : nullptr, c ? ck_q + qs * c : nullptr,
+                            ck_p + ns * (c + 1), ck_q + qs * (c + 1), nullptr, nullptr);
+      launches += (F.ld4 + std::max(F.shape.lpr, 1) - 1) / std::max(F.shape.lpr, 1);
+    }
+    if (rc != MG_OK && rc != MG_ERR_UNSUPPORTED) return rc;
+  }
+  const bool res = F.shape.lpr > 0;
   auto fwd_slots = [&](StepRef sr, cudaStream_t s) {   // p_l in its slot, p_{l+1} the next
     F.step_q(seg, q, s, sr, sl);
     F.step_p(q, seg, trd, sr, s, nullptr, sl);
@@ -978,9 +1059,9 @@ extern "C" int mg_jacobian_T_apply_pml(mg_mesh* M, int level, const double* eps,
   };
   // graph chunks: keep, CL steps; else one checkpoint interval of K steps
   const int LF = keep ? CL : (CL ? K : 0);
-  int l = 0;
+  int l = res ? nt : 0;
   Chunk chf;
-  if (LF >= 2 && nt >= LF) {
+  if (LF >= 2 && nt - l >= LF) {
     MG_FX(launch_set_int(base, 0, st));
     MG_FX(chf.record([&](cudaStream_t cs) {
       for (int j = 0; j < LF; ++j) fwd({j, base}, cs);
@@ -1023,7 +1104,7 @@ extern "C" int mg_jacobian_T_apply_pml(mg_mesh* M, int level, const double* eps,
   // forward steps into slots 1..len (q in place), then the reverse steps
   // l0 + len - 1 .. l0; s0 is step l0
   auto segment = [&](int len, StepRef s0, cudaStream_t s) {
-    for (int j = 0; j < len; ++j) fwd_slots({s0.l + j, s0.base}, s);
+    for (int j = 0; j < len && !res; ++j) fwd_slots({s0.l + j, s0.base}, s);
     for (int j = len - 1; j >= 0; --j) rev({s0.l + j, s0.base}, s);
   };
   Chunk chr;
@@ -1046,7 +1127,15 @@ extern "C" int mg_jacobian_T_apply_pml(mg_mesh* M, int level, const double* eps,
     }
   } else {
     const int nfull = nt / K;
-    auto load = [&](int c) {   // checkpoint c into slot 0 and q
+    auto load = [&](int c) {   // checkpoint c into slot 0 and q (resident: its segment)
+      const int len = std::min(K, nt - c * K);
+      if (res) {
+        launches += (F.ld4 + F.shape.lpr - 1) / F.shape.lpr - 2 * (int64_t)len;
+        return cudaMemcpyAsync(seg, ck_p + ns * c, ns * sizeof(float), cudaMemcpyDeviceToDevice,
+                               st) == cudaSuccess &&
+               F.advance(c * K, len, ck_p + ns * c, ck_q + qs * c, nullptr, nullptr, seg + ns,
+                         nullptr) == MG_OK;
+      }
       return cudaMemcpyAsync(seg, ck_p + ns * c, ns * sizeof(float), cudaMemcpyDeviceToDevice,
                              st) == cudaSuccess &&
              cudaMemcpyAsync(q, ck_q + qs * c, qs * sizeof(float), cudaMemcpyDeviceToDevice,
@@ -1087,5 +1176,5 @@ extern "C" int mg_jacobian_T_apply_pml(mg_mesh* M, int level, const double* eps,
   if (F.host && cudaMemcpyAsync(g, go, nc * sizeof(double), cudaMemcpyDeviceToHost, st) !=
                     cudaSuccess)
     return MG_ERR_CUDA;
-  return cudaStreamSynchronize(st) == cudaSuccess ? MG_OK : MG_ERR_CUDA;
+  return F.finish();
 }
