@@ -19,7 +19,7 @@ LIB = os.path.join(BUILD, "libmgwave.so")
 SOURCES = ["mesh_host.cpp", "kernels.cu", "kernels_rows.cu", "kernels_ring.cu", "kernels_tiled.cu",
            "kernels_bulk.cu", "kernels_tma.cu", "capi.cu", "resident_plan.cpp", "resident.cu",
            "resident_tangent.cu", "resident_adjoint.cu", "resident_flux_plan.cpp",
-           "resident_flux.cu",
+           "resident_flux.cu", "resident_flux_adjoint.cu",
            "static_scratch.cu", "batch.cu", "projected.cu",
            "inversion.cu", "approx.cu", "mixed.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

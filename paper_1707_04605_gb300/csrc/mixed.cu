@@ -477,6 +477,7 @@ struct Flux {
   float2* coef = nullptr;
   ResidentShape shape;      // lpr = 0: launches per step
   ResidentFluxArgs ra{};
+  ResidentShape rshape;     // reverse steps
 
   // Steps [l, l + steps) with the resident kernel, from (p, q) (null: rest);
   // the last states into (out_p, out_q), every new p into hist, `state` floats
@@ -786,7 +787,7 @@ int flux_setup(mg_mesh* M, const double* eps, const mg_shots* shots, const doubl
 // Chooses the path of a call's forward steps, `steps` of them at a time:
 // the resident kernel when its estimate is below that of two launches per step
 // (latency, then the gathers and states through L2).
-int flux_path(mg_mesh* M, int steps, Scratch& X, Flux& F) {
+int flux_path(mg_mesh* M, int steps, Scratch& X, Flux& F, bool reverse = false) {
   if (!F.geo.patches.B || steps < 16) return MG_OK;
   int smem = 0;
   if (cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, mesh_device(M)))
@@ -797,7 +798,12 @@ int flux_path(mg_mesh* M, int steps, Scratch& X, Flux& F) {
   // 18 TB/s with states in L2 and 10 beyond it, tetrahedra 5 to 10
   const double moved = ((double)F.m * (F.k1 * F.d + 3 * F.d + 1) + 2.0 * F.n) * F.ld4 * 16.0;
   const double held = ((double)F.m * F.d + F.n) * F.ld4 * 16.0;
-  if (us > 5.0 + moved / (F.d == 2 && held < 100e6 ? 17e6 : 10e6)) F.shape.lpr = 0;
+  const double rows = 5.0 + moved / (F.d == 2 && held < 100e6 ? 17e6 : 10e6);
+  if (us > rows) F.shape.lpr = 0;
+  if (reverse && F.shape.lpr) {   // after resident forward steps only
+    resident_flux_adj_shape(F.geo.patches, F.d, F.ld4, smem - 1024, F.rshape, us);
+    if (us > rows) F.rshape.lpr = 0;
+  }
   if (!F.shape.lpr) return MG_OK;
   ResidentFluxArgs& a = F.ra;
   a.P = F.geo.patches;
@@ -812,7 +818,7 @@ int flux_path(mg_mesh* M, int steps, Scratch& X, Flux& F) {
   a.dt = (float)F.dt;
   a.state = F.n * F.ld;
   a.budget = mesh_wait_budget(M);
-  a.xbuf = X.get<uint4>((size_t)2 * a.P.n_x * F.shape.lpr * 2);
+  a.xbuf = X.get<uint4>((size_t)2 * a.P.n_x * std::max(F.shape.lpr, F.rshape.lpr) * 2);
   a.status = X.get<int>(1);
   if (!a.xbuf || !a.status) return MG_ERR_OOM;
   return cudaMemsetAsync(a.status, 0, sizeof(int), F.st) == cudaSuccess ? MG_OK : MG_ERR_CUDA;
@@ -1030,7 +1036,7 @@ extern "C" int mg_jacobian_T_apply_pml(mg_mesh* M, int level, const double* eps,
   if (keep && cudaMemsetAsync(seg, 0, ns * sizeof(float), st)) return MG_ERR_CUDA;
   // resident: the forward steps in intervals of K; the last one's only as the
   // first segment's recompute
-  MG_FX(flux_path(M, K, X, F));
+  MG_FX(flux_path(M, K, X, F, true));
   if (F.shape.lpr) {
     int rc = MG_OK;
     if (!keep && (cudaMemsetAsync(ck_p, 0, ns * sizeof(float), st) ||
@@ -1107,10 +1113,47 @@ extern "C" int mg_jacobian_T_apply_pml(mg_mesh* M, int level, const double* eps,
     for (int j = 0; j < len && !res; ++j) fwd_slots({s0.l + j, s0.base}, s);
     for (int j = len - 1; j >= 0; --j) rev({s0.l + j, s0.base}, s);
   };
+  // reverse steps l0 + len - 1 .. l0 with the resident kernel, p_{l0} in slot 0
+  auto reverse = [&](int l0, int len) {
+    ResidentFluxAdjArgs a{};
+    a.P = F.geo.patches;
+    a.ev = F.ev;
+    a.coef = F.coef;
+    a.cell = F.geo.cell;
+    a.keep = F.keep;
+    a.w = W;
+    a.nt = nt;
+    a.k = l0 + len - 1;
+    a.steps = len;
+    a.ld = F.ld;
+    a.nseg = nseg;
+    a.m = m;
+    a.dt = fdt;
+    a.p = seg + ns * (len - 1);
+    a.state = (int64_t)ns;
+    a.tp = tp;
+    a.Qt = Qt;
+    a.hacc = hacc;
+    a.xbuf = F.ra.xbuf;
+    a.status = F.ra.status;
+    a.budget = F.ra.budget;
+    int rc = MG_OK;
+    for (; a.col0 < F.ld && rc == MG_OK; a.col0 += 4 * F.rshape.lpr) {
+      rc = launch_resident_flux_adj(a, F.d, F.rshape, st);
+      launches += 1;
+    }
+    if (rc == MG_ERR_UNSUPPORTED && l0 + len == nt) F.rshape.lpr = 0;   // nothing has run
+    return rc;
+  };
   Chunk chr;
   if (keep) {   // reverse steps nt-1 .. 0 in chunks of CL (base: the chunk's first step)
     int k = nt;   // steps below k remain
-    if (CL >= 2 && nt >= CL) {
+    if (res && F.rshape.lpr) {
+      const int rc = reverse(0, nt);
+      if (rc == MG_OK) k = 0;
+      else if (rc != MG_ERR_UNSUPPORTED) return rc;
+    }
+    if (CL >= 2 && k >= CL) {
       MG_FX(launch_set_int(base, nt - 1, st));
       MG_FX(chr.record([&](cudaStream_t cs) {
         for (int j = 0; j < CL; ++j) rev({-j, base}, cs);
@@ -1130,7 +1173,7 @@ extern "C" int mg_jacobian_T_apply_pml(mg_mesh* M, int level, const double* eps,
     auto load = [&](int c) {   // checkpoint c into slot 0 and q (resident: its segment)
       const int len = std::min(K, nt - c * K);
       if (res) {
-        launches += (F.ld4 + F.shape.lpr - 1) / F.shape.lpr - 2 * (int64_t)len;
+        launches += (F.ld4 + F.shape.lpr - 1) / F.shape.lpr;
         return cudaMemcpyAsync(seg, ck_p + ns * c, ns * sizeof(float), cudaMemcpyDeviceToDevice,
                                st) == cudaSuccess &&
                F.advance(c * K, len, ck_p + ns * c, ck_q + qs * c, nullptr, nullptr, seg + ns,
@@ -1141,12 +1184,20 @@ extern "C" int mg_jacobian_T_apply_pml(mg_mesh* M, int level, const double* eps,
              cudaMemcpyAsync(q, ck_q + qs * c, qs * sizeof(float), cudaMemcpyDeviceToDevice,
                              st) == cudaSuccess;
     };
-    if (nt % K) {   // the last, shorter segment: plain launches
+    int c0 = nck;   // segments below c0 remain
+    while (res && F.rshape.lpr && c0 > 0) {
+      const int c = c0 - 1, len = std::min(K, nt - c * K);
+      if (!load(c)) return MG_ERR_CUDA;
+      const int rc = reverse(c * K, len);
+      if (rc == MG_OK) c0 = c;
+      else if (rc != MG_ERR_UNSUPPORTED) return rc;
+    }
+    if (c0 > 0 && nt % K) {   // the last, shorter segment: plain launches
       if (!load(nfull)) return MG_ERR_CUDA;
       segment(nt - nfull * K, {nfull * K, nullptr}, st);
-      launches += 4 * (int64_t)(nt - nfull * K);
+      launches += (res ? 2 : 4) * (int64_t)(nt - nfull * K);
     }
-    if (CL && K >= 2 && nfull >= 1) {   // full segments: one graph launch each
+    if (CL && K >= 2 && nfull >= 1 && c0 > 0) {   // full segments: one graph launch each
       MG_FX(launch_set_int(base, (nfull - 1) * K, st));
       MG_FX(chr.record([&](cudaStream_t cs) {
         segment(K, {0, base}, cs);
@@ -1155,13 +1206,13 @@ extern "C" int mg_jacobian_T_apply_pml(mg_mesh* M, int level, const double* eps,
       for (int c = nfull - 1; c >= 0; --c) {
         if (!load(c)) return MG_ERR_CUDA;
         MG_FX(chr.launch(st));
-        launches += 4 * (int64_t)K;
+        launches += (res ? 2 : 4) * (int64_t)K;
       }
     } else {
-      for (int c = nfull - 1; c >= 0; --c) {
+      for (int c = std::min(c0, nfull) - 1; c >= 0; --c) {
         if (!load(c)) return MG_ERR_CUDA;
         segment(K, {c * K, nullptr}, st);
-        launches += 4 * (int64_t)K;
+        launches += (res ? 2 : 4) * (int64_t)K;
       }
     }
   }

@@ -62,12 +62,38 @@ struct ResidentFluxArgs {
   long long budget;
 };
 
+// Reverse steps k, k - 1, ... (`steps` of them) on the shot columns [col0, col0 +
+// 4 lpr), a whole group of the node adjoint's sum over the shots.
+struct ResidentFluxAdjArgs {
+  DevFluxPatches P;
+  DevEvents ev;
+  const float2* coef;
+  const float4* cell;
+  const float* keep;
+  const float* w;           // [n_traces][nt] trace weights
+  int32_t nt, k, steps, ld, col0, nseg;
+  int64_t m;
+  float dt;
+  const float* p;           // p_k; p_{k+1} state floats after it, p_{k-j} before it
+  int64_t state;
+  float *tp, *Qt;           // adjoint states, read (not at step nt - 1) and written
+  double* hacc;             // [n][nseg]
+  uint4* xbuf;
+  int* status;
+  long long budget;
+};
+
 // Lanes per row (4 columns each) whose patches fit smem_max bytes and whose
 // launches take the least time by the estimate; us: that of a step of ld4 float4
 // columns.  shape.lpr = 0: none fits.
 void resident_flux_shape(const DevFluxPatches& P, int d, int ld4, int smem_max,
                          ResidentShape& shape, double& us);
+// The same for reverse steps, whose lanes are given: min(32, ld4).
+void resident_flux_adj_shape(const DevFluxPatches& P, int d, int ld4, int smem_max,
+                             ResidentShape& shape, double& us);
 int launch_resident_flux(const ResidentFluxArgs& a, int d, const ResidentShape& s,
                          cudaStream_t st);
+int launch_resident_flux_adj(const ResidentFluxAdjArgs& a, int d, const ResidentShape& s,
+                             cudaStream_t st);
 
 }  // namespace mg

@@ -28,6 +28,7 @@ CASES = [
     (configs.asteroid_2d, dict(n_refine=1, S=1, nt=41)),      # one patch per 32 rows
     (configs.asteroid_2d, dict(n_refine=1, S=10, nt=17)),     # columns beyond the shots
     (configs.asteroid_2d, dict(n_refine=2, S=37, nt=40)),     # a ragged last column group
+    (configs.asteroid_2d, dict(n_refine=1, S=130, nt=20)),    # two groups of 32 lanes
     (configs.asteroid_2d, dict(n_refine=3, S=12, nt=24)),     # patches that fill an SM
     (configs.ellipsoid_3d, dict(n_refine=0, S=5, nt=33)),
     (configs.tiny_3d, dict(nt=20)),
