@@ -660,7 +660,7 @@ int flux_geometry(mg_mesh* M, const HostMesh& hm, FluxGeometry& out) {
     return MG_ERR_CUDA;
   const int B = (int)std::min<int64_t>(n_sm, std::max<int64_t>(1, n / 32));
   HostFluxPatches H;
-  if ((n + (int64_t)m * d + m * (cw + 1) + (int64_t)inc.size()) * 16 / B < smem) {
+  if (((n + m * d) * 16 + m * 36 + (int64_t)inc.size() * 12) / B < smem) {
     const int rc = build_flux_patches(hm, B, inc, H);
     if (rc == MG_ERR_UNSUPPORTED) H = HostFluxPatches();
     else if (rc != MG_OK) return rc;

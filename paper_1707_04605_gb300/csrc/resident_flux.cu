@@ -5,7 +5,7 @@
 // fluxes, a row reads D fluxes per incident cell (42 accesses of 16 bytes per
 // row and 4 columns in two dimensions), against two launches per step whose
 // gathers go through L2.  Us per step, launches -> resident (lanes per row that
-// fit): 62,641 nodes, 128 shots 91.6 -> 59.8 (2), 4 shots 9.8 -> 2.8 (1);
+// fit): 62,641 nodes, 128 shots 91.6 -> 44 (4; 60 with 2), 4 shots 9.8 -> 2.8 (1);
 // 15,769 nodes, 32 shots 8.1 -> 3.1 (8), 128 shots 17.1 -> 11.5 (16); 3,997
 // nodes, 10 shots 5.9 -> 2.1 (4), 256 shots 11.2 -> 10.4 (32); 4,199 nodes of
 // tetrahedra, 64 shots 29.8 -> 18.3 (4).
@@ -31,7 +31,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1) k_resident_flux(ResidentF
   const unsigned ps = smem_u32(sm), qs = ps + P.max_slots * SLOT;
   const unsigned qk = P.max_cells * SLOT;
   const FluxPatch t = fill_flux<D, LPR>(P, a.ev, a.cell, a.keep, a.coef,
-                                        sm + (size_t)(P.max_slots + D * P.max_cells) * SLOT);
+                                        sm + (size_t)(P.max_slots + D * P.max_cells) * SLOT, false);
   const int own = t.own;
   if (tid == 0) failed = 0;
   // a lane keeps its column: the strides over items are whole warps
@@ -47,8 +47,10 @@ __global__ void __launch_bounds__(kResidentThreads, 1) k_resident_flux(ResidentF
   __syncthreads();
 
   unsigned pl = ps + tid % LPR * 16, ql = qs + tid % LPR * 16, cell0 = smem_u32(t.cell),
-           inc0 = smem_u32(t.inc), row0 = smem_u32(t.row);
-  asm volatile("" : "+r"(pl), "+r"(ql), "+r"(cell0), "+r"(inc0), "+r"(row0));
+           inc0 = smem_u32(t.inc), row0 = smem_u32(t.row),
+           slots0 = smem_u32(t.slots), w10 = smem_u32(t.w1);
+  asm volatile("" : "+r"(pl), "+r"(ql), "+r"(cell0), "+r"(inc0), "+r"(row0),
+               "+r"(slots0), "+r"(w10));
   const int units = t.halo * 2 * LPR;
   const int copy = copy_threads(units);
   const size_t xhalf = (size_t)P.n_x * (2 * LPR);
@@ -59,11 +61,11 @@ __global__ void __launch_bounds__(kResidentThreads, 1) k_resident_flux(ResidentF
                            units, (unsigned)j, tid - (threads - copy), copy, a.status, a.budget))
         failed = 1;
     } else {
-      step_cells<D, LPR, 1>(cell0, pl, ql, qk, 0, t.inner, tid, wait ? threads - copy : threads, a.dt);
+      step_cells<D, LPR, 1>(cell0, slots0, P.max_cells, pl, ql, qk, 0, t.inner, tid, wait ? threads - copy : threads, a.dt);
     }
     __syncthreads();
     if (failed) return;
-    step_cells<D, LPR, 1>(cell0, pl, ql, qk, t.inner, t.cells, tid, threads, a.dt);
+    step_cells<D, LPR, 1>(cell0, slots0, P.max_cells, pl, ql, qk, t.inner, t.cells, tid, threads, a.dt);
     __syncthreads();
     const int l = a.step0 + j;
     uint4* const xo = a.xbuf + (size_t)((j & 1) ^ 1) * xhalf + (size_t)t.x0 * (2 * LPR);
@@ -73,7 +75,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1) k_resident_flux(ResidentF
       const unsigned at = pl + i / LPR * SLOT;
       float4 pv = lds4(at);
       const int inc = __float_as_int(rw.z), r = __float_as_int(rw.w);
-      const float4 bt = row_fluxes<D>(inc, inc0, ql, qk);
+      const float4 bt = row_fluxes<D>(inc, inc0, w10, ql, qk);
       float4 rhs = make_float4(-bt.x, -bt.y, -bt.z, -bt.w);
       const int rr = r & ~kEventBit;
       if (r < 0) {
@@ -124,13 +126,14 @@ namespace {
 // within 15% of them (barriers and exchange, halo, the states' and the
 // constants' accesses to shared memory).
 int64_t flux_smem(const DevFluxPatches& P, int d, int lpr, int more, int bytes) {
-  const int rec = d == 2 ? kRecW<2> : kRecW<3>;
+  if (d == 2 && P.max_slots > 1 << kSlotBits) return INT64_MAX;
+  const int64_t cell = d == 2 ? 16 * kRecW<2> + kCellMore<2> : 16 * kRecW<3>;
+  const int64_t inc = d == 2 ? kIncBytes<2> + kIncMore<2> : kIncBytes<3>;
   return (int64_t)(P.max_slots + more * P.max_own + d * P.max_cells) * 16 * lpr +
-         16 * ((int64_t)P.max_cells * rec + P.max_inc + P.max_own) + 4 * ((P.max_halo + 1) & ~1) +
-         bytes * P.max_own;
+         P.max_cells * cell + P.max_inc * inc + P.max_own * (16 + bytes) + 4 * P.max_halo;
 }
 double flux_us(const DevFluxPatches& P, int d, int lpr) {
-  const int rec = d == 2 ? kRecW<2> : kRecW<3>;
+  const int rec = d == 2 ? 3 : 5;
   const double states = P.max_cells * (3.0 * d + 1.0) + (double)P.max_inc * d + 2.0 * P.max_own;
   const double constants = (double)P.max_cells * rec + P.max_inc + P.max_own;
   return 1.2 + 4e-3 * P.max_halo + 0.775e-4 * lpr * states + 0.8e-4 * constants;

@@ -9,26 +9,55 @@
 namespace mg {
 namespace {
 
-// A cell in shared memory: slots (byte offsets), gradients, damping factors.
+// Constants in shared memory.  Three dimensions: a cell's slots (byte offsets),
+// gradients and damping factors in 5 float4, an incidence {offset of the cell,
+// weights}.  Two dimensions, smaller (36 bytes per cell and 12 per incidence
+// instead of 48 and 16: 62,641 nodes then fit 4 lanes per row, not 2): gradients
+// and factors in two planes of float4, the slots packed; {offset, weight}, and a
+// plane of the other weight.
+constexpr int kSlotBits = 10;
 template <int D>
-constexpr int kRecW = ((D + 1) * (D + 1) + D + 3) / 4;   // float4: 3, 5
+constexpr int kRecW = D == 2 ? 2 : 5;                 // float4 per cell
+template <int D>
+constexpr int kIncBytes = D == 2 ? 8 : 16;
+template <int D>
+constexpr int kCellMore = D == 2 ? 4 : 0;             // bytes in the other planes
+template <int D>
+constexpr int kIncMore = D == 2 ? 4 : 0;
 
 // Advances the patch's cells [c0, c1), thread t of `threads` taking every
 // threads-th float4: q <- keep q + dt sum g p, SIGN < 0: q <- keep q - sum g p.
 template <int D, int LPR, int SIGN>
-__device__ __forceinline__ void step_cells(unsigned cell0, unsigned p0, unsigned q0, unsigned qk,
+__device__ __forceinline__ void step_cells(unsigned cell0, unsigned slots, int max_cells,
+                                           unsigned p0, unsigned q0, unsigned qk,
                                            int c0, int c1, int t, int threads, float dt) {
 #pragma unroll 1
   for (int i = c0 * LPR + t; i < c1 * LPR; i += threads) {
     const int e = i / LPR;
-    float w[4 * kRecW<D>];
+    float w[4 * 5];   // slots, gradients, factors
+    if (D == 2) {
+      const float4 x = lds4(cell0 + e * 16), y = lds4(cell0 + (max_cells + e) * 16);
+      const int v = lds1(slots + e * 4);
 #pragma unroll
-    for (int j = 0; j < kRecW<D>; ++j) {
-      const float4 x = lds4(cell0 + e * (16 * kRecW<D>) + 16 * j);
-      w[4 * j] = x.x;
-      w[4 * j + 1] = x.y;
-      w[4 * j + 2] = x.z;
-      w[4 * j + 3] = x.w;
+      for (int a = 0; a <= D; ++a)
+        w[a] = __int_as_float((v >> (a * kSlotBits) & ((1 << kSlotBits) - 1)) * (16 * LPR));
+      w[3] = x.x;
+      w[4] = x.y;
+      w[5] = x.z;
+      w[6] = x.w;
+      w[7] = y.x;
+      w[8] = y.y;
+      w[9] = y.z;
+      w[10] = y.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < kRecW<D>; ++j) {
+        const float4 x = lds4(cell0 + e * (16 * kRecW<D>) + 16 * j);
+        w[4 * j] = x.x;
+        w[4 * j + 1] = x.y;
+        w[4 * j + 2] = x.z;
+        w[4 * j + 3] = x.w;
+      }
     }
     float4 pv[D + 1], o[D];
 #pragma unroll
@@ -57,15 +86,19 @@ __device__ __forceinline__ void step_cells(unsigned cell0, unsigned p0, unsigned
 struct FluxPatch {
   int r0, own, h0, halo, e0, cells, border, inner, x0;
   float4* cell;
-  int4 *inc, *row;
-  int* halo_x;
+  int4* row;
+  unsigned char* inc;
+  double* sums;         // per own row, when asked for
+  int *slots, *halo_x;
+  float* w1;
 };
 
 template <int D, int LPR>
 __device__ __forceinline__ FluxPatch fill_flux(const DevFluxPatches& P, const DevEvents& ev,
                                                const float4* __restrict__ geo,
                                                const float* __restrict__ keep,
-                                               const float2* __restrict__ coef, void* at) {
+                                               const float2* __restrict__ coef, void* at,
+                                               bool sums) {
   constexpr int SLOT = 16 * LPR;
   const int b = blockIdx.x, tid = threadIdx.x, threads = blockDim.x;
   FluxPatch t;
@@ -79,14 +112,17 @@ __device__ __forceinline__ FluxPatch fill_flux(const DevFluxPatches& P, const De
   t.inner = __ldg(P.inner + b);
   t.x0 = __ldg(P.x_off + b);
   t.cell = static_cast<float4*>(at);
-  t.inc = reinterpret_cast<int4*>(t.cell + P.max_cells * kRecW<D>);
-  t.row = t.inc + P.max_inc;
-  t.halo_x = reinterpret_cast<int*>(t.row + P.max_own);
+  t.row = reinterpret_cast<int4*>(t.cell + P.max_cells * kRecW<D>);
+  t.inc = reinterpret_cast<unsigned char*>(t.row + P.max_own);
+  t.sums = reinterpret_cast<double*>(t.inc + (size_t)P.max_inc * kIncBytes<D>);
+  t.slots = reinterpret_cast<int*>(t.sums + (sums ? P.max_own : 0));
+  t.w1 = reinterpret_cast<float*>(t.slots + P.max_cells * (kCellMore<D> / 4));
+  t.halo_x = reinterpret_cast<int*>(t.w1 + P.max_inc * (kIncMore<D> / 4));
   const int i0 = __ldg(P.inc_off + b), incs = __ldg(P.inc_off + b + 1) - i0;
   for (int i = tid; i < t.cells; i += threads) {
     int e = __ldg(P.cell + t.e0 + i);
     if (e < 0) e = ~e;
-    float w[4 * kRecW<D>] = {}, c[4 * kCellW<D>];
+    float w[4 * 5] = {}, c[4 * kCellW<D>];   // gradients and factors, the packed cell
     for (int j = 0; j < kCellW<D>; ++j) {
       const float4 x = __ldg(geo + (int64_t)e * kCellW<D> + j);
       c[4 * j] = x.x;
@@ -94,17 +130,29 @@ __device__ __forceinline__ FluxPatch fill_flux(const DevFluxPatches& P, const De
       c[4 * j + 2] = x.z;
       c[4 * j + 3] = x.w;
     }
-    for (int j = 0; j <= D; ++j)
-      w[j] = __int_as_float(__ldg(P.cell_slot + (size_t)(t.e0 + i) * 4 + j) * SLOT);
-    for (int j = D + 1; j < (D + 1) * (D + 1); ++j) w[j] = c[j];
-    for (int k = 0; k < D; ++k) w[(D + 1) * (D + 1) + k] = __ldg(keep + (int64_t)e * D + k);
+    constexpr int G = D == 2 ? 0 : D + 1;
+    int packed = 0;
+    for (int j = 0; j <= D; ++j) {
+      const int v = __ldg(P.cell_slot + (size_t)(t.e0 + i) * 4 + j);
+      if (D == 2) packed |= v << (j * kSlotBits);
+      else w[j] = __int_as_float(v * SLOT);
+    }
+    for (int j = 0; j < (D + 1) * D; ++j) w[G + j] = c[D + 1 + j];
+    for (int k = 0; k < D; ++k) w[G + (D + 1) * D + k] = __ldg(keep + (int64_t)e * D + k);
     for (int j = 0; j < kRecW<D>; ++j)
-      t.cell[i * kRecW<D> + j] = make_float4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+      t.cell[D == 2 ? j * P.max_cells + i : i * kRecW<D> + j] =
+          make_float4(w[4 * j], w[4 * j + 1], w[4 * j + 2], w[4 * j + 3]);
+    if (D == 2) t.slots[i] = packed;
   }
   for (int i = tid; i < incs; i += threads) {
     int4 q = __ldg(P.inc + i0 + i);
     q.x *= SLOT;
-    t.inc[i] = q;
+    if (D == 2) {
+      reinterpret_cast<int2*>(t.inc)[i] = make_int2(q.x, q.y);
+      t.w1[i] = __int_as_float(q.z);
+    } else {
+      reinterpret_cast<int4*>(t.inc)[i] = q;
+    }
   }
   for (int i = tid; i < t.own; i += threads) {
     int r = __ldg(P.row + t.r0 + i);
@@ -146,17 +194,26 @@ __device__ __forceinline__ void store_fluxes(const DevFluxPatches& P, const Flux
 
 // sum_k w[e,i,k] q^(k)_e over a row's incidences `inc`, in their order.
 template <int D>
-__device__ __forceinline__ float4 row_fluxes(int inc, unsigned inc0, unsigned ql, unsigned qk) {
+__device__ __forceinline__ float4 row_fluxes(int inc, unsigned inc0, unsigned w1, unsigned ql,
+                                             unsigned qk) {
   float4 bt = make_float4(0.f, 0.f, 0.f, 0.f);
-  unsigned s = inc0 + (inc & ((1 << kIncShift) - 1)) * 16;
-  const unsigned end = s + (inc >> kIncShift) * 16;
+  int s = inc & ((1 << kIncShift) - 1);
+  const int end = s + (inc >> kIncShift);
 #pragma unroll 2
-  for (; s < end; s += 16) {
-    const float4 w = lds4(s);
-    const unsigned q = ql + __float_as_uint(w.x);
+  for (; s < end; ++s) {
+    if (D == 2) {
+      const int2 w = lds2(inc0 + s * 8);
+      const float v = __int_as_float(lds1(w1 + s * 4));
+      const unsigned q = ql + w.x;
+      bt = fma4f(__int_as_float(w.y), lds4(q), bt);
+      bt = fma4f(v, lds4(q + qk), bt);
+    } else {
+      const float4 w = lds4(inc0 + s * 16);
+      const unsigned q = ql + __float_as_uint(w.x);
 #pragma unroll
-    for (int k = 0; k < D; ++k)
-      bt = fma4f(k == 0 ? w.y : k == 1 ? w.z : w.w, lds4(q + k * qk), bt);
+      for (int k = 0; k < D; ++k)
+        bt = fma4f(k == 0 ? w.y : k == 1 ? w.z : w.w, lds4(q + k * qk), bt);
+    }
   }
   return bt;
 }

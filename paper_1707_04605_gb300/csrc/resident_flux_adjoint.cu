@@ -30,8 +30,8 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
   const unsigned qk = P.max_cells * SLOT;
   const FluxPatch t =
       fill_flux<D, LPR>(P, a.ev, a.cell, a.keep, a.coef,
-                        sm + (size_t)(P.max_slots + P.max_own + D * P.max_cells) * SLOT);
-  double* const hs = reinterpret_cast<double*>(t.halo_x + ((P.max_halo + 1) & ~1));
+                        sm + (size_t)(P.max_slots + P.max_own + D * P.max_cells) * SLOT, true);
+  double* const hs = t.sums;
   const int own = t.own;
   const int ld4 = a.ld / 4, c4 = a.col0 / 4 + tid % LPR, seg = a.col0 / 128;
   const bool start = a.k == a.nt - 1;
@@ -47,8 +47,10 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
   __syncthreads();
 
   unsigned rl = rs + tid % LPR * 16, tl = ts + tid % LPR * 16, ql = qs + tid % LPR * 16,
-           cell0 = smem_u32(t.cell), inc0 = smem_u32(t.inc), row0 = smem_u32(t.row);
-  asm volatile("" : "+r"(rl), "+r"(tl), "+r"(ql), "+r"(cell0), "+r"(inc0), "+r"(row0));
+           cell0 = smem_u32(t.cell), inc0 = smem_u32(t.inc), row0 = smem_u32(t.row),
+           slots0 = smem_u32(t.slots), w10 = smem_u32(t.w1);
+  asm volatile("" : "+r"(rl), "+r"(tl), "+r"(ql), "+r"(cell0), "+r"(inc0), "+r"(row0),
+               "+r"(slots0), "+r"(w10));
   const int units = t.halo * 2 * LPR, copy = copy_threads(units);
   const size_t xhalf = (size_t)P.n_x * (2 * LPR);
   const unsigned gmask = LPR == 32 ? 0xffffffffu
@@ -70,7 +72,7 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
       const float4 x1 = i == tid ? n1 : __ldg(pk + st4 + at), x0 = i == tid ? n0 : __ldg(pk + at);
       float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
       if (!start || j > 0)
-        v = fma4f(a.dt, row_fluxes<D>(__float_as_int(rw.z), inc0, ql, qk),
+        v = fma4f(a.dt, row_fluxes<D>(__float_as_int(rw.z), inc0, w10, ql, qk),
                   lds4(tl + i / LPR * SLOT));
       if (r < 0)
         for (int q = __ldg(a.ev.rec_ptr + rr); q < __ldg(a.ev.rec_ptr + rr + 1); ++q) {
@@ -107,12 +109,12 @@ __global__ void __launch_bounds__(kResidentThreads, 1)
                            a.budget))
         failed = 1;
     } else {
-      step_cells<D, LPR, -1>(cell0, rl, ql, qk, 0, t.inner, tid,
+      step_cells<D, LPR, -1>(cell0, slots0, P.max_cells, rl, ql, qk, 0, t.inner, tid,
                              units > 0 ? threads - copy : threads, 1.0f);
     }
     __syncthreads();
     if (failed) return;
-    step_cells<D, LPR, -1>(cell0, rl, ql, qk, t.inner, t.cells, tid, threads, 1.0f);
+    step_cells<D, LPR, -1>(cell0, slots0, P.max_cells, rl, ql, qk, t.inner, t.cells, tid, threads, 1.0f);
     __syncthreads();
   }
   for (int i = tid; i < own * LPR; i += threads)
