@@ -168,7 +168,20 @@ int mg_cfl_dt(mg_mesh* mesh, const double* eps, int flags, void* stream,
  * All shots advance together in one node-major FP32 state (sources in the
  * fast dimension); MG_SINGLE_SOURCE runs them one at a time instead;
  * MG_PERSISTENT runs several steps per cooperative launch
- * (mg_mesh_set_persistent).  Flags: MG_HOST_PTRS, MG_NO_GRAPH,
+ * (mg_mesh_set_persistent).
+ * A handle whose forward launch shape has not been set (mg_mesh_set_tuning
+ * with a batch, tile or source width, mg_mesh_set_kernel_tuning, shot groups,
+ * register cap, ring, sweep, tiles or bulk copies) chooses by an estimate
+ * between the resident kernel (one cooperative launch for all steps between
+ * two checkpoints and for a group of shots, the states in shared memory, one
+ * patch of the mesh per SM) and one row-kernel launch per step; the same bits
+ * either way.  The tangent and the reverse steps choose likewise, each by its
+ * own kind's shape.  The patches' waits for one another are bounded by
+ * mg_mesh_set_persistent's wait_cycles: when one runs out the call's outputs
+ * are NaN and mg_mesh_device_status returns MG_ERR_TIMEOUT.  With fewer
+ * than 16 steps between checkpoints, and where no patch fits, the row kernels
+ * run.
+ * Flags: MG_HOST_PTRS, MG_NO_GRAPH,
  * MG_ALLOW_CFL, MG_SINGLE_SOURCE, MG_PERSISTENT, MG_KEEP_CHECKPOINTS,
  * MG_KEEP_STATES; any other bit is MG_ERR_UNSUPPORTED. */
 int mg_forward(mg_mesh* mesh, const double* eps, const mg_shots* shots,
@@ -309,9 +322,12 @@ int mg_mesh_set_kernel_tuning(mg_mesh* mesh, int kind, int batch, int tile_rows,
  * graphs.  Errors: MG_ERR_ARG for other values. */
 int mg_mesh_set_shot_groups(mg_mesh* mesh, int kind, int groups);
 
-/* Register cap of the forward row kernel: 0 (none, default) or 5 (at least
+/* Register cap of the forward row kernel: 0 (none) or 5 (at least
  * five resident 256-thread CTAs per SM; more warps in flight for
- * HBM-bound meshes, a few spilled registers).  Drops the cached graphs.
+ * HBM-bound meshes, a few spilled registers).  A handle whose launch shape
+ * has not been set runs its row kernels under the cap of 5 with two float4
+ * per lane (tangent: one) where the shot count allows it; setting either value
+ * counts as setting the shape.  Drops the cached graphs.
  * Errors: MG_ERR_ARG for other values. */
 int mg_mesh_set_min_blocks(mg_mesh* mesh, int min_blocks);
 
@@ -383,8 +399,9 @@ int mg_mesh_get_wide_lanes(const mg_mesh* mesh);
  * entries instead of one 32-entry column per lane.  Built on the device
  * from the handle's entries (host time and ceil(w_max / chunk) * 32 * chunk
  * * 8 bytes per slice of device memory); used by the wide-lane forward when
- * its launch shape has `chunk` lanes per row, ignored otherwise.  Same
- * results.  Drops the cached graphs.  Errors: MG_ERR_ARG for other values,
+ * its launch shape has `chunk` lanes per row, ignored otherwise.  A handle
+ * whose launch shape has not been set builds the copy for its own default
+ * shape on first use.  Same results.  Drops the cached graphs.  Errors: MG_ERR_ARG for other values,
  * MG_ERR_OOM, MG_ERR_CUDA. */
 int mg_mesh_set_chunked_ell(mg_mesh* mesh, int chunk);
 
@@ -447,7 +464,8 @@ int64_t mg_mesh_checkpoint_generation(const mg_mesh* mesh);
  * longer, or that sees another CTA give up, records the time-out in the
  * handle's status word and leaves; mg_forward then synchronises with the
  * stream, clears the word and returns MG_ERR_TIMEOUT (its traces are
- * incomplete).  `extra_arrivals` (0..2^20; 0 in normal use) makes every
+ * incomplete).  The same bound holds for the waits of the resident kernels
+ * (mg_forward, mg_forward_pml).  `extra_arrivals` (0..2^20; 0 in normal use) makes every
  * barrier wait for that many CTAs beyond the grid, which never arrive: it
  * exists to exercise the time-out path.  MG_PERSISTENT applies to
  * mg_forward only, without MG_SINGLE_SOURCE or MG_KEEP_STATES
@@ -500,7 +518,7 @@ int mg_mesh_set_dependent_launch(mg_mesh* mesh, int on);
 
 /* Status of the handle's bounded device waits since the last call:
  * MG_OK, MG_ERR_TIMEOUT (a wait ran out; the step it belongs to is
- * incomplete), MG_ERR_ARG (a copy address failed its alignment check).
+ * incomplete; the outputs of a resident launch are NaN), MG_ERR_ARG (a copy address failed its alignment check).
  * Synchronises with the device and clears the status. */
 int mg_mesh_device_status(mg_mesh* mesh);
 
@@ -523,7 +541,8 @@ int mg_mesh_get_tuning(const mg_mesh* mesh, int32_t* out);
  * mg_mesh_get_gather_ring); for the forward the row kernels with 1 vector
  * per lane, and with 2 and 4 under the register cap, sweeping 4 row blocks
  * per CTA (mg_mesh_get_row_sweep); then 2, 4 and 8 shot groups on the two
- * fastest of those.  The handle's L1 streaming, prefetch, wide-lane and
+ * fastest of those; and, where patches fit, the resident kernel of the kind
+ * (when it wins, chosen[] still holds the fastest of the others).  The handle's L1 streaming, prefetch, wide-lane and
  * stiffness-layout switches stay as they are.  Each
  * candidate is timed as the best of three runs after the GPU has been
  * warmed up; shapes within 1% of the fastest count as equal (the earliest
@@ -695,13 +714,19 @@ int mg_approx_jacobian(mg_mesh* mesh, int level, const double* eps, const mg_sho
  *   traces, shots, wavelet, dt, nt, flags (MG_HOST_PTRS, MG_ALLOW_CFL,
  *   MG_NO_GRAPH) as mg_forward; dt is checked against the CFL bound of
  *   mg_cfl_dt (the explicit damping terms need dt zeta and dt (sigma + xi)/eps
- *   below 1 in addition, which the caller chooses).  Synchronous; one launch
+ *   below 1 in addition, which the caller chooses).  Synchronous.  The mesh's
+ *   packed geometry is kept on the handle from the first call on, the work
+ *   buffers between calls (up to 2 GB; mg_mesh_trim frees them).  Calls of 16
+ *   steps and more run the resident kernel (as mg_forward's: pressures and
+ *   fluxes in shared memory, one launch for all steps of a group of shots)
+ *   where a patch of the mesh fits an SM and an estimate says it is faster; a
+ *   wait that runs out is MG_ERR_TIMEOUT.  Otherwise one launch
  *   per flux and per node update, whole chunks of the handle's graph chunk
  *   length replayed as one CUDA graph each (recorded once per call; step
  *   index read from a device counter the graph advances) unless
  *   MG_NO_GRAPH; the same results either way.
  * Errors: MG_ERR_ARG (null, negative zeta, degenerate cell), MG_ERR_CFL,
- * MG_ERR_UNSUPPORTED (other flags), MG_ERR_OOM, MG_ERR_CUDA. */
+ * MG_ERR_UNSUPPORTED (other flags), MG_ERR_OOM, MG_ERR_CUDA, MG_ERR_TIMEOUT. */
 int mg_forward_pml(mg_mesh* mesh, const double* eps, const mg_shots* shots, const double* wavelet,
                    double dt, int nt, const double* xi, const double* zeta, float* traces,
                    void* stream, int flags);
@@ -736,7 +761,10 @@ int mg_jacobian_apply_pml(mg_mesh* mesh, int level, const double* eps, const mg_
  *   ckpt_every  checkpoint spacing >= 1 (memory: ceil(nt / ckpt_every)
  *            copies of p and q, and ckpt_every + 1 copies of p).
  * Each segment's recomputed p states are written straight into their
- * slots of the segment buffer; a full segment (recompute and reverse
+ * slots of the segment buffer.  Forward and reverse steps run the resident
+ * kernels under mg_forward_pml's rule, applied to the checkpoint interval (the
+ * reverse steps where a patch holds 128 shots, or all when there are fewer);
+ * otherwise a full segment (recompute and reverse
  * steps) replays as one CUDA graph, as do chunks of the reverse steps when
  * one segment holds the whole run (unless MG_NO_GRAPH).
  * Other arguments and flags as mg_jacobian_apply_pml.  Synchronous. */
@@ -771,7 +799,9 @@ int mg_mesh_trim(mg_mesh* mesh);
  *  chunk      leapfrog steps captured per CUDA graph; an even number >= 2,
  *             or 0 for one plain launch per step.  Default 128.
  *  batch      untiled kernels: float4 vectors (4 shots each) carried per
- *             lane, 1, 2 or 4.  Default 1.  More vectors share each row's
+ *             lane, 1, 2 or 4.  Setting it, tile_rows or src_tile selects the
+ *             row or tiled kernels in this shape; unset (mg_forward) the
+ *             library chooses.  More vectors share each row's
  *             stiffness loads among more shots and keep more neighbour
  *             loads in flight per lane.
  *  tile_rows  rows per shared-memory tile (a multiple of 32, <= 8192), or 0

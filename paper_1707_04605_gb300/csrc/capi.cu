@@ -1567,8 +1567,12 @@ int mg_mesh_get_info(const mg_mesh* M, mg_mesh_info_t* info) {
                       &M->vol, &M->cf_ptr, &M->cf_facet, &M->bnd, &M->bnd_meas, &M->eps_h,
                       &M->wav_h, &M->wavf, &M->coef, &M->tcoef, &M->mass, &M->scal, &M->stA,
                       &M->stB, &M->stC, &M->stD, &M->out_h, &M->w_h, &M->v_h, &M->g_h, &M->ev,
-                      &M->G, &M->ckpt, &M->seg, &M->gfine, &M->step_base, &M->tr, &M->trf};
+                      &M->G, &M->ckpt, &M->seg, &M->gfine, &M->step_base, &M->tr, &M->trf,
+                      &M->xbuf, &M->flux_cell, &M->flux_ptr, &M->flux_inc, &M->flux_pinc};
   for (const Buf* b : all) bytes += (int64_t)b->bytes;
+  for (const auto& kv : M->auto_ellc) bytes += (int64_t)kv.second.bytes;
+  for (const Buf& b : M->flux_tab) bytes += (int64_t)b.bytes;
+  for (const mg::FluxBuffer& b : M->flux_scratch) bytes += (int64_t)b.bytes;
   info->device_bytes = bytes;
   return MG_OK;
 }
