@@ -6,12 +6,27 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <cstdlib>
+#include <new>
 #include <vector>
 
 #include "kernels.cuh"
 #include "mg_internal.h"
 
 namespace mg {
+
+// A thread's marks over all rows or cells while it works on one patch: zero
+// pages of which a patch touches few.
+struct Stamps {
+  int32_t* p;
+  explicit Stamps(int64_t n) : p(static_cast<int32_t*>(std::calloc(n, sizeof(int32_t)))) {
+    if (!p) throw std::bad_alloc();
+  }
+  ~Stamps() { std::free(p); }
+  Stamps(const Stamps&) = delete;
+  Stamps& operator=(const Stamps&) = delete;
+  int32_t& operator[](int64_t i) { return p[i]; }
+};
 
 // Rows cut into B patches: a patch's border rows (coupled to rows of other
 // patches) first, then its inner rows.

@@ -30,28 +30,26 @@ int build_flux_patches(const HostMesh& hm, int B, const std::vector<int4>& geo_i
     }
   }
   int bad = 0;
-#pragma omp parallel for schedule(dynamic, 4) reduction(+ : bad)
-  for (int b = 0; b < B; ++b) {
-    std::vector<int32_t>& c = cells[b];
-    for (int i = P.own_off[b]; i < P.own_off[b + 1]; ++i)
-      c.insert(c.end(), hm.nc_cell.begin() + hm.nc_ptr[P.row[i]],
-               hm.nc_cell.begin() + hm.nc_ptr[P.row[i] + 1]);
-    std::sort(c.begin(), c.end());
-    c.erase(std::unique(c.begin(), c.end()), c.end());
-    auto inner = [&](int32_t e) {
-      for (int a = 0; a < k1; ++a)
-        if (P.part[hm.cells[(size_t)e * k1 + a]] != b) return false;
-      return true;
-    };
-    F.inner[b] = (int)(std::stable_partition(c.begin(), c.end(), inner) - c.begin());
-    // the rows of a cell couple with one another: a foreign one is a halo row
-    for (size_t i = F.inner[b]; i < c.size(); ++i)
-      for (int a = 0; a < k1; ++a) {
-        const int32_t r = hm.cells[(size_t)c[i] * k1 + a];
-        if (P.part[r] != b && !std::binary_search(P.halo[b].begin(), P.halo[b].end(), r)) ++bad;
-      }
+#pragma omp parallel reduction(+ : bad)
+  {
+    Stamps seen(hm.m);
+#pragma omp for schedule(dynamic, 4)
+    for (int b = 0; b < B; ++b) {
+      std::vector<int32_t>& c = cells[b];
+      for (int i = P.own_off[b]; i < P.own_off[b + 1]; ++i)
+        for (int64_t q = hm.nc_ptr[P.row[i]]; q < hm.nc_ptr[P.row[i] + 1]; ++q) {
+          if (!seen[hm.nc_cell[q]]) c.push_back(hm.nc_cell[q]);
+          seen[hm.nc_cell[q]] = 1;
+        }
+      for (int32_t e : c) seen[e] = 0;
+      auto inner = [&](int32_t e) {
+        for (int a = 0; a < k1; ++a)
+          if (P.part[hm.cells[(size_t)e * k1 + a]] != b) return false;
+        return true;
+      };
+      F.inner[b] = (int)(std::stable_partition(c.begin(), c.end(), inner) - c.begin());
+    }
   }
-  if (bad) return MG_ERR_UNSUPPORTED;
   for (int b = 0; b < B; ++b) {
     int inc = 0;
     for (int i = P.own_off[b]; i < P.own_off[b + 1]; ++i)
@@ -72,37 +70,43 @@ int build_flux_patches(const HostMesh& hm, int B, const std::vector<int4>& geo_i
   F.cell.resize(F.cell_off[B]);
   F.cell_slot.assign((size_t)F.cell_off[B] * 4, 0);
   F.inc.resize(F.inc_off[B]);
-#pragma omp parallel for schedule(dynamic, 4) reduction(+ : bad)
-  for (int b = 0; b < B; ++b) {
-    const std::vector<int32_t>&c = cells[b], &h = P.halo[b];
-    const int own = P.own_off[b + 1] - P.own_off[b];
-    for (size_t i = 0; i < h.size(); ++i) {
-      F.halo[F.halo_off[b] + i] = h[i];
-      F.halo_x[F.halo_off[b] + i] = xrow[h[i]];
-    }
-    std::vector<std::pair<int32_t, int32_t>> at(c.size());   // cell, its place
-    for (size_t i = 0; i < c.size(); ++i) {
-      const int32_t* v = hm.cells.data() + (size_t)c[i] * k1;
-      at[i] = {c[i], (int32_t)i};
-      F.cell[F.cell_off[b] + i] = P.part[v[0]] == b ? c[i] : ~c[i];
-      for (int a = 0; a < k1; ++a)
-        F.cell_slot[(size_t)(F.cell_off[b] + i) * 4 + a] =
-            P.part[v[a]] == b
-                ? slot[v[a]]
-                : own + (int)(std::lower_bound(h.begin(), h.end(), v[a]) - h.begin());
-    }
-    std::sort(at.begin(), at.end());
-    int k = 0;
-    for (int i = P.own_off[b]; i < P.own_off[b + 1]; ++i) {
-      const int32_t r = P.row[i];
-      const int cnt = (int)(hm.nc_ptr[r + 1] - hm.nc_ptr[r]);
-      if (cnt >= 1 << (31 - kIncShift)) ++bad;
-      F.row_inc[i] = k | cnt << kIncShift;
-      for (int64_t s = hm.nc_ptr[r]; s < hm.nc_ptr[r + 1]; ++s) {
-        int4 q = geo_inc[s];
-        q.x = std::lower_bound(at.begin(), at.end(), std::make_pair(q.x, 0))->second;
-        F.inc[F.inc_off[b] + k++] = q;
+#pragma omp parallel reduction(+ : bad)
+  {
+    Stamps at(hm.m), halo(hm.n);   // place of a cell, slot of a halo row, plus 1
+#pragma omp for schedule(dynamic, 4)
+    for (int b = 0; b < B; ++b) {
+      const std::vector<int32_t>&c = cells[b], &h = P.halo[b];
+      const int own = P.own_off[b + 1] - P.own_off[b];
+      for (size_t i = 0; i < h.size(); ++i) {
+        F.halo[F.halo_off[b] + i] = h[i];
+        F.halo_x[F.halo_off[b] + i] = xrow[h[i]];
+        halo[h[i]] = own + (int32_t)i + 1;
       }
+      for (size_t i = 0; i < c.size(); ++i) {
+        const int32_t* v = hm.cells.data() + (size_t)c[i] * k1;
+        at[c[i]] = (int32_t)i + 1;
+        F.cell[F.cell_off[b] + i] = P.part[v[0]] == b ? c[i] : ~c[i];
+        for (int a = 0; a < k1; ++a) {
+          // the rows of a cell couple with one another: a foreign one is a halo row
+          const int32_t s = P.part[v[a]] == b ? slot[v[a]] : halo[v[a]] - 1;
+          if (s < 0) ++bad;
+          F.cell_slot[(size_t)(F.cell_off[b] + i) * 4 + a] = s;
+        }
+      }
+      int k = 0;
+      for (int i = P.own_off[b]; i < P.own_off[b + 1]; ++i) {
+        const int32_t r = P.row[i];
+        const int cnt = (int)(hm.nc_ptr[r + 1] - hm.nc_ptr[r]);
+        if (cnt >= 1 << (31 - kIncShift)) ++bad;
+        F.row_inc[i] = k | cnt << kIncShift;
+        for (int64_t s = hm.nc_ptr[r]; s < hm.nc_ptr[r + 1]; ++s) {
+          int4 q = geo_inc[s];
+          q.x = at[q.x] - 1;
+          F.inc[F.inc_off[b] + k++] = q;
+        }
+      }
+      for (int32_t r : h) halo[r] = 0;
+      for (int32_t e : c) at[e] = 0;
     }
   }
   return bad ? MG_ERR_UNSUPPORTED : MG_OK;

@@ -80,18 +80,24 @@ int build_patches(const HostMesh& hm, int B, HostPatches& P) {
   std::vector<uint8_t> border(n, 0);
   P.halo.resize(B);
   std::vector<std::vector<int32_t>> reads(B);   // patches that a patch reads
-#pragma omp parallel for schedule(dynamic, 4)
-  for (int b = 0; b < B; ++b) {
-    for (int i = P.own_off[b]; i < P.own_off[b + 1]; ++i)
-      for (int64_t q = hm.rowptr[P.row[i]]; q < hm.rowptr[P.row[i] + 1]; ++q)
-        if (part[hm.col[q]] != b) {
+#pragma omp parallel
+  {
+    Stamps row(n), other(B);   // halo rows and patches seen
+#pragma omp for schedule(dynamic, 4)
+    for (int b = 0; b < B; ++b) {
+      for (int i = P.own_off[b]; i < P.own_off[b + 1]; ++i)
+        for (int64_t q = hm.rowptr[P.row[i]]; q < hm.rowptr[P.row[i] + 1]; ++q) {
+          const int32_t c = hm.col[q], o = part[c];
+          if (o == b) continue;
           border[P.row[i]] = 1;
-          P.halo[b].push_back(hm.col[q]);
-          reads[b].push_back(part[hm.col[q]]);
+          if (!row[c]) P.halo[b].push_back(c);
+          if (!other[o]) reads[b].push_back(o);
+          row[c] = other[o] = 1;
         }
-    for (auto* v : {&P.halo[b], &reads[b]}) {
-      std::sort(v->begin(), v->end());
-      v->erase(std::unique(v->begin(), v->end()), v->end());
+      for (int32_t c : P.halo[b]) row[c] = 0;
+      for (int32_t o : reads[b]) other[o] = 0;
+      std::sort(P.halo[b].begin(), P.halo[b].end());
+      std::sort(reads[b].begin(), reads[b].end());
     }
   }
   for (int b = 0; b < B; ++b) {
