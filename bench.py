@@ -576,7 +576,8 @@ def pml_leg(mg, torch, mesh, w, eps_d, wav_d, dt, nt=1000, ckpt=1000):
             "forward_GB_per_s": bytes_fwd / (us["forward"] * 1e-6) / 1e9,
             "adjoint_vs_forward": secs["adjoint"] / secs["forward"],
             "graphs": mesh.tuning()["chunk"] >= 2,
-            "note": f"two launches per step (flux and node updates), whole chunks of "
+            "note": f"forward: the resident flux kernel where patches fit; tangent and reverse: "
+                    f"launches per step (flux and node updates), whole chunks of "
                     f"{mesh.tuning()['chunk']} steps replayed as CUDA graphs; the adjoint "
                     f"includes its forward, which keeps every state (checkpoint spacing {ckpt} "
                     f">= {nt} steps: one segment, no recompute)"}

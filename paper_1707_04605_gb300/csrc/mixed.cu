@@ -144,10 +144,12 @@ __device__ __forceinline__ Item item_of(int64_t count, int ld4) {
 // adjoint's Qt^(k) <- keep_k Qt^(k) - sum_a grad[a][k] r[v_a].
 //
 // Bound by the states' traffic through L2: a step gathers and writes 900 MB at
-// 62,641 nodes, 124,416 cells and 128 shots in its two kernels, 98 us (with one
-// load per constant and 64-bit divisions 103).
-// Advancing 32 shots at a time, with states that fit L2, takes 88 us there, 16
-// shots at a time 142.
+// 62,641 nodes, 124,416 cells and 128 shots in its two kernels.  Against one
+// load per constant and 64-bit divisions, us per step: tangent 183 -> 169,
+// reverse 133 -> 131; tetrahedra (30,525 nodes, 32 shots) forward 51 -> 44,
+// tangent 132 -> 116, with reverse 117 -> 102; 249,697 nodes, 64 shots forward
+// 186 -> 184, tangent 375 -> 342.  Advancing 32 shots at a time gains 10% on the
+// forward, 16 at a time loses 40%: left out.
 template <int D, int SIGN>
 __global__ void __launch_bounds__(256) k_flux_q(int64_t m, int ld4,
                                                 const float4* __restrict__ cell,
@@ -183,9 +185,12 @@ __global__ void __launch_bounds__(256) k_flux_q(int64_t m, int ld4,
 }
 
 // bt_n += sum_{e ni i} sum_k w[e,i,k] q_n^(k)_e for NQ flux fields, in the order
-// of the incidences.  One incidence at a time: with two, three or four of them
-// in flight the registers cost more warps than the loads gain (62,641 nodes,
-// 128 shots, forward step 98, 112, 114, 128 us).
+// of the incidences.  One incidence at a time, and the row's own values are
+// loaded after it: what is in flight across the loop costs more warps than it
+// gains (62,641 nodes, 128 shots, 256 forward steps with one, two, three and
+// four incidences in flight 25.0, 28.6, 29.1, 32.8 ms; with the row's values
+// loaded ahead the tangent 200 us per step instead of 169, tetrahedra forward 59
+// instead of 44).
 template <int D, int NQ>
 __device__ __forceinline__ void gather_flux(int s0, int s1, const int4* __restrict__ inc,
                                             int64_t m, int ld4, int c4,
@@ -222,13 +227,13 @@ __global__ void __launch_bounds__(256) k_flux_p(
   if (!it.ok) return;
   const int64_t i = it.i, t = i * ld4 + it.c4;
   const int c4 = it.c4;
+  float4 bt[1] = {make_float4(0.f, 0.f, 0.f, 0.f)};
+  const float4* const qs[1] = {q};
+  gather_flux<D, 1>(__ldg(inc_ptr + i), __ldg(inc_ptr + i + 1), inc, m, ld4, c4, qs, bt);
   float4 pv = p[t];
   const float2 c = __ldg(coef + i);
   const int s0 = __ldg(ev.src_ptr + i), s1 = __ldg(ev.src_ptr + i + 1);
   const int r0 = __ldg(ev.rec_ptr + i), r1 = __ldg(ev.rec_ptr + i + 1);
-  float4 bt[1] = {make_float4(0.f, 0.f, 0.f, 0.f)};
-  const float4* const qs[1] = {q};
-  gather_flux<D, 1>(__ldg(inc_ptr + i), __ldg(inc_ptr + i + 1), inc, m, ld4, c4, qs, bt);
   float4 rhs = make_float4(-bt[0].x, -bt[0].y, -bt[0].z, -bt[0].w);
   if (s0 != s1) add_source(ev, s0, s1, c4, __ldg(fl + l), rhs);
   pv.x = fmaf(c.x, fmaf(-c.y, pv.x, rhs.x), pv.x);
@@ -269,14 +274,14 @@ __global__ void __launch_bounds__(256) k_flux_p_tan(
   if (!it.ok) return;
   const int64_t i = it.i, t = i * ld4 + it.c4;
   const int c4 = it.c4;
+  float4 b2[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
+  const float4* const qs[2] = {q, dq};
+  gather_flux<D, 2>(__ldg(inc_ptr + i), __ldg(inc_ptr + i + 1), inc, m, ld4, c4, qs, b2);
   float4 pv = p[t], dv = dp[t];
   const float2 c = __ldg(coef + i);
   const float rt = __ldg(ratio + i);
   const int s0 = __ldg(ev.src_ptr + i), s1 = __ldg(ev.src_ptr + i + 1);
   const int r0 = __ldg(ev.rec_ptr + i), r1 = __ldg(ev.rec_ptr + i + 1);
-  float4 b2[2] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-  const float4* const qs[2] = {q, dq};
-  gather_flux<D, 2>(__ldg(inc_ptr + i), __ldg(inc_ptr + i + 1), inc, m, ld4, c4, qs, b2);
   const float4 dbt = b2[1];
   float4 rhs = make_float4(-b2[0].x, -b2[0].y, -b2[0].z, -b2[0].w);
   if (s0 != s1) add_source(ev, s0, s1, c4, __ldg(fl + l), rhs);
@@ -321,17 +326,14 @@ __global__ void __launch_bounds__(256) k_flux_adj_p(
   if (!it.ok) return;
   const int64_t i = it.i, t = i * ld4 + it.c4;
   const int c4 = it.c4;
-  const float4 x1 = __ldg(p1 + t), x0 = __ldg(p0 + t);
-  const float2 c = __ldg(coef + i);
-  const int r0 = __ldg(ev.rec_ptr + i), r1 = __ldg(ev.rec_ptr + i + 1);
   float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
   if (!first) {
-    const float4 tv = tp[t];
     float4 bt[1] = {a};
     const float4* const qs[1] = {Qt};
     gather_flux<D, 1>(__ldg(inc_ptr + i), __ldg(inc_ptr + i + 1), inc, m, ld4, c4, qs, bt);
-    a = fma4f(dt, bt[0], tv);
+    a = fma4f(dt, bt[0], tp[t]);
   }
+  const int r0 = __ldg(ev.rec_ptr + i), r1 = __ldg(ev.rec_ptr + i + 1);
   for (int r = r0; r < r1; ++r) {
     const int d = __ldg(ev.rec_shot + r) - 4 * c4;
     if (d < 0 || d > 3) continue;
@@ -341,6 +343,7 @@ __global__ void __launch_bounds__(256) k_flux_adj_p(
     if (d == 2) a.z += v;
     if (d == 3) a.w += v;
   }
+  const float4 x1 = __ldg(p1 + t), x0 = __ldg(p0 + t);
   float h = a.x * (x1.x - x0.x);
   h = fmaf(a.y, x1.y - x0.y, h);
   h = fmaf(a.z, x1.z - x0.z, h);
@@ -355,6 +358,7 @@ __global__ void __launch_bounds__(256) k_flux_adj_p(
     const int nseg = ld4 < 32 ? 1 : ld4 / 32;
     hacc[i * nseg + c4 / 32] += (double)h;
   }
+  const float2 c = __ldg(coef + i);
   const float4 r = make_float4(a.x * c.x, a.y * c.x, a.z * c.x, a.w * c.x);
   rr[t] = r;
   tp[t] = make_float4(fmaf(-c.y, r.x, a.x), fmaf(-c.y, r.y, a.y), fmaf(-c.y, r.z, a.z),
