@@ -96,7 +96,7 @@ def parse():
 
 def apply_tuning(mesh, spec):
     """Applies a tuning dict {kind: {batch, tile_rows, src_tile, groups,
-    ring, min_blocks, sweep}} (the shape of Mesh.tuning()) to a handle."""
+    ring, min_blocks, sweep, path}} (the shape of Mesh.tuning()) to a handle."""
     for kind, t in spec.items():
         if kind not in ("forward", "tangent", "adjoint"):
             continue
@@ -111,6 +111,7 @@ def apply_tuning(mesh, spec):
             mesh.set_wide_lanes(t.get("wide", 1))
             mesh.set_row_sweep(t.get("sweep", 0))
             mesh.set_tma_tiles(t.get("tma", 0))
+        mesh.set_kernel_path(t.get("path", "shape"), kind)
 
 
 def dist_env():
@@ -651,6 +652,7 @@ def tune_kept(mg, torch, mesh, w, eps_d, wav_d, dt, v_d, level, nt_probe=1024):
     chosen = {}
     for kind, fn in calls.items():
         best = None
+        mesh.set_kernel_path("shape", kind)
         for cap in {"tangent": (0, 5), "adjoint": (0, 5, 6)}[kind]:
             mesh.set_min_blocks(cap, kind)
             for g in (1, 2, 4):
@@ -897,6 +899,7 @@ def main():
         kept_groups = dict(zip(("forward", "adjoint", "tangent"),
                                (int(x) for x in args.kept_groups.split(","))))
         for kind, g in kept_groups.items():
+            mesh.set_kernel_path("shape", kind)
             mesh.set_shot_groups(g, kind)
     elif keep_states and not args.no_autotune:
         kept_groups = tune_kept(mg, torch, mesh, w, eps_d, wav_d, dt, v_d, LEVEL)
@@ -1055,14 +1058,15 @@ def main():
     # the same step with C3's memory bound: checkpoints every 256 steps
     c3 = None
     if keep_states and not args.no_c3_leg:
-        for kind in ("forward", "tangent", "adjoint"):   # the autotuned groups
-            mesh.set_shot_groups(tuning[kind].get("groups", 1), kind)
+        apply_tuning(mesh, tuning)   # as autotuned
         tc, _, _ = timed_steps(step_ckpt, max(1, min(args.steps, 2)))
         tcs = total_seconds(tc)
         ph = {"forward": statistics.mean(e[0].elapsed_time(e[1]) for e in tc),
               "adjoint": statistics.mean(e[1].elapsed_time(e[2]) for e in tc),
               "tangent": statistics.mean(e[2].elapsed_time(e[3]) for e in tc)}
-        tname = "k_tangent_tiled" if tuning["tangent"]["tile_rows"] else "k_tangent_rows"
+        resident = tuning["tangent"].get("path") in ("auto", "resident")
+        tname = ("k_resident_step" if resident else
+                 "k_tangent_tiled" if tuning["tangent"]["tile_rows"] else "k_tangent_rows")
         c3 = {"value": units_per_step * len(tc) * ws / tcs, "unit": UNIT,
               "ms_per_step": 1e3 * tcs / len(tc), "phases_ms": ph,
               "workload": describe(w, "checkpoints"), "tuning": tuning,
@@ -1071,6 +1075,7 @@ def main():
               "roofline": roofline(
                   f"{tname} (lockstep forward + tangent step, J v)", b_tan,
                   ph["tangent"] / 1e3 / nt,
+                  None if resident else
                   traffic_for("asteroid_2d tangent", tuning["tangent"], uniform), peak,
                   peak_kind, l2_note, "per-step time = J v phase / nt (launch gaps included)",
                   bound=L2_BOUND)}

@@ -169,9 +169,8 @@ int mg_cfl_dt(mg_mesh* mesh, const double* eps, int flags, void* stream,
  * fast dimension); MG_SINGLE_SOURCE runs them one at a time instead;
  * MG_PERSISTENT runs several steps per cooperative launch
  * (mg_mesh_set_persistent).
- * A handle whose forward launch shape has not been set (mg_mesh_set_tuning
- * with a batch, tile or source width, mg_mesh_set_kernel_tuning, shot groups,
- * register cap, ring, sweep, tiles or bulk copies) chooses by an estimate
+ * A handle whose forward launch shape has not been set
+ * (mg_mesh_set_kernel_path says what sets it) chooses by an estimate
  * between the resident kernel (one cooperative launch for all steps between
  * two checkpoints and for a group of shots, the states in shared memory, one
  * patch of the mesh per SM) and one row-kernel launch per step; the same bits
@@ -310,6 +309,27 @@ int mg_jacobian_T_apply_batch(int n_inst, mg_mesh* const* meshes, const int* lev
 #define MG_KERNEL_ADJOINT 2
 int mg_mesh_set_kernel_tuning(mg_mesh* mesh, int kind, int batch, int tile_rows, int src_tile);
 
+/* Which kernels a kind runs (kind -1: all three):
+ *  MG_PATH_AUTO      the resident kernel or the row kernels in the library's
+ *                    own launch shape, by an estimate of both (default)
+ *  MG_PATH_SHAPE     the launch shape on the handle
+ *  MG_PATH_RESIDENT  the resident kernel wherever it can run (mg_forward),
+ *                    the launch shape on the handle elsewhere
+ *  MG_PATH_ROWS      the row kernels in the library's own launch shape
+ * Setting a launch shape selects MG_PATH_SHAPE: a batch, tile or source width
+ * always, a number of shot groups, a register cap, ring, sweep, tiles or bulk
+ * copies when the value differs from the one on the handle.  The shape stays on
+ * the handle under every path, so a tuning that was read with its path can be
+ * set again: the shape first, then the path.  Same results on every path.
+ * Drops the cached graphs.  Errors: MG_ERR_ARG for other values. */
+#define MG_PATH_AUTO     0
+#define MG_PATH_SHAPE    1
+#define MG_PATH_RESIDENT 2
+#define MG_PATH_ROWS     3
+int mg_mesh_set_kernel_path(mg_mesh* mesh, int kind, int path);
+/* The paths of the forward, tangent and adjoint kinds into out[3]. */
+int mg_mesh_get_kernel_path(const mg_mesh* mesh, int32_t* out);
+
 /* Shot groups of a kernel kind (kind = -1: all kinds): the padded shot
  * columns are split into `groups` equal groups (1, 2, 4 or 8) and, inside
  * each CUDA-graph chunk of steps (forward, tangent) and each checkpoint
@@ -326,8 +346,8 @@ int mg_mesh_set_shot_groups(mg_mesh* mesh, int kind, int groups);
  * five resident 256-thread CTAs per SM; more warps in flight for
  * HBM-bound meshes, a few spilled registers).  A handle whose launch shape
  * has not been set runs its row kernels under the cap of 5 with two float4
- * per lane (tangent: one) where the shot count allows it; setting either value
- * counts as setting the shape.  Drops the cached graphs.
+ * per lane (tangent: one) where the shot count allows it.  Drops the cached
+ * graphs.
  * Errors: MG_ERR_ARG for other values. */
 int mg_mesh_set_min_blocks(mg_mesh* mesh, int min_blocks);
 
@@ -524,7 +544,8 @@ int mg_mesh_device_status(mg_mesh* mesh);
 
 /* Current tuning into out[17]: chunk, then (batch, tile_rows, src_tile,
  * groups, min_blocks) for the forward, tangent and adjoint kinds, then the
- * forward's bulk-copy switch. */
+ * forward's bulk-copy switch.  Whether that shape is in force is the kind's
+ * path (mg_mesh_get_kernel_path). */
 int mg_mesh_get_tuning(const mg_mesh* mesh, int32_t* out);
 
 /* Autotuner: times every candidate launch shape of each kernel kind on the

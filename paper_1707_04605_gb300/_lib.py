@@ -38,6 +38,8 @@ class mg_shots(C.Structure):
                 ("rec_ptr", C.POINTER(C.c_int64)), ("rec", C.POINTER(C.c_int32))]
 
 
+MG_PATHS = {"auto": 0, "shape": 1, "resident": 2, "rows": 3}
+
 MG_DATA_TRACES = 0
 MG_DATA_PROJECTED = 1
 
@@ -85,6 +87,8 @@ SIGNATURES = {
     "mg_prolong": (C.c_int, [C.c_void_p, C.c_int, C.c_void_p, C.c_void_p, C.c_void_p,
                              C.c_void_p, C.c_int]),
     "mg_mesh_set_kernel_tuning": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_int, C.c_int]),
+    "mg_mesh_set_kernel_path": (C.c_int, [C.c_void_p, C.c_int, C.c_int]),
+    "mg_mesh_get_kernel_path": (C.c_int, [C.c_void_p, C.c_void_p]),
     "mg_mesh_set_shot_groups": (C.c_int, [C.c_void_p, C.c_int, C.c_int]),
     "mg_mesh_set_conductivity": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_int]),
     "mg_mesh_set_min_blocks": (C.c_int, [C.c_void_p, C.c_int]),

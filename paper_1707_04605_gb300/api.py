@@ -129,6 +129,14 @@ class Mesh:
                                                     int(tile_rows), int(src_tile)),
                 "mg_mesh_set_kernel_tuning")
 
+    def set_kernel_path(self, path: str, kind: str = None):
+        """Which kernels a kind (None: all) runs: "auto" (by estimate), "shape"
+        (the launch shape on the handle), "resident" (wherever it can run) or
+        "rows" (the library's own row shape); mg_mesh_set_kernel_path."""
+        L.check(self._lib.mg_mesh_set_kernel_path(self.handle,
+                                                  -1 if kind is None else self.KINDS[kind],
+                                                  L.MG_PATHS[path]), "mg_mesh_set_kernel_path")
+
     def set_shot_groups(self, groups: int, kind: str = None):
         """Shot groups advanced one after another per graph chunk / checkpoint
         segment (mg_mesh_set_shot_groups); kind None sets all kinds."""
@@ -268,6 +276,12 @@ class Mesh:
                 "mg_mesh_get_l1_streaming")
         for name, k in self.KINDS.items():
             d[name]["stream"] = int(l1[k])
+        path = np.zeros(3, dtype=np.int32)
+        L.check(self._lib.mg_mesh_get_kernel_path(self.handle, C.c_void_p(path.ctypes.data)),
+                "mg_mesh_get_kernel_path")
+        names = {v: k for k, v in L.MG_PATHS.items()}
+        for name, k in self.KINDS.items():
+            d[name]["path"] = names[int(path[k])]
         return d
 
     def autotune(self, eps, shots, wavelet, dt, steps=128, level=1, allow_cfl=False,

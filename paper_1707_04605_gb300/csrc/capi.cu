@@ -125,7 +125,7 @@ struct mg_mesh {
     int stream = 0;       // row kernels: once-read loads bypass L1 allocation
     int prefetch = 0;     // capped row kernels: prefetch of late-loaded rows (1 L1, 2 L2)
     int wide = 1;         // capped forward: 8 consecutive shots per lane (256-bit loads)
-    int shaped = 0;       // a launch shape was asked for: no resident kernel in its place
+    int path = MG_PATH_AUTO;   // what runs (mg_mesh_set_kernel_path)
   } tune[3];
   int dep_launch = 1;                     // row kernels launched as programmatic dependents
   Buf ellu;                               // ELL with every slice padded to wu columns
@@ -337,6 +337,7 @@ int cfl_lambda(mg_mesh* M, const double* eps_d, cudaStream_t st, double* lam) {
 }
 
 int ensure_tiles(mg_mesh* M);
+mg_mesh::Tuning in_force(const mg_mesh* M, int kind);
 
 // Common preparation of a propagation call: inputs on the device, per-row
 // coefficients, wavelet in FP32, event lists, dt check.
@@ -377,7 +378,8 @@ int prepare(mg_mesh* M, const double* eps, const mg_shots* shots, const double* 
   MG_TRY(build_events(M, shots, pp.ev));
   MG_TRY(ensure_tiles(M));
   // the status word of bounded device waits exists before any graph capture
-  if ((M->tune[0].bulk || M->tune[0].tma) && !err_word(M)) return MG_ERR_OOM;
+  const mg_mesh::Tuning t = in_force(M, 0);
+  if ((t.bulk || t.tma) && !err_word(M)) return MG_ERR_OOM;
   return MG_OK;
 }
 
@@ -385,7 +387,7 @@ int prepare(mg_mesh* M, const double* eps, const mg_shots* shots, const double* 
 // and uploaded on first use.
 int ensure_tiles(mg_mesh* M) {
   for (int k = 0; k < 4; ++k) {
-    const int P = k < 3 ? M->tune[k].tile_rows : M->tune[0].tma;
+    const int P = k < 3 ? in_force(M, k).tile_rows : in_force(M, 0).tma;
     if (P <= 0 || M->tiles.count(P)) continue;
     mg::HostTiles T;
     MG_TRY(mg::build_tiles(M->hm, P, T));
@@ -408,11 +410,24 @@ int ensure_tiles(mg_mesh* M) {
   return MG_OK;
 }
 
+// Launch shape in force for a kind: the one on the handle where its path says
+// so, else the defaults (row_shape picks the library's own).
+mg_mesh::Tuning in_force(const mg_mesh* M, int kind) {
+  const mg_mesh::Tuning& t = M->tune[kind];
+  if (t.path == MG_PATH_SHAPE || t.path == MG_PATH_RESIDENT) return t;
+  mg_mesh::Tuning d;
+  d.stream = t.stream;
+  d.prefetch = t.prefetch;
+  d.wide = t.wide;
+  d.path = t.path;
+  return d;
+}
+
 // Shot columns per group of a kernel kind: S_pad / groups when that is a
 // valid launch width (a power of two >= 4 up to 128, or a multiple of 128),
 // else S_pad (one group).
 int group_cols(const mg_mesh* M, int kind, int S_pad) {
-  const int G = M->tune[kind].groups;
+  const int G = in_force(M, kind).groups;
   if (G <= 1 || S_pad % G) return S_pad;
   const int W = S_pad / G;
   const bool ok = W >= 4 && (W % 128 == 0 || (W <= 128 && (W & (W - 1)) == 0));
@@ -446,7 +461,8 @@ mg::DevTiles tile_tables(mg_mesh* M, int P) {
 
 mg::DevTiles dev_tiles(mg_mesh* M, int cols, int kind) {
   mg::DevTiles T{};
-  const int P = M->tune[kind].tile_rows;
+  const mg_mesh::Tuning t = in_force(M, kind);
+  const int P = t.tile_rows;
   auto it = M->tiles.find(P);
   if (P <= 0 || it == M->tiles.end()) return T;
   const mg_mesh::TileTables& D = it->second;
@@ -461,7 +477,7 @@ mg::DevTiles dev_tiles(mg_mesh* M, int cols, int kind) {
   T.halo = P_<const int32_t>(D.halo);
   T.max_ell = D.max_ell;
   T.max_halo = D.max_halo;
-  T.st_w = std::min(M->tune[kind].src_tile, cols);
+  T.st_w = std::min(t.src_tile, cols);
   if (kind == 1) T.st_w = std::max(4, T.st_w / 2);
   if (mg::tiled_smem_bytes(T, kind) > (size_t)M->smem_optin) T.n_tiles = 0;
   return T;
@@ -491,8 +507,9 @@ struct RowShape {
   bool chunked;   // from M->auto_ellc
 };
 RowShape row_shape(const mg_mesh* M, int kind, int cols) {
-  const mg_mesh::Tuning& t = M->tune[kind];
-  if (t.shaped || cols < 16) return {t.batch, t.min_blocks, 512, false};
+  const mg_mesh::Tuning t = in_force(M, kind);
+  if (t.path == MG_PATH_SHAPE || t.path == MG_PATH_RESIDENT || cols < 16)
+    return {t.batch, t.min_blocks, 512, false};
   return {kind == 1 ? 1 : 2, 5, 128, !M->chunked_ell};
 }
 
@@ -533,20 +550,21 @@ int do_step(mg_mesh* M, const mg::StepArgs& a, int S_pad, cudaStream_t st) {
   b.batch = rs.batch;
   b.min_blocks = rs.min_blocks;
   use_auto_entries(M, rs, 0, cols, b.K);
-  b.ring = M->tune[0].ring;
-  b.sweep = M->tune[0].sweep;
-  b.stream = M->tune[0].stream;
-  b.prefetch = M->tune[0].prefetch;
-  b.wide = M->tune[0].wide;
+  const mg_mesh::Tuning t = in_force(M, 0);
+  b.ring = t.ring;
+  b.sweep = t.sweep;
+  b.stream = t.stream;
+  b.prefetch = t.prefetch;
+  b.wide = t.wide;
   b.pdl = M->dep_launch;
-  if (M->tune[0].tma) {
-    const mg::DevTiles TT = tile_tables(M, M->tune[0].tma);
+  if (t.tma) {
+    const mg::DevTiles TT = tile_tables(M, t.tma);
     int* err = err_word(M);
     if (!err) return MG_ERR_OOM;
     if (!TT.n_tiles) return MG_ERR_ARG;
     return mg::launch_step_tma(b, TT, S_pad, err, st);
   }
-  if (M->tune[0].bulk) {
+  if (t.bulk) {
     int* err = err_word(M);
     if (!err) return MG_ERR_OOM;
     return mg::launch_step_bulk(b, S_pad, err, st);
@@ -559,9 +577,10 @@ void row_tangent_args(mg_mesh* M, int cols, mg::TangentArgs& b) {
   b.f.batch = rs.batch;
   b.f.min_blocks = rs.min_blocks;
   use_auto_entries(M, rs, 1, cols, b.f.K);
-  b.f.ring = M->tune[1].ring;
-  b.f.stream = M->tune[1].stream;
-  b.f.prefetch = M->tune[1].prefetch;
+  const mg_mesh::Tuning t = in_force(M, 1);
+  b.f.ring = t.ring;
+  b.f.stream = t.stream;
+  b.f.prefetch = t.prefetch;
   b.f.pdl = M->dep_launch;
 }
 
@@ -583,9 +602,10 @@ int do_adjoint(mg_mesh* M, const mg::AdjointArgs& a, int S_pad, cudaStream_t st)
   b.min_blocks = rs.min_blocks;
   b.most_cols = rs.most_cols;
   use_auto_entries(M, rs, 2, cols, b.K);
-  b.ring = M->tune[2].ring;
-  b.stream = M->tune[2].stream;
-  b.prefetch = M->tune[2].prefetch;
+  const mg_mesh::Tuning t = in_force(M, 2);
+  b.ring = t.ring;
+  b.stream = t.stream;
+  b.prefetch = t.prefetch;
   b.pdl = M->dep_launch;
   return mg::launch_adjoint(b, S_pad, st);
 }
@@ -608,7 +628,7 @@ mg::StepArgs step_args(mg_mesh* M, const Prep& pp, int ld, int nt) {
   a.wavelet = P<const float>(M->wavf);
   a.nt = nt;
   a.step_base = nullptr;
-  a.batch = M->tune[0].batch;
+  a.batch = in_force(M, 0).batch;
   return a;
 }
 
@@ -761,11 +781,14 @@ double rows_us(const mg_mesh* M, int kind, int S_pad) {
 // same with p and dp as columns (2 lpr shots per launch); adjoint: whole source
 // tiles of the row kernel only, for the same sums over the shots.
 // shape.lpr = 0: the row kernels are the path (nothing fits, they are estimated
-// to be faster, or a launch shape of theirs was asked for).
+// to be faster, or the kind's path asks for them; MG_PATH_RESIDENT leaves the
+// estimate out).
 int resident_shape(mg_mesh* M, int kind, int S_pad, int steps, mg::DevPatches& D,
                    mg::ResidentShape& shape) {
   shape = mg::ResidentShape();
-  if (M->tune[kind].shaped || steps < 16 || M->hm.max_row_nnz > 256) return MG_OK;
+  const int path = M->tune[kind].path;
+  if (path == MG_PATH_SHAPE || path == MG_PATH_ROWS || steps < 16 || M->hm.max_row_nnz > 256)
+    return MG_OK;
   if (!M->n_sm)
     MG_CU(cudaDeviceGetAttribute(&M->n_sm, cudaDevAttrMultiProcessorCount, M->device));
   const int B = (int)std::min<int64_t>(M->n_sm, std::max<int64_t>(1, M->hm.n / 32));
@@ -781,7 +804,9 @@ int resident_shape(mg_mesh* M, int kind, int S_pad, int steps, mg::DevPatches& D
     }
     if (kind == 2) break;
   }
-  if (shape.lpr && resident_us(D, shape, kind, S_pad) > rows_us(M, kind, S_pad)) shape.lpr = 0;
+  if (shape.lpr && path == MG_PATH_AUTO &&
+      resident_us(D, shape, kind, S_pad) > rows_us(M, kind, S_pad))
+    shape.lpr = 0;
   return MG_OK;
 }
 
@@ -1272,8 +1297,16 @@ static void drop_graphs(mg_mesh* M) {
   M->graphs.clear();
 }
 
+// A setter of one launch-shape field: another value than the one on the handle
+// asks for the shape, the same one asks for nothing.
+static void set_field(mg_mesh::Tuning& t, int mg_mesh::Tuning::* field, int value) {
+  if (t.*field == value) return;
+  t.*field = value;
+  t.path = MG_PATH_SHAPE;
+}
+
 static void apply_tuning(mg_mesh::Tuning& t, int batch, int tile_rows, int src_tile) {
-  if (batch != -1 || tile_rows != -1 || src_tile != -1) t.shaped = 1;
+  if (batch != -1 || tile_rows != -1 || src_tile != -1) t.path = MG_PATH_SHAPE;
   if (batch != -1) t.batch = batch;
   if (tile_rows != -1) t.tile_rows = tile_rows;
   if (src_tile != -1) t.src_tile = src_tile;
@@ -1301,10 +1334,7 @@ int mg_mesh_set_shot_groups(mg_mesh* M, int kind, int groups) {
     return MG_ERR_ARG;
   drop_graphs(M);
   for (int k = 0; k < 3; ++k)
-    if (kind == -1 || kind == k) {
-      M->tune[k].groups = groups;
-      M->tune[k].shaped = 1;
-    }
+    if (kind == -1 || kind == k) set_field(M->tune[k], &mg_mesh::Tuning::groups, groups);
   return MG_OK;
 }
 
@@ -1413,8 +1443,7 @@ int mg_mesh_set_dependent_launch(mg_mesh* M, int on) {
 int mg_mesh_set_bulk_copies(mg_mesh* M, int on) {
   if (!M || (on != 0 && on != 1)) return MG_ERR_ARG;
   drop_graphs(M);
-  M->tune[0].bulk = on;
-  M->tune[0].shaped = 1;
+  set_field(M->tune[0], &mg_mesh::Tuning::bulk, on);
   return MG_OK;
 }
 
@@ -1434,18 +1463,14 @@ int mg_mesh_set_gather_ring(mg_mesh* M, int kind, int depth) {
   if (!M || kind < -1 || kind > 2 || (depth != 0 && depth != 4 && depth != 8)) return MG_ERR_ARG;
   drop_graphs(M);
   for (int k = 0; k < 3; ++k)
-    if (kind == -1 || kind == k) {
-      M->tune[k].ring = depth;
-      M->tune[k].shaped = 1;
-    }
+    if (kind == -1 || kind == k) set_field(M->tune[k], &mg_mesh::Tuning::ring, depth);
   return MG_OK;
 }
 
 int mg_mesh_set_row_sweep(mg_mesh* M, int blocks) {
   if (!M || blocks < 0 || blocks > 65536) return MG_ERR_ARG;
   drop_graphs(M);
-  M->tune[0].sweep = blocks;
-  M->tune[0].shaped = 1;
+  set_field(M->tune[0], &mg_mesh::Tuning::sweep, blocks);
   return MG_OK;
 }
 
@@ -1492,8 +1517,7 @@ int mg_mesh_get_l1_streaming(const mg_mesh* M, int32_t* out) {
 int mg_mesh_set_tma_tiles(mg_mesh* M, int rows) {
   if (!M || rows < 0 || rows > 1024 || rows % mg::kSliceH) return MG_ERR_ARG;
   drop_graphs(M);
-  M->tune[0].tma = rows;
-  M->tune[0].shaped = 1;
+  set_field(M->tune[0], &mg_mesh::Tuning::tma, rows);
   return MG_OK;
 }
 
@@ -1520,8 +1544,7 @@ int mg_mesh_get_gather_ring(const mg_mesh* M, int32_t* out) {
 int mg_mesh_set_min_blocks(mg_mesh* M, int min_blocks) {
   if (!M || (min_blocks != 0 && min_blocks != 5)) return MG_ERR_ARG;
   drop_graphs(M);
-  M->tune[0].min_blocks = min_blocks;
-  M->tune[0].shaped = 1;
+  set_field(M->tune[0], &mg_mesh::Tuning::min_blocks, min_blocks);
   return MG_OK;
 }
 
@@ -1530,8 +1553,22 @@ int mg_mesh_set_kernel_min_blocks(mg_mesh* M, int kind, int min_blocks) {
       (min_blocks != 0 && min_blocks != 5 && (min_blocks != 6 || kind != 2)))
     return MG_ERR_ARG;
   drop_graphs(M);
-  M->tune[kind].min_blocks = min_blocks;
-  M->tune[kind].shaped = 1;
+  set_field(M->tune[kind], &mg_mesh::Tuning::min_blocks, min_blocks);
+  return MG_OK;
+}
+
+int mg_mesh_set_kernel_path(mg_mesh* M, int kind, int path) {
+  if (!M || kind < -1 || kind > 2 || path < MG_PATH_AUTO || path > MG_PATH_ROWS)
+    return MG_ERR_ARG;
+  drop_graphs(M);
+  for (int k = 0; k < 3; ++k)
+    if (kind == -1 || kind == k) M->tune[k].path = path;
+  return MG_OK;
+}
+
+int mg_mesh_get_kernel_path(const mg_mesh* M, int32_t* out) {
+  if (!M || !out) return MG_ERR_ARG;
+  for (int k = 0; k < 3; ++k) out[k] = M->tune[k].path;
   return MG_OK;
 }
 
@@ -1717,9 +1754,10 @@ int mg_jacobian_apply(mg_mesh* M, int level, const double* eps, const mg_shots* 
                       M->ck_ev_gen == M->ev_gen;
     if (!kept) return MG_ERR_ARG;
     float* seg = P<float>(M->seg);
-    a.f.batch = M->tune[1].batch;
-    a.f.ring = M->tune[1].ring;
-    a.f.stream = M->tune[1].stream;
+    const mg_mesh::Tuning t = in_force(M, 1);
+    a.f.batch = t.batch;
+    a.f.ring = t.ring;
+    a.f.stream = t.stream;
     a.f.pdl = M->dep_launch;
     a.f.hint = M->cache_hints;
     const int W = group_cols(M, 1, pp.S_pad), NG = pp.S_pad / W;
@@ -1893,7 +1931,7 @@ int mg_forward_jacobian_apply(mg_mesh* M, int level, const double* eps, const mg
   mg::TangentArgs a{};
   a.f = step_args(M, pp, pp.S_pad, nt);
   a.f.traces = trf;
-  a.f.batch = M->tune[1].batch;   // MG_PERSISTENT
+  a.f.batch = in_force(M, 1).batch;   // MG_PERSISTENT
   a.f.hint = keep ? M->cache_hints : 0;   // p_{l-1} is last read here only when kept
   a.tcoef = P<const float2>(M->tcoef);
   a.dtraces = tr;
@@ -2041,11 +2079,12 @@ int mg_jacobian_T_apply(mg_mesh* M, int level, const double* eps, const mg_shots
   aa.w = wd;
   aa.nt = nt;
   aa.step_base = nullptr;
-  aa.batch = M->tune[2].batch;
-  aa.ring = M->tune[2].ring;
-  aa.stream = M->tune[2].stream;
-  aa.prefetch = M->tune[2].prefetch;
-  aa.min_blocks = M->tune[2].min_blocks;
+  const mg_mesh::Tuning ta = in_force(M, 2);
+  aa.batch = ta.batch;
+  aa.ring = ta.ring;
+  aa.stream = ta.stream;
+  aa.prefetch = ta.prefetch;
+  aa.min_blocks = ta.min_blocks;
   aa.G = G;
   aa.Gc = G + acc;
   aa.H = G + 2 * acc;
@@ -2324,10 +2363,10 @@ int mg_autotune(mg_mesh* M, const double* eps, const mg_shots* shots, const doub
   if (rc == MG_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = MG_ERR_CUDA;
   // the L1 policy is the caller's setting, not a candidate
   const int l1[3] = {M->tune[0].stream, M->tune[1].stream, M->tune[2].stream};
-  auto time_of = [&](int kind, mg_mesh::Tuning c, float* out, int shaped = 1) -> int {
+  auto time_of = [&](int kind, mg_mesh::Tuning c, float* out, int path = MG_PATH_SHAPE) -> int {
     drop_graphs(M);
     c.stream = l1[kind];
-    c.shaped = shaped;
+    c.path = path;
     M->tune[kind] = c;
     int r = run(kind);  // warm-up: tile tables, buffers, graphs
     float cand = 1e30f;
@@ -2379,6 +2418,7 @@ int mg_autotune(mg_mesh* M, const double* eps, const mg_shots* shots, const doub
         mg_mesh::Tuning c = shapes[order[top]];
         c.groups = G;
         c.stream = l1[kind];
+        c.path = MG_PATH_SHAPE;
         M->tune[kind] = c;
         if (group_cols(M, kind, S_pad) == S_pad) continue;
         float t = 0.0f;
@@ -2387,7 +2427,7 @@ int mg_autotune(mg_mesh* M, const double* eps, const mg_shots* shots, const doub
         if (t < best * 0.99f) { best = t; pick = c; }   // groups must win by more than 1%
       }
     }
-    pick.shaped = 1;
+    pick.path = MG_PATH_SHAPE;
     // the resident kernel, where the problem fits it, against the best of these
     mg::DevPatches D;
     mg::ResidentShape shape;
@@ -2395,8 +2435,8 @@ int mg_autotune(mg_mesh* M, const double* eps, const mg_shots* shots, const doub
     if (rc == MG_OK) rc = resident_shape(M, kind, S_pad, steps, D, shape);
     if (rc == MG_OK && shape.lpr) {
       float t = 0.0f;
-      rc = time_of(kind, pick, &t, 0);
-      if (t < best) pick.shaped = 0;
+      rc = time_of(kind, pick, &t, MG_PATH_AUTO);
+      if (t < best) pick.path = MG_PATH_AUTO;
     }
     M->tune[kind] = pick;
   }
@@ -2499,7 +2539,7 @@ int mesh_view(mg_mesh* M, MeshView* v) {
   v->row_abs = P<const double>(M->row_abs);
   v->perm_host = M->hm.perm.data();
   v->launches = &M->launches;
-  v->batch = M->tune[0].batch;
+  v->batch = in_force(M, 0).batch;
   return MG_OK;
 }
 

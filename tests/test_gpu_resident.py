@@ -151,3 +151,62 @@ def test_default_row_shapes_carry_the_plain_shape_bits(mg, make, kw):
 
     for x, y in zip(run(a), run(b)):
         assert torch.equal(x, y)
+
+
+def _steps_per_launch(mg, mesh, w, eps, s, dt):
+    n0 = mesh.launch_count()
+    mg.forward(mesh, eps, w.shots, s, dt)
+    return w.nt / (mesh.launch_count() - n0)
+
+
+def test_a_setter_that_changes_nothing_keeps_the_path(mg):
+    """Only a value that differs, or an explicit batch or tile, selects a launch
+    shape in place of the resident kernels."""
+    w = configs.asteroid_2d(n_refine=2, S=24, nt=64)
+    m = mg.mesh_from_workload(w)
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    s = _dev(w.wavelet(dt))
+    m.set_shot_groups(1)
+    m.set_gather_ring(0)
+    m.set_row_sweep(0)
+    m.set_tma_tiles(0)
+    m.set_bulk_copies(False)
+    for kind in ("forward", "tangent", "adjoint"):
+        m.set_min_blocks(0, kind)
+        assert m.tuning()[kind]["path"] == "auto"
+    assert _steps_per_launch(mg, m, w, eps, s, dt) > 4
+    m.set_min_blocks(5)
+    assert m.tuning()["forward"]["path"] == "shape" and m.tuning()["adjoint"]["path"] == "auto"
+    assert _steps_per_launch(mg, m, w, eps, s, dt) < 2
+
+
+def test_a_tuning_that_is_read_and_set_again_keeps_the_path(mg):
+    w = configs.asteroid_2d(n_refine=2, S=24, nt=64)
+    a, b, c = (mg.mesh_from_workload(w) for _ in range(3))
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    s = _dev(w.wavelet(dt))
+    a.set_kernel_tuning("adjoint", 2, 64, 16)
+    a.set_shot_groups(2, "adjoint")
+    a.set_kernel_path("resident", "adjoint")
+    a.set_kernel_path("rows", "tangent")
+    t = a.tuning()
+    for kind in ("forward", "tangent", "adjoint"):
+        b.set_kernel_tuning(kind, t[kind]["batch"], t[kind]["tile_rows"], t[kind]["src_tile"])
+        b.set_shot_groups(t[kind]["groups"], kind)
+        b.set_kernel_path(t[kind]["path"], kind)
+    assert b.tuning() == t
+    assert _steps_per_launch(mg, b, w, eps, s, dt) > 4
+    # every path, the same bits
+    rng = np.random.default_rng(2)
+    v = _dev(rng.standard_normal(w.mesh.n_cells[1]))
+    W = _dev(rng.standard_normal((w.shots.n_traces, w.nt)), torch.float32)
+    ref = None
+    for path in ("shape", "auto", "resident", "rows"):
+        c.set_kernel_path(path)
+        out = (mg.forward(c, eps, w.shots, s, dt),
+               mg.jacobian_apply(c, 1, eps, w.shots, s, dt, v),
+               mg.jacobian_T_apply(c, 1, eps, w.shots, s, dt, W, ckpt_every=17))
+        ref = ref or out
+        assert all(torch.equal(x, y) for x, y in zip(out, ref)), path
+    with pytest.raises(KeyError):
+        c.set_kernel_path("fastest")
