@@ -2062,9 +2062,19 @@ int mg_jacobian_T_apply(mg_mesh* M, int level, const double* eps, const mg_shots
   // reverse steps).
   const int Wf = group_cols(M, 0, pp.S_pad), NGf = pp.S_pad / Wf;
   const int Wa = group_cols(M, 2, pp.S_pad), NGa = pp.S_pad / Wa;
+  // resident kernels for the recompute and the reverse steps of a segment (not
+  // for one too short; MG_PERSISTENT asks for its own kernels)
+  mg::DevPatches Df, Da;
+  mg::ResidentShape shf, sha;
+  if (!(flags & MG_PERSISTENT)) {
+    MG_TRY(resident_shape(M, 0, pp.S_pad, std::min(ckpt_every, nt), Df, shf));
+    MG_TRY(resident_shape(M, 2, pp.S_pad, std::min(ckpt_every, nt), Da, sha));
+  }
   // accumulators: one set per source tile of the untiled kernel; the tiled
-  // kernel sums all shots of a row inside its CTA
-  const int acc_sets = adjoint_sets(M, pp.S_pad, Wa);
+  // kernel sums all shots of a row inside its CTA; the resident kernel, which
+  // either of them may share the segments with, one per source tile
+  int acc_sets = adjoint_sets(M, pp.S_pad, Wa);
+  if (sha.lpr) acc_sets = std::max(acc_sets, pp.S_pad / (4 * sha.lpr));
   const size_t acc = (size_t)acc_sets * n;
   MG_TRY(ensure(M->G, 4 * acc * sizeof(float)));
   MG_CU(cudaMemsetAsync(M->G.p, 0, 4 * acc * sizeof(float), st));
@@ -2095,14 +2105,6 @@ int mg_jacobian_T_apply(mg_mesh* M, int level, const double* eps, const mg_shots
   if (use_graph) {
     MG_TRY(ensure(M->step_base, 16));
     base = P<int32_t>(M->step_base);
-  }
-  // resident kernels for the recompute and the reverse steps of a segment (not
-  // for one too short; MG_PERSISTENT asks for its own kernels)
-  mg::DevPatches Df, Da;
-  mg::ResidentShape shf, sha;
-  if (!(flags & MG_PERSISTENT)) {
-    MG_TRY(resident_shape(M, 0, pp.S_pad, std::min(ckpt_every, nt), Df, shf));
-    MG_TRY(resident_shape(M, 2, pp.S_pad, std::min(ckpt_every, nt), Da, sha));
   }
   if (!shf.lpr && !states) MG_TRY(ensure_auto_entries(M, 0, Wf, st));
   if (!sha.lpr) MG_TRY(ensure_auto_entries(M, 2, Wa, st));

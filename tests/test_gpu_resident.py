@@ -210,3 +210,25 @@ def test_a_tuning_that_is_read_and_set_again_keeps_the_path(mg):
         assert all(torch.equal(x, y) for x, y in zip(out, ref)), path
     with pytest.raises(KeyError):
         c.set_kernel_path("fastest")
+
+
+@pytest.mark.parametrize("S,nt,ckpt,tol", [(256, 64, 32, 0.0), (300, 48, 48, 0.0),
+                                           (256, 70, 32, 1e-5)])
+def test_resident_reverse_steps_beside_a_tiled_shape(mg, S, nt, ckpt, tol):
+    """The tiled kernel keeps one accumulator set for all shots, the resident one
+    a set per 128: the same gradient where the handle's shape is tiled and the
+    reverse steps run resident (the last, short segment, if any, on the tiled
+    kernel, which adds the shots in another order)."""
+    w = configs.asteroid_2d(n_refine=2, S=S, nt=nt)
+    a, b = _pair(mg, w)
+    a.set_kernel_tuning("adjoint", 1, 64, 32)
+    a.set_kernel_path("resident", "adjoint")
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    s = _dev(w.wavelet(dt))
+    W = _dev(np.random.default_rng(6).standard_normal((w.shots.n_traces, w.nt)), torch.float32)
+    run = lambda m: mg.jacobian_T_apply(m, 1, eps, w.shots, s, dt, W, ckpt_every=ckpt)
+    n0 = a.launch_count()
+    x = run(a)
+    assert a.launch_count() - n0 < nt            # resident: not a launch per reverse step
+    y = run(b)
+    assert torch.equal(x, y) if tol == 0.0 else float((x - y).norm() / y.norm()) < tol
