@@ -177,7 +177,8 @@ int mg_cfl_dt(mg_mesh* mesh, const double* eps, int flags, void* stream,
  * either way.  The tangent and the reverse steps choose likewise, each by its
  * own kind's shape.  The patches' waits for one another are bounded by
  * mg_mesh_set_persistent's wait_cycles: when one runs out the call's outputs
- * are NaN and mg_mesh_device_status returns MG_ERR_TIMEOUT.  With fewer
+ * are NaN and mg_mesh_device_status returns MG_ERR_TIMEOUT; the same for a later
+ * call that reuses checkpoints or states which such a call kept.  With fewer
  * than 16 steps between checkpoints, and where no patch fits, the row kernels
  * run.
  * Flags: MG_HOST_PTRS, MG_NO_GRAPH,
@@ -641,7 +642,8 @@ int mg_projected_weights(const float* u, const double* z, int64_t n_traces, int 
  *   flags      MG_HOST_PTRS (eps0, wavelet, dy, u, x_out on the host),
  *              MG_ALLOW_CFL.  Synchronous.
  * Errors: MG_ERR_ARG (levels, params out of range, null pointers),
- * MG_ERR_NESTING (children of a coarse cell not facet-connected), plus
+ * MG_ERR_NESTING (children of a coarse cell not facet-connected),
+ * MG_ERR_TIMEOUT (a device wait of one of its wave calls ran out), plus
  * those of the Jacobian calls. */
 #define MG_DATA_TRACES    0
 #define MG_DATA_PROJECTED 1

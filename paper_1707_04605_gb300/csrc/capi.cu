@@ -483,8 +483,10 @@ mg::DevTiles dev_tiles(mg_mesh* M, int cols, int kind) {
   return T;
 }
 
-// One launch over the shot columns [a.col0, a.col0 + a.cols) (cols = 0:
-// all S_pad columns).
+// Device words of bounded waits: status (mg_mesh_device_status), arrivals of the
+// persistent kernels' barrier, whether the kept states come from a launch whose
+// wait ran out, and how many outputs were set to NaN so far.
+enum { kWordStatus, kWordArrivals, kWordKept, kWordPoisoned };
 int* err_word(mg_mesh* M) {
   if (!M->errbuf.p) {
     if (ensure(M->errbuf, 16) != MG_OK) return nullptr;
@@ -680,7 +682,7 @@ int persist_args(mg_mesh* M, cudaStream_t st, float* seg, size_t state, mg::Pers
   int* status = err_word(M);
   if (!status) return MG_ERR_OOM;
   MG_CU(cudaMemsetAsync(status, 0, sizeof(int), st));
-  pa.count = reinterpret_cast<unsigned*>(status + 1);
+  pa.count = reinterpret_cast<unsigned*>(status + kWordArrivals);
   pa.status = status;
   pa.budget = M->persist_budget;
   pa.extra = M->persist_extra;
@@ -823,6 +825,29 @@ int resident_buffers(mg_mesh* M, const mg::DevPatches& D, int lpr, cudaStream_t 
   return MG_OK;
 }
 
+// Outputs of a call become NaN where one of its resident launches ran out of a
+// wait, or (reused) those that kept the states it has read.
+int poison(mg_mesh* M, float* x, int64_t n, bool reused, cudaStream_t st) {
+  if (!M->errbuf.p || !(M->status_clear || reused)) return MG_OK;
+  int* w = P<int>(M->errbuf);
+  M->launches += 1;
+  return mg::launch_poison(x, n, M->status_clear ? w + kWordStatus : nullptr,
+                           reused ? w + kWordKept : nullptr, w + kWordStatus, w + kWordPoisoned,
+                           st);
+}
+
+// After the launches of a call that keeps states: whether they can be trusted.
+int note_kept(mg_mesh* M, cudaStream_t st) {
+  if (!M->errbuf.p) return MG_OK;
+  int* w = P<int>(M->errbuf);
+  if (M->status_clear)
+    MG_CU(cudaMemcpyAsync(w + kWordKept, w + kWordStatus, sizeof(int), cudaMemcpyDeviceToDevice,
+                          st));
+  else
+    MG_CU(cudaMemsetAsync(w + kWordKept, 0, sizeof(int), st));
+  return MG_OK;
+}
+
 mg::ResidentArgs resident_args(mg_mesh* M, const Prep& pp, int nt, const mg::DevPatches& D) {
   mg::ResidentArgs r{};
   r.P = D;
@@ -870,10 +895,7 @@ int run_tangent_resident(mg_mesh* M, const Prep& pp, int nt, float* traces, floa
     M->launches += 1;
   }
   for (float* x : {traces, dtraces})
-    if (x) {
-      MG_TRY(mg::launch_poison(x, pp.R * nt, r.status, st));
-      M->launches += 1;
-    }
+    if (x) MG_TRY(poison(M, x, pp.R * nt, false, st));
   return MG_OK;
 }
 
@@ -906,11 +928,7 @@ int run_forward_resident(mg_mesh* M, const Prep& pp, int nt, float* traces, int 
       M->launches += 1;
     }
   }
-  if (traces) {
-    MG_TRY(mg::launch_poison(traces, pp.R * nt, r.status, st));
-    M->launches += 1;
-  }
-  return MG_OK;
+  return traces ? poison(M, traces, pp.R * nt, false, st) : MG_OK;
 }
 
 // Batched forward loop over steps [0, nt); optional traces and checkpoints.
@@ -1664,6 +1682,7 @@ int mg_forward(mg_mesh* M, const double* eps, const mg_shots* shots, const doubl
     const size_t state = (size_t)M->hm.n * pp.S_pad;
     MG_TRY(ensure(M->seg, (size_t)(nt + 2) * state * sizeof(float)));
     MG_TRY(run_forward_states(M, pp, nt, tr, P<float>(M->seg), st, flags));
+    MG_TRY(note_kept(M, st));
     M->ck_valid = true;  M->ck_gen++;
     M->seg_full = true;
     M->ck_every = nt;
@@ -1685,6 +1704,7 @@ int mg_forward(mg_mesh* M, const double* eps, const mg_shots* shots, const doubl
     // the barrier waits are bounded: read (and clear) the status word
     if (flags & MG_PERSISTENT) MG_TRY(persist_status(M, st));
     if (ck) {
+      MG_TRY(note_kept(M, st));
       M->ck_valid = true;  M->ck_gen++;
       M->ck_every = ckpt_every;
       M->ck_nt = nt;
@@ -1798,6 +1818,7 @@ int mg_jacobian_apply(mg_mesh* M, int level, const double* eps, const mg_shots* 
       MG_TRY(record(st));
       M->launches += (int64_t)NG * nt;
     }
+    MG_TRY(poison(M, tr, pp.R * nt, true, st));
     return deliver(M->tr, jv, tbytes, flags, st);
   }
   int l = 0;
@@ -1891,6 +1912,7 @@ int mg_forward_jacobian_apply(mg_mesh* M, int level, const double* eps, const mg
   }
   auto finish = [&]() -> int {
     if (keep) {
+      MG_TRY(note_kept(M, st));
       M->ck_valid = true;  M->ck_gen++;
       M->seg_full = true;
       M->ck_every = nt;
@@ -2294,10 +2316,7 @@ int mg_jacobian_T_apply(mg_mesh* M, int level, const double* eps, const mg_shots
   MG_TRY(mg::launch_restrict(nc, P<int64_t>(M->lvl_ptr[level]), P<int32_t>(M->lvl_idx[level]),
                              ga.g_fine, P<double>(M->g_h), st));
   M->launches += 2;
-  if (M->status_clear) {   // resident launches ran: NaN if one of their waits ran out
-    MG_TRY(mg::launch_poison(P<float>(M->g_h), 2 * nc, err_word(M), st));
-    M->launches += 1;
-  }
+  MG_TRY(poison(M, P<float>(M->g_h), 2 * nc, reuse, st));
   return deliver(M->g_h, g, nc * sizeof(double), flags, st);
 }
 
@@ -2459,6 +2478,15 @@ const HostMesh* host_mesh(const mg_mesh* M) { return M ? &M->hm : nullptr; }
 int mesh_device(const mg_mesh* M) { return M->device; }
 int mesh_graph_chunk(const mg_mesh* M) { return M->chunk; }
 void add_launches(mg_mesh* M, int64_t n) { M->launches += n; }
+
+int mesh_poisoned(mg_mesh* M, cudaStream_t st, int* count) {
+  *count = 0;
+  if (!M->errbuf.p) return MG_OK;
+  MG_CU(cudaMemcpyAsync(count, P<int>(M->errbuf) + kWordPoisoned, sizeof(int),
+                        cudaMemcpyDeviceToHost, st));
+  MG_CU(cudaStreamSynchronize(st));
+  return MG_OK;
+}
 
 void mesh_take_scratch(mg_mesh* M, std::vector<FluxBuffer>& bufs) {
   std::lock_guard<std::mutex> lock(M->flux_mu);

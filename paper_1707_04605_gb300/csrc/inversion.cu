@@ -638,9 +638,15 @@ extern "C" int mg_tv_reconstruct_levels(mg_mesh* M, const int* levels, int n_lev
   }
   MG_CK(cudaMemsetAsync(xc, 0, n_c * sizeof(double), st));
 
-  // one forward with checkpoints; every J^T reuses them
+  // one forward with checkpoints; every J^T reuses them.  A wave call whose
+  // device wait ran out gives NaN, which the CG loops would take for a breakdown:
+  // such calls are counted instead.
+  int poisoned0 = 0, poisoned = 0;
+  MG_RC(mesh_poisoned(M, st, &poisoned0));
   MG_RC(mg_forward(M, S.eps, shots, S.wav, dt, nt, S.tr, Pm.ckpt_every, st,
                    S.fl | MG_KEEP_CHECKPOINTS));
+  MG_RC(mesh_poisoned(M, st, &poisoned));
+  if (poisoned != poisoned0) return MG_ERR_TIMEOUT;
   // b_c = L_c^T dy (the same on every outer step)
   MG_RC(S.apply_LT(level_c, S.dy, bc));
 
@@ -752,6 +758,8 @@ extern "C" int mg_tv_reconstruct_levels(mg_mesh* M, const int* levels, int n_lev
       level_prev = f.level;
     }
   }
+  MG_RC(mesh_poisoned(M, st, &poisoned));
+  if (poisoned != poisoned0) return MG_ERR_TIMEOUT;
   // (4) x = R_c x_c + sum_i R_fi x_fi on the last level
   const int64_t n_out = nf ? FL[nf - 1].n : n_c;
   const double* xl = nf ? FL[nf - 1].comp : xc;

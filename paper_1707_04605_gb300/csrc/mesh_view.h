@@ -41,6 +41,9 @@ const HostMesh* host_mesh(const mg_mesh* mesh);
 int mesh_device(const mg_mesh* mesh);
 int mesh_graph_chunk(const mg_mesh* mesh);   // steps per CUDA-graph chunk (0: off)
 void add_launches(mg_mesh* mesh, int64_t n);
+// Outputs that the handle's calls have set to NaN so far because a device wait
+// ran out; synchronises with the stream.
+int mesh_poisoned(mg_mesh* mesh, cudaStream_t st, int* count);
 
 // Work buffers of the flux path's calls: taken from the handle for a call, and
 // left on it again (false: it holds a set already).

@@ -9,8 +9,14 @@
 namespace mg {
 namespace {
 
-__global__ void k_poison(float* x, int64_t n, const int* status) {
-  if (*status == 0) return;
+// (a may be status: every block finds it set, whoever comes first)
+__global__ void k_poison(float* x, int64_t n, const int* a, const int* b, int* status,
+                         int* count) {
+  if (!(a && *a) && !(b && *b)) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *status = 1;
+    ++*count;
+  }
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     x[i] = __int_as_float(0x7fffffff);
@@ -58,9 +64,11 @@ int launch_resident_step(const ResidentArgs& a, const ResidentShape& s, cudaStre
   return MG_ERR_ARG;
 }
 
-int launch_poison(float* x, int64_t n, const int* status, cudaStream_t st) {
+int launch_poison(float* x, int64_t n, const int* a, const int* b, int* status, int* count,
+                  cudaStream_t st) {
   if (n <= 0) return MG_OK;
-  k_poison<<<(unsigned)std::min<int64_t>((n + 255) / 256, 1024), 256, 0, st>>>(x, n, status);
+  k_poison<<<(unsigned)std::min<int64_t>((n + 255) / 256, 1024), 256, 0, st>>>(x, n, a, b, status,
+                                                                               count);
   return check_launch();
 }
 

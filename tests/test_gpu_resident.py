@@ -232,3 +232,67 @@ def test_resident_reverse_steps_beside_a_tiled_shape(mg, S, nt, ckpt, tol):
     assert a.launch_count() - n0 < nt            # resident: not a launch per reverse step
     y = run(b)
     assert torch.equal(x, y) if tol == 0.0 else float((x - y).norm() / y.norm()) < tol
+
+
+@pytest.mark.parametrize("path", ["auto", "rows"])
+def test_kept_states_of_a_wait_that_ran_out_are_not_used(mg, path):
+    """Checkpoints and histories that a timed-out launch left behind: every call
+    that reads them gives NaN and MG_ERR_TIMEOUT, on either path, until states
+    are kept anew."""
+    from paper_1707_04605_gb300 import _lib as L
+
+    w = configs.asteroid_2d(n_refine=2, S=37, nt=200)
+    a, b = _pair(mg, w)
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    s = _dev(w.wavelet(dt))
+    rng = np.random.default_rng(7)
+    v = _dev(rng.standard_normal(w.mesh.n_cells[1]))
+    W = _dev(rng.standard_normal((w.shots.n_traces, w.nt)), torch.float32)
+    keeps = [
+        (lambda m: mg.forward(m, eps, w.shots, s, dt, keep_checkpoints=True, ckpt_every=50), 50),
+        (lambda m: mg.forward(m, eps, w.shots, s, dt, keep_states=True), w.nt),
+        (lambda m: mg.forward_jacobian_apply(m, 1, eps, w.shots, s, dt, v, keep_states=True),
+         w.nt)]
+
+    def reuse(m, every):
+        out = [mg.jacobian_T_apply(m, 1, eps, w.shots, s, dt, W, ckpt_every=every,
+                                   reuse_checkpoints=True)]
+        if every == w.nt:
+            out.append(mg.jacobian_apply(m, 1, eps, w.shots, s, dt, v, reuse_states=True))
+        return out
+
+    for keep, every in keeps:
+        a.set_kernel_path("auto")
+        a.set_persistent(wait_cycles=1000)
+        keep(a)
+        assert a.device_status() == L.MG_ERR_TIMEOUT
+        a.set_persistent()
+        a.set_kernel_path(path)
+        for x in reuse(a, every):
+            assert bool(torch.isnan(x).all())
+        assert a.device_status() == L.MG_ERR_TIMEOUT
+        keep(a)
+        keep(b)
+        for x, y in zip(reuse(a, every), reuse(b, every)):
+            assert torch.equal(x, y)
+        assert a.device_status() == 0
+
+
+def test_a_reconstruction_whose_waits_run_out_is_an_error(mg):
+    from paper_1707_04605_gb300 import _lib as L
+
+    w = configs.asteroid_2d(n_refine=1, S=12, nt=120)
+    m = mg.mesh_from_workload(w)
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    s = _dev(w.wavelet(dt))
+    dy = _dev(1e-3 * np.random.default_rng(8).standard_normal((w.shots.n_traces, w.nt)),
+              torch.float32)
+    run = lambda: mg.tv_reconstruct(m, 0, eps, w.shots, s, dt, dy, level_f=1, alpha=1e-2, beta=1.0,
+                                    n_outer=1, n_cg=2, ckpt_every=40)
+    x0, _ = run()
+    m.set_persistent(wait_cycles=1000)
+    with pytest.raises(L.MgError) as e:
+        run()
+    assert e.value.code == L.MG_ERR_TIMEOUT
+    m.set_persistent()
+    assert torch.equal(run()[0], x0)
