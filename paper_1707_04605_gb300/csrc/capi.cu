@@ -10,7 +10,9 @@
 #include <cstring>
 #include <initializer_list>
 #include <map>
+#include <memory>
 #include <mutex>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -153,10 +155,12 @@ struct mg_mesh {
   // partitions of the resident kernels by patch count, their row groups by rows
   // per warp
   struct PatchTables {
-    mg::HostPatches host;
+    mg::HostPatches host;                 // B = 0: the mesh cannot be cut so
     struct Groups {
-      Buf grp_off, border, pair_off, halo_off, x_off, hdr, row, halo, halo_x, diag, pair;
-      mg::DevPatches dev{};
+      std::array<Buf, 11> buf;
+      mg::DevPatches dev{};               // sizes; the pointers once on_device
+      bool on_device = false;
+      std::unique_ptr<mg::HostGroups> host;   // kept between a choice's sizes and its upload
     };
     std::map<int, Groups> groups;
   };
@@ -516,7 +520,7 @@ RowShape row_shape(const mg_mesh* M, int kind, int cols) {
 }
 
 // Chunk-major entries for the default shape of a kind, built on the device on
-// first use (before any graph capture).
+// first use (before any graph capture) where there is memory for them.
 int ensure_auto_entries(mg_mesh* M, int kind, int cols, cudaStream_t st) {
   const RowShape r = row_shape(M, kind, cols);
   const int chunk = mg::rows_lanes(cols, r.batch, kind == 2 ? r.most_cols : 512);
@@ -526,7 +530,8 @@ int ensure_auto_entries(mg_mesh* M, int kind, int cols, cudaStream_t st) {
   int w = 0;
   for (int32_t x : M->hm.slice_w) w = std::max(w, (int)x);
   const int64_t stride = (int64_t)(w + chunk - 1) / chunk * mg::kSliceH * chunk;
-  MG_TRY(ensure(b, (size_t)M->hm.n_slices * stride * sizeof(int2)));
+  if (ensure(b, (size_t)M->hm.n_slices * stride * sizeof(int2)) != MG_OK)
+    return MG_OK;   // no memory: the entries as they are
   M->launches += 1;
   return mg::launch_chunk_entries(dev_ell(M), chunk, stride, P<int2>(b), st);
 }
@@ -702,56 +707,83 @@ int persist_status(mg_mesh* M, cudaStream_t st) {
   return MG_ERR_TIMEOUT;
 }
 
-// Device tables of the partition into B patches with rpw rows per warp,
-// built on first use.
-int patch_tables(mg_mesh* M, int B, int rpw, mg::DevPatches& D) {
-  auto it = M->patches.find(B);
-  if (it == M->patches.end()) {
-    mg::HostPatches H;
-    MG_TRY(mg::build_patches(M->hm, B, H));
-    it = M->patches.emplace(B, mg_mesh::PatchTables()).first;
-    it->second.host = std::move(H);
+// Row groups of the partition into B patches with rpw rows per warp, built on
+// the host on first use: their sizes in R.dev.  MG_ERR_UNSUPPORTED (remembered)
+// when the mesh cannot be cut so, MG_ERR_OOM when the host's memory runs out.
+using PatchGroups = mg_mesh::PatchTables::Groups;
+int patch_groups(mg_mesh* M, int B, int rpw, PatchGroups*& out) {
+  try {
+    auto it = M->patches.find(B);
+    if (it == M->patches.end()) {
+      mg::HostPatches H;
+      const int rc = mg::build_patches(M->hm, B, H);
+      if (rc == MG_ERR_OOM) return rc;
+      if (rc != MG_OK) H = mg::HostPatches();
+      it = M->patches.emplace(B, mg_mesh::PatchTables()).first;
+      it->second.host = std::move(H);
+    }
+    mg_mesh::PatchTables& T = it->second;
+    if (!T.host.B) return MG_ERR_UNSUPPORTED;
+    auto ig = T.groups.find(rpw);
+    if (ig == T.groups.end() || (!ig->second.on_device && !ig->second.host)) {
+      std::unique_ptr<mg::HostGroups> G(new mg::HostGroups());
+      mg::group_rows(M->hm, T.host, rpw, *G);
+      PatchGroups& R = T.groups[rpw];
+      mg::DevPatches& d = R.dev;
+      d.B = B;
+      d.n_x = G->x_off[B];
+      d.max_pairs = G->max_pairs;
+      d.max_groups = G->max_groups;
+      d.uniform = G->uniform;
+      d.max_halo = G->max_halo;
+      d.max_slots = G->max_slots;
+      R.host = std::move(G);
+      ig = T.groups.find(rpw);
+    }
+    out = &ig->second;
+    return MG_OK;
+  } catch (const std::bad_alloc&) {
+    return MG_ERR_OOM;
   }
-  mg_mesh::PatchTables& T = it->second;
-  auto ig = T.groups.find(rpw);
-  if (ig == T.groups.end()) {
-    mg::HostGroups G;
-    mg::group_rows(M->hm, T.host, rpw, G);
-    mg_mesh::PatchTables::Groups& R = T.groups[rpw];
-    MG_TRY(upload(R.grp_off, G.grp_off));
-    MG_TRY(upload(R.border, G.border));
-    MG_TRY(upload(R.pair_off, G.pair_off));
-    MG_TRY(upload(R.halo_off, G.halo_off));
-    MG_TRY(upload(R.x_off, G.x_off));
-    MG_TRY(upload(R.hdr, G.hdr));
-    MG_TRY(upload(R.row, G.row));
-    MG_TRY(upload(R.halo, G.halo));
-    MG_TRY(upload(R.halo_x, G.halo_x));
-    MG_TRY(upload(R.diag, G.diag));
-    MG_TRY(upload(R.pair, G.pair));
-    mg::DevPatches& d = R.dev;
-    d.n_x = G.x_off[B];
-    d.max_pairs = G.max_pairs;
-    d.max_groups = G.max_groups;
-    d.uniform = G.uniform;
-    d.max_halo = G.max_halo;
-    d.max_slots = G.max_slots;
-    d.grp_off = P_<const int32_t>(R.grp_off);
-    d.border = P_<const int32_t>(R.border);
-    d.pair_off = P_<const int32_t>(R.pair_off);
-    d.halo_off = P_<const int32_t>(R.halo_off);
-    d.x_off = P_<const int32_t>(R.x_off);
-    d.hdr = P_<const int32_t>(R.hdr);
-    d.row = P_<const int32_t>(R.row);
-    d.halo = P_<const int32_t>(R.halo);
-    d.halo_x = P_<const int32_t>(R.halo_x);
-    d.diag = P_<const float>(R.diag);
-    d.pair = P_<const int4>(R.pair);
-    d.B = B;   // set last: the tables are complete
-    ig = T.groups.find(rpw);
+}
+
+// The groups' tables on the device, all of them or none.
+int upload_groups(PatchGroups& R) {
+  if (R.on_device) return MG_OK;
+  const mg::HostGroups& G = *R.host;
+  std::array<Buf, 11> b;
+  int k = 0, rc = MG_OK;
+  auto put = [&](const auto& v) {
+    Buf& x = b[k++];
+    if (rc == MG_OK) rc = upload(x, v);
+    return x.p;
+  };
+  mg::DevPatches d = R.dev;
+  d.grp_off = static_cast<const int32_t*>(put(G.grp_off));
+  d.border = static_cast<const int32_t*>(put(G.border));
+  d.pair_off = static_cast<const int32_t*>(put(G.pair_off));
+  d.halo_off = static_cast<const int32_t*>(put(G.halo_off));
+  d.x_off = static_cast<const int32_t*>(put(G.x_off));
+  d.hdr = static_cast<const int32_t*>(put(G.hdr));
+  d.row = static_cast<const int32_t*>(put(G.row));
+  d.halo = static_cast<const int32_t*>(put(G.halo));
+  d.halo_x = static_cast<const int32_t*>(put(G.halo_x));
+  d.diag = static_cast<const float*>(put(G.diag));
+  d.pair = static_cast<const int4*>(put(G.pair));
+  // a copy from pageable memory may still be under way when it returns: the
+  // caller's stream need not wait for the one that it ran on
+  if (rc == MG_OK && cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess) rc = MG_ERR_CUDA;
+  if (rc != MG_OK) {
+    cudaGetLastError();
+    for (Buf& x : b)
+      if (x.p) cudaFree(x.p);
+    return rc;
   }
-  D = ig->second.dev;
-  return D.B ? MG_OK : MG_ERR_OOM;
+  R.dev = d;
+  R.buf = b;
+  R.host.reset();
+  R.on_device = true;
+  return MG_OK;
 }
 
 // Estimates of a step's time on the two paths, in us, from measurements at 2, 8,
@@ -783,8 +815,8 @@ double rows_us(const mg_mesh* M, int kind, int S_pad) {
 // same with p and dp as columns (2 lpr shots per launch); adjoint: whole source
 // tiles of the row kernel only, for the same sums over the shots.
 // shape.lpr = 0: the row kernels are the path (nothing fits, they are estimated
-// to be faster, or the kind's path asks for them; MG_PATH_RESIDENT leaves the
-// estimate out).
+// to be faster, the kind's path asks for them, or there is no memory for the
+// tables, which they need none of; MG_PATH_RESIDENT leaves the estimate out).
 int resident_shape(mg_mesh* M, int kind, int S_pad, int steps, mg::DevPatches& D,
                    mg::ResidentShape& shape) {
   shape = mg::ResidentShape();
@@ -796,28 +828,37 @@ int resident_shape(mg_mesh* M, int kind, int S_pad, int steps, mg::DevPatches& D
   const int B = (int)std::min<int64_t>(M->n_sm, std::max<int64_t>(1, M->hm.n / 32));
   const int widest = kind == 1 ? std::min(32, S_pad / 2) : std::min(S_pad, 128) / 4;
   const int row_bytes = kind == 1 ? 8 : kind == 2 ? 16 : 0;
+  PatchGroups* R = nullptr;
   for (int lpr = widest; lpr >= (kind == 1 ? 2 : 1); lpr >>= 1) {
     // where rows and entries alone are too large no tables are needed to see it
     const int64_t rows = M->hm.n / B, entries = (M->hm.rowptr.back() - M->hm.n) / B;
     if (rows * (32 * lpr + 20 + row_bytes) + entries * 8 <= M->smem_optin) {
-      MG_TRY(patch_tables(M, B, 32 / lpr, D));
-      if (mg::resident_fit(D, lpr, row_bytes, M->smem_optin - 1024, shape) == MG_OK) break;
+      if (patch_groups(M, B, 32 / lpr, R) != MG_OK) return MG_OK;
+      if (mg::resident_fit(R->dev, lpr, row_bytes, M->smem_optin - 1024, shape) == MG_OK) break;
       shape = mg::ResidentShape();
+      R->host.reset();
     }
     if (kind == 2) break;
   }
-  if (shape.lpr && path == MG_PATH_AUTO &&
-      resident_us(D, shape, kind, S_pad) > rows_us(M, kind, S_pad))
+  if (!shape.lpr) return MG_OK;
+  if (path == MG_PATH_AUTO && resident_us(R->dev, shape, kind, S_pad) > rows_us(M, kind, S_pad)) {
     shape.lpr = 0;
-  return MG_OK;
+    R->host.reset();
+    return MG_OK;
+  }
+  const int rc = upload_groups(*R);
+  if (rc == MG_OK) D = R->dev;
+  else shape.lpr = 0;
+  return rc == MG_ERR_OOM ? MG_OK : rc;
 }
 
-// Exchange buffer and status word (cleared once per call) of resident launches.
+// Exchange buffer and status word (cleared once per call) of resident launches;
+// MG_ERR_UNSUPPORTED (the row kernels are the path) when there is no memory.
 template <class A>
 int resident_buffers(mg_mesh* M, const mg::DevPatches& D, int lpr, cudaStream_t st, A& r) {
-  MG_TRY(ensure(M->xbuf, (size_t)2 * D.n_x * lpr * 2 * sizeof(uint4)));
   r.status = err_word(M);
-  if (!r.status) return MG_ERR_OOM;
+  if (!r.status || ensure(M->xbuf, (size_t)2 * D.n_x * lpr * 2 * sizeof(uint4)) != MG_OK)
+    return MG_ERR_UNSUPPORTED;
   if (!M->status_clear) MG_CU(cudaMemsetAsync(r.status, 0, sizeof(int), st));
   M->status_clear = true;
   r.xbuf = P<uint4>(M->xbuf);
@@ -1216,12 +1257,9 @@ void mg_mesh_destroy(mg_mesh* M) {
       if (b->p) cudaFree(b->p);
   }
   for (auto& kv : M->patches) {
-    for (auto& g : kv.second.groups) {
-      mg_mesh::PatchTables::Groups& R = g.second;
-      for (Buf* b : {&R.grp_off, &R.border, &R.pair_off, &R.halo_off, &R.x_off, &R.hdr, &R.row,
-                     &R.halo, &R.halo_x, &R.diag, &R.pair})
-        if (b->p) cudaFree(b->p);
-    }
+    for (auto& g : kv.second.groups)
+      for (Buf& b : g.second.buf)
+        if (b.p) cudaFree(b.p);
   }
   mg_mesh_trim(M);
   if (M->cap) cudaStreamDestroy(M->cap);
@@ -2519,27 +2557,26 @@ int mesh_set_flux_geometry(mg_mesh* M, const std::vector<float>& cell,
                            const HostFluxPatches& H, FluxGeometry* g) {
   if (H.B) {
     DevFluxPatches D{};
-    int k = 0;
+    int k = 0, rc = MG_OK;
     auto put = [&](const std::vector<int32_t>& v, const int32_t*& to) {
       Buf& b = M->flux_tab[k++];
-      const int rc = upload(b, v);
+      if (rc == MG_OK) rc = upload(b, v);
       to = P<const int32_t>(b);
-      return rc;
     };
-    MG_TRY(put(H.own_off, D.own_off));
-    MG_TRY(put(H.border, D.border));
-    MG_TRY(put(H.halo_off, D.halo_off));
-    MG_TRY(put(H.x_off, D.x_off));
-    MG_TRY(put(H.cell_off, D.cell_off));
-    MG_TRY(put(H.inner, D.inner));
-    MG_TRY(put(H.inc_off, D.inc_off));
-    MG_TRY(put(H.row, D.row));
-    MG_TRY(put(H.row_inc, D.row_inc));
-    MG_TRY(put(H.halo, D.halo));
-    MG_TRY(put(H.halo_x, D.halo_x));
-    MG_TRY(put(H.cell, D.cell));
-    MG_TRY(put(H.cell_slot, D.cell_slot));
-    MG_TRY(upload(M->flux_pinc, H.inc));
+    put(H.own_off, D.own_off);
+    put(H.border, D.border);
+    put(H.halo_off, D.halo_off);
+    put(H.x_off, D.x_off);
+    put(H.cell_off, D.cell_off);
+    put(H.inner, D.inner);
+    put(H.inc_off, D.inc_off);
+    put(H.row, D.row);
+    put(H.row_inc, D.row_inc);
+    put(H.halo, D.halo);
+    put(H.halo_x, D.halo_x);
+    put(H.cell, D.cell);
+    put(H.cell_slot, D.cell_slot);
+    if (rc == MG_OK) rc = upload(M->flux_pinc, H.inc);
     D.inc = P<const int4>(M->flux_pinc);
     D.n_x = H.x_off[H.B];
     D.max_own = H.max_own;
@@ -2548,11 +2585,22 @@ int mesh_set_flux_geometry(mg_mesh* M, const std::vector<float>& cell,
     D.max_cells = H.max_cells;
     D.max_inc = H.max_inc;
     D.B = H.B;
-    M->flux_patches = D;
+    if (rc == MG_OK) {
+      M->flux_patches = D;
+    } else {   // no memory for them: launches per step
+      for (Buf* b = M->flux_tab.data(); b != M->flux_tab.data() + M->flux_tab.size(); ++b) {
+        if (b->p) cudaFree(b->p);
+        *b = Buf{};
+      }
+      if (M->flux_pinc.p) cudaFree(M->flux_pinc.p);
+      M->flux_pinc = Buf{};
+      if (rc != MG_ERR_OOM) return rc;
+    }
   }
   MG_TRY(upload(M->flux_cell, cell));
   MG_TRY(upload(M->flux_ptr, ptr));
   MG_TRY(upload(M->flux_inc, inc));   // last: its presence marks the set
+  MG_CU(cudaStreamSynchronize(cudaStreamLegacy));   // as in upload_groups
   mesh_flux_geometry(M, g);
   return MG_OK;
 }

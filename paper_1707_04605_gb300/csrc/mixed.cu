@@ -30,6 +30,7 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <new>
 #include <vector>
 
 #include "../../include/mgwave.h"
@@ -665,8 +666,13 @@ int flux_geometry(mg_mesh* M, const HostMesh& hm, FluxGeometry& out) {
   const int B = (int)std::min<int64_t>(n_sm, std::max<int64_t>(1, n / 32));
   HostFluxPatches H;
   if (((n + m * d) * 16 + m * 36 + (int64_t)inc.size() * 12) / B < smem) {
-    const int rc = build_flux_patches(hm, B, inc, H);
-    if (rc == MG_ERR_UNSUPPORTED) H = HostFluxPatches();
+    int rc;
+    try {
+      rc = build_flux_patches(hm, B, inc, H);
+    } catch (const std::bad_alloc&) {
+      rc = MG_ERR_OOM;
+    }
+    if (rc == MG_ERR_UNSUPPORTED || rc == MG_ERR_OOM) H = HostFluxPatches();   // no patches
     else if (rc != MG_OK) return rc;
   }
   return mesh_set_flux_geometry(M, cell, ptr, inc, H, &out);
@@ -824,7 +830,11 @@ int flux_path(mg_mesh* M, int steps, Scratch& X, Flux& F, bool reverse = false) 
   a.budget = mesh_wait_budget(M);
   a.xbuf = X.get<uint4>((size_t)2 * a.P.n_x * std::max(F.shape.lpr, F.rshape.lpr) * 2);
   a.status = X.get<int>(1);
-  if (!a.xbuf || !a.status) return MG_ERR_OOM;
+  if (!a.xbuf || !a.status) {   // no memory: launches per step
+    F.shape.lpr = F.rshape.lpr = 0;
+    a.status = nullptr;
+    return MG_OK;
+  }
   return cudaMemsetAsync(a.status, 0, sizeof(int), F.st) == cudaSuccess ? MG_OK : MG_ERR_CUDA;
 }
 

@@ -19,7 +19,8 @@ namespace mg {
 // pages of which a patch touches few.
 struct Stamps {
   int32_t* p;
-  explicit Stamps(int64_t n) : p(static_cast<int32_t*>(std::calloc(n, sizeof(int32_t)))) {
+  explicit Stamps(int64_t n) : p(static_cast<int32_t*>(std::calloc(n, sizeof(int32_t)))) {}
+  void need() const {
     if (!p) throw std::bad_alloc();
   }
   ~Stamps() { std::free(p); }
@@ -27,6 +28,17 @@ struct Stamps {
   Stamps& operator=(const Stamps&) = delete;
   int32_t& operator[](int64_t i) { return p[i]; }
 };
+
+// Runs one iteration of a parallel loop, which no exception may leave: memory
+// that it does not get is counted.
+template <class F>
+void no_throw(int& oom, F&& body) {
+  try {
+    body();
+  } catch (const std::bad_alloc&) {
+    ++oom;
+  }
+}
 
 // Rows cut into B patches: a patch's border rows (coupled to rows of other
 // patches) first, then its inner rows.
@@ -38,7 +50,8 @@ struct HostPatches {
   std::vector<int32_t> row;
   std::vector<std::vector<int32_t>> halo;   // per patch: rows of others that it reads
 };
-// MG_ERR_UNSUPPORTED when the coupling of two patches is not mutual.
+// MG_ERR_UNSUPPORTED when the coupling of two patches is not mutual, MG_ERR_OOM
+// when the host's memory runs out.
 int build_patches(const HostMesh& hm, int B, HostPatches& out);
 
 // The rows in groups of rpw that a warp advances together (rpw = 32 / lanes

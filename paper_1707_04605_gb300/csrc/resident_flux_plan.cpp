@@ -29,12 +29,13 @@ int build_flux_patches(const HostMesh& hm, int B, const std::vector<int4>& geo_i
       if (s < P.n_border[b]) xrow[P.row[i]] = F.x_off[b] + s;
     }
   }
-  int bad = 0;
-#pragma omp parallel reduction(+ : bad)
+  int bad = 0, oom = 0;
+#pragma omp parallel reduction(+ : oom)
   {
     Stamps seen(hm.m);
 #pragma omp for schedule(dynamic, 4)
-    for (int b = 0; b < B; ++b) {
+    for (int b = 0; b < B; ++b) no_throw(oom, [&] {
+      seen.need();
       std::vector<int32_t>& c = cells[b];
       for (int i = P.own_off[b]; i < P.own_off[b + 1]; ++i)
         for (int64_t q = hm.nc_ptr[P.row[i]]; q < hm.nc_ptr[P.row[i] + 1]; ++q) {
@@ -48,8 +49,9 @@ int build_flux_patches(const HostMesh& hm, int B, const std::vector<int4>& geo_i
         return true;
       };
       F.inner[b] = (int)(std::stable_partition(c.begin(), c.end(), inner) - c.begin());
-    }
+    });
   }
+  if (oom) return MG_ERR_OOM;
   for (int b = 0; b < B; ++b) {
     int inc = 0;
     for (int i = P.own_off[b]; i < P.own_off[b + 1]; ++i)
@@ -70,11 +72,13 @@ int build_flux_patches(const HostMesh& hm, int B, const std::vector<int4>& geo_i
   F.cell.resize(F.cell_off[B]);
   F.cell_slot.assign((size_t)F.cell_off[B] * 4, 0);
   F.inc.resize(F.inc_off[B]);
-#pragma omp parallel reduction(+ : bad)
+#pragma omp parallel reduction(+ : bad, oom)
   {
     Stamps at(hm.m), halo(hm.n);   // place of a cell, slot of a halo row, plus 1
 #pragma omp for schedule(dynamic, 4)
-    for (int b = 0; b < B; ++b) {
+    for (int b = 0; b < B; ++b) no_throw(oom, [&] {
+      at.need();
+      halo.need();
       const std::vector<int32_t>&c = cells[b], &h = P.halo[b];
       const int own = P.own_off[b + 1] - P.own_off[b];
       for (size_t i = 0; i < h.size(); ++i) {
@@ -107,9 +111,9 @@ int build_flux_patches(const HostMesh& hm, int B, const std::vector<int4>& geo_i
       }
       for (int32_t r : h) halo[r] = 0;
       for (int32_t e : c) at[e] = 0;
-    }
+    });
   }
-  return bad ? MG_ERR_UNSUPPORTED : MG_OK;
+  return oom ? MG_ERR_OOM : bad ? MG_ERR_UNSUPPORTED : MG_OK;
 }
 
 }  // namespace mg

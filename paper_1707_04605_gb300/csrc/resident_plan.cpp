@@ -80,11 +80,14 @@ int build_patches(const HostMesh& hm, int B, HostPatches& P) {
   std::vector<uint8_t> border(n, 0);
   P.halo.resize(B);
   std::vector<std::vector<int32_t>> reads(B);   // patches that a patch reads
-#pragma omp parallel
+  int oom = 0;
+#pragma omp parallel reduction(+ : oom)
   {
     Stamps row(n), other(B);   // halo rows and patches seen
 #pragma omp for schedule(dynamic, 4)
-    for (int b = 0; b < B; ++b) {
+    for (int b = 0; b < B; ++b) no_throw(oom, [&] {
+      row.need();
+      other.need();
       for (int i = P.own_off[b]; i < P.own_off[b + 1]; ++i)
         for (int64_t q = hm.rowptr[P.row[i]]; q < hm.rowptr[P.row[i] + 1]; ++q) {
           const int32_t c = hm.col[q], o = part[c];
@@ -98,8 +101,9 @@ int build_patches(const HostMesh& hm, int B, HostPatches& P) {
       for (int32_t o : reads[b]) other[o] = 0;
       std::sort(P.halo[b].begin(), P.halo[b].end());
       std::sort(reads[b].begin(), reads[b].end());
-    }
+    });
   }
+  if (oom) return MG_ERR_OOM;
   for (int b = 0; b < B; ++b) {
     for (int32_t o : reads[b])
       if (!std::binary_search(reads[o].begin(), reads[o].end(), b)) return MG_ERR_UNSUPPORTED;

@@ -296,3 +296,72 @@ def test_a_reconstruction_whose_waits_run_out_is_an_error(mg):
     assert e.value.code == L.MG_ERR_TIMEOUT
     m.set_persistent()
     assert torch.equal(run()[0], x0)
+
+
+class _FullMemory:
+    """Takes the device memory that is left, down to blocks of 1 MiB."""
+
+    def __enter__(self):
+        import ctypes as C
+
+        self.cu = C.CDLL("libcuda.so.1")
+        self.cu.cuMemAlloc_v2.argtypes = [C.c_void_p, C.c_size_t]
+        self.cu.cuMemFree_v2.argtypes = [C.c_uint64]
+        torch.cuda.synchronize()
+        self.blocks = []
+        size = 1 << 37
+        while size >= 1 << 20:
+            p = C.c_uint64()
+            if self.cu.cuMemAlloc_v2(C.byref(p), size) == 0:
+                self.blocks.append(p.value)
+            else:
+                size >>= 1
+        return self
+
+    def __exit__(self, *exc):
+        torch.cuda.synchronize()
+        for p in self.blocks:
+            self.cu.cuMemFree_v2(p)
+
+
+@pytest.mark.parametrize("S,before", [(8, "rows"), (32, "shape")])
+def test_tables_without_memory_leave_the_row_kernels(mg, S, before):
+    """Patch tables (and, with 32 shots, the default shape's entries) that find no
+    device memory: the row kernels run instead, the same bits, and the resident
+    kernels once there is memory again."""
+    w = configs.asteroid_2d(n_refine=3, S=S, nt=60)
+    m = mg.mesh_from_workload(w)
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    s = _dev(w.wavelet(dt))
+    rng = np.random.default_rng(9)
+    v = _dev(rng.standard_normal(w.mesh.n_cells[1]))
+    W = _dev(rng.standard_normal((w.shots.n_traces, w.nt)), torch.float32)
+
+    def run():
+        n0 = m.launch_count()
+        out = (mg.forward(m, eps, w.shots, s, dt), mg.jacobian_apply(m, 1, eps, w.shots, s, dt, v),
+               mg.jacobian_T_apply(m, 1, eps, w.shots, s, dt, W, ckpt_every=21))
+        return m.launch_count() - n0, out
+
+    m.set_kernel_path(before)        # every other buffer and kernel of the calls
+    ref = run()[1]
+    run()
+    if before == "shape":            # the kernels of the default shape, without its entries
+        other = mg.mesh_from_workload(w)
+        other.set_kernel_path("rows")
+        mg.forward(other, eps, w.shots, s, dt)
+        other.close()
+        m.set_tuning(-1, 2, 0, 32)
+        m.set_min_blocks(5)
+        m.set_min_blocks(5, "adjoint")
+        m.set_kernel_tuning("tangent", 1, 0, 32)
+        m.set_min_blocks(5, "tangent")
+        run()
+    m.set_kernel_path("auto")
+    spare = [x.clone() for x in ref]  # cached blocks for the results
+    del spare
+    with _FullMemory():
+        n, out = run()
+    assert n > 5 * w.nt and all(torch.equal(x, y) for x, y in zip(out, ref))
+    n, out = run()
+    assert n < 2 * w.nt and all(torch.equal(x, y) for x, y in zip(out, ref))
