@@ -390,9 +390,11 @@ __global__ void k_flux_cell_grad(int64_t m, int k1, const int32_t* __restrict__ 
 // Work buffers of a call, left on the handle for the next one (in the order of
 // use, so the same call finds its sizes again).  A call takes them away from
 // the handle while it runs: a second thread's call finds none and allocates
-// its own.  More than kKeepBytes, or a second set, is freed at the end.  The
-// calls end with a stream synchronisation, on errors in the destructor: the
-// next call may use another stream.
+// its own.  More than kKeepBytes, or a second set, is freed at the end.
+// Allocated and freed in the order of the call's stream: cudaMalloc and cudaFree
+// wait for the whole device, other streams and handles included.  The calls end
+// with a synchronisation of their stream, on errors in the destructor: the next
+// call may use another one.
 constexpr size_t kKeepBytes = (size_t)2 << 30;
 struct Scratch {
   mg_mesh* M;
@@ -405,7 +407,8 @@ struct Scratch {
     size_t total = 0;
     for (const FluxBuffer& b : own) total += b.bytes;
     if (total > kKeepBytes || !mesh_keep_scratch(M, own))
-      for (const FluxBuffer& b : own) cudaFree(b.p);
+      for (const FluxBuffer& b : own)
+        if (b.p) cudaFreeAsync(b.p, st);
   }
   Scratch(const Scratch&) = delete;
   Scratch& operator=(const Scratch&) = delete;
@@ -415,9 +418,9 @@ struct Scratch {
     if (next == own.size()) own.push_back({nullptr, 0});
     FluxBuffer& b = own[next++];
     if (b.bytes < bytes) {
-      cudaFree(b.p);
+      if (b.p) cudaFreeAsync(b.p, st);
       b = {nullptr, 0};
-      if (cudaMalloc(&b.p, bytes) != cudaSuccess) {
+      if (cudaMallocAsync(&b.p, bytes, st) != cudaSuccess) {
         cudaGetLastError();
         b.p = nullptr;
         return nullptr;

@@ -75,3 +75,30 @@ def test_a_flux_wait_that_runs_out_raises(mg):
         mg.forward_pml(mesh, eps, w.shots, wav, dt)
     mesh.set_persistent()
     assert mg.forward_pml(mesh, eps, w.shots, wav, dt).equal(y)
+
+
+def test_a_large_call_does_not_wait_for_other_streams(mg):
+    """Work buffers above what a handle keeps (2 GB) are allocated and freed in the
+    order of the call's own stream (launches per step: they need no SM to
+    themselves)."""
+    import torch
+
+    w = configs.asteroid_2d(n_refine=4, S=256, nt=6)
+    m = mg.mesh_from_workload(w)
+    eps = cu(w.eps)
+    dt = 0.5 * mg.cfl_dt(m, eps)
+    s = cu(w.wavelet(dt))
+    v = cu(np.ones(w.mesh.n_cells[0]))
+    run = lambda: mg.jacobian_apply_pml(m, 0, eps, w.shots, s, dt, v)
+    ref = run()
+    n, cells = w.mesh.coords.shape[0], len(w.mesh.cells)
+    assert 4 * 256 * (2 * n + 4 * cells) > 2 << 30   # p, dp, q and dq
+    side, done = torch.cuda.Stream(), torch.cuda.Event()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(3_000_000_000)             # more than a second
+        done.record()
+    jv = run()
+    assert not done.query()
+    assert torch.equal(jv, ref)
+    torch.cuda.synchronize()
