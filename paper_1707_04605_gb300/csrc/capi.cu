@@ -1665,6 +1665,9 @@ int mg_mesh_get_info(const mg_mesh* M, mg_mesh_info_t* info) {
   for (const Buf* b : all) bytes += (int64_t)b->bytes;
   for (const auto& kv : M->auto_ellc) bytes += (int64_t)kv.second.bytes;
   for (const Buf& b : M->flux_tab) bytes += (int64_t)b.bytes;
+  for (const auto& kv : M->patches)
+    for (const auto& g : kv.second.groups)
+      for (const Buf& b : g.second.buf) bytes += (int64_t)b.bytes;
   for (const mg::FluxBuffer& b : M->flux_scratch) bytes += (int64_t)b.bytes;
   info->device_bytes = bytes;
   return MG_OK;

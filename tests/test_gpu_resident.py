@@ -365,3 +365,17 @@ def test_tables_without_memory_leave_the_row_kernels(mg, S, before):
     assert n > 5 * w.nt and all(torch.equal(x, y) for x, y in zip(out, ref))
     n, out = run()
     assert n < 2 * w.nt and all(torch.equal(x, y) for x, y in zip(out, ref))
+
+
+def test_device_bytes_count_the_patch_tables(mg):
+    """What stays on the handle after a resident call and mg_mesh_trim: at least a
+    pair of slots and values per two entries, and a row number and a diagonal
+    entry per row."""
+    w = configs.asteroid_2d(n_refine=3, S=8, nt=40)
+    m = mg.mesh_from_workload(w)
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    before = m.info()
+    mg.forward(m, eps, w.shots, _dev(w.wavelet(dt)), dt)
+    m.trim()
+    added = m.info()["device_bytes"] - before["device_bytes"]
+    assert added >= 8 * (before["nnz"] - before["n_nodes"]) + 8 * before["n_nodes"]
