@@ -160,7 +160,7 @@ struct mg_mesh {
       std::array<Buf, 11> buf;
       mg::DevPatches dev{};               // sizes; the pointers once on_device
       bool on_device = false;
-      std::unique_ptr<mg::HostGroups> host;   // kept between a choice's sizes and its upload
+      std::unique_ptr<mg::HostGroups> host;   // until uploaded, where the choice took them
     };
     std::map<int, Groups> groups;
   };
@@ -708,10 +708,11 @@ int persist_status(mg_mesh* M, cudaStream_t st) {
 }
 
 // Row groups of the partition into B patches with rpw rows per warp, built on
-// the host on first use: their sizes in R.dev.  MG_ERR_UNSUPPORTED (remembered)
-// when the mesh cannot be cut so, MG_ERR_OOM when the host's memory runs out.
+// the host on first use: their sizes (kept) and, when asked for, their tables on
+// the host or the device.  MG_ERR_UNSUPPORTED (remembered) when the mesh cannot
+// be cut so, MG_ERR_OOM when the host's memory runs out.
 using PatchGroups = mg_mesh::PatchTables::Groups;
-int patch_groups(mg_mesh* M, int B, int rpw, PatchGroups*& out) {
+int patch_groups(mg_mesh* M, int B, int rpw, bool tables, PatchGroups*& out) {
   try {
     auto it = M->patches.find(B);
     if (it == M->patches.end()) {
@@ -725,7 +726,7 @@ int patch_groups(mg_mesh* M, int B, int rpw, PatchGroups*& out) {
     mg_mesh::PatchTables& T = it->second;
     if (!T.host.B) return MG_ERR_UNSUPPORTED;
     auto ig = T.groups.find(rpw);
-    if (ig == T.groups.end() || (!ig->second.on_device && !ig->second.host)) {
+    if (ig == T.groups.end() || (tables && !ig->second.on_device && !ig->second.host)) {
       std::unique_ptr<mg::HostGroups> G(new mg::HostGroups());
       mg::group_rows(M->hm, T.host, rpw, *G);
       PatchGroups& R = T.groups[rpw];
@@ -833,7 +834,7 @@ int resident_shape(mg_mesh* M, int kind, int S_pad, int steps, mg::DevPatches& D
     // where rows and entries alone are too large no tables are needed to see it
     const int64_t rows = M->hm.n / B, entries = (M->hm.rowptr.back() - M->hm.n) / B;
     if (rows * (32 * lpr + 20 + row_bytes) + entries * 8 <= M->smem_optin) {
-      if (patch_groups(M, B, 32 / lpr, R) != MG_OK) return MG_OK;
+      if (patch_groups(M, B, 32 / lpr, false, R) != MG_OK) return MG_OK;
       if (mg::resident_fit(R->dev, lpr, row_bytes, M->smem_optin - 1024, shape) == MG_OK) break;
       shape = mg::ResidentShape();
       R->host.reset();
@@ -846,7 +847,8 @@ int resident_shape(mg_mesh* M, int kind, int S_pad, int steps, mg::DevPatches& D
     R->host.reset();
     return MG_OK;
   }
-  const int rc = upload_groups(*R);
+  int rc = patch_groups(M, B, 32 / shape.lpr, true, R);
+  if (rc == MG_OK) rc = upload_groups(*R);
   if (rc == MG_OK) D = R->dev;
   else shape.lpr = 0;
   return rc == MG_ERR_OOM ? MG_OK : rc;

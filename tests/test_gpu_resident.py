@@ -303,7 +303,10 @@ class _FullMemory:
 
     def __enter__(self):
         import ctypes as C
+        import gc
 
+        gc.collect()                     # no handle of an earlier test is freed inside
+        gc.disable()
         self.cu = C.CDLL("libcuda.so.1")
         self.cu.cuMemAlloc_v2.argtypes = [C.c_void_p, C.c_size_t]
         self.cu.cuMemFree_v2.argtypes = [C.c_uint64]
@@ -319,6 +322,9 @@ class _FullMemory:
         return self
 
     def __exit__(self, *exc):
+        import gc
+
+        gc.enable()
         torch.cuda.synchronize()
         for p in self.blocks:
             self.cu.cuMemFree_v2(p)
@@ -365,6 +371,32 @@ def test_tables_without_memory_leave_the_row_kernels(mg, S, before):
     assert n > 5 * w.nt and all(torch.equal(x, y) for x, y in zip(out, ref))
     n, out = run()
     assert n < 2 * w.nt and all(torch.equal(x, y) for x, y in zip(out, ref))
+
+
+def test_a_choice_of_the_row_kernels_is_not_planned_anew(mg):
+    """A mesh whose patches fit but whose estimate prefers the row kernels: repeated
+    calls do not build the patches' host tables again (more than a ms on a mesh of
+    this size; the call itself takes two)."""
+    import time
+
+    w = configs.asteroid_2d(n_refine=4, S=64, nt=16)
+    m = mg.mesh_from_workload(w)
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    s = _dev(w.wavelet(dt))
+
+    def run(path):
+        m.set_kernel_path(path)
+        times = []
+        for _ in range(8):
+            t0 = time.perf_counter()
+            mg.jacobian_apply(m, 0, eps, w.shots, s, dt, v)
+            torch.cuda.synchronize()
+            times.append(time.perf_counter() - t0)
+        return min(times)
+
+    v = _dev(np.ones(w.mesh.n_cells[0]))
+    rows, auto = run("rows"), run("auto")
+    assert auto < 1.3 * rows
 
 
 def test_device_bytes_count_the_patch_tables(mg):
