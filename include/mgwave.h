@@ -314,8 +314,10 @@ int mg_mesh_set_kernel_tuning(mg_mesh* mesh, int kind, int batch, int tile_rows,
  *  MG_PATH_AUTO      the resident kernel or the row kernels in the library's
  *                    own launch shape, by an estimate of both (default)
  *  MG_PATH_SHAPE     the launch shape on the handle
- *  MG_PATH_RESIDENT  the resident kernel wherever it can run (mg_forward),
- *                    the launch shape on the handle elsewhere
+ *  MG_PATH_RESIDENT  the resident kernel wherever it can run (mg_forward; for
+ *                    steps that write a history, J^T's recompute among them,
+ *                    where the estimate prefers it), the launch shape on the
+ *                    handle elsewhere
  *  MG_PATH_ROWS      the row kernels in the library's own launch shape
  * Setting a launch shape selects MG_PATH_SHAPE: a batch, tile or source width
  * always, a number of shot groups, a register cap, ring, sweep, tiles or bulk

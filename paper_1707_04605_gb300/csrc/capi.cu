@@ -787,27 +787,50 @@ int upload_groups(PatchGroups& R) {
   return MG_OK;
 }
 
-// Estimates of a step's time on the two paths, in us, from measurements at 2, 8,
-// 16, 64, 128 and 256 columns on triangles (3,997 to 249,697 nodes) and
-// tetrahedra (30,525), most within 15% of them.  Resident: a launch per column
-// group, each the exchange of border rows, the patch's shared memory accesses
-// (a row read by fewer than 8 lanes conflicts with others) and its halo's.  Row
-// kernels: launch and tail, then the gathers, or the states' traffic when they
-// exceed L2.
-double resident_us(const mg::DevPatches& D, const mg::ResidentShape& s, int kind, int S_pad) {
-  const double conflicts = s.lpr >= 8 ? 1.0 : s.lpr == 4 ? 1.5 : s.lpr == 2 ? 2.4 : 1.6;
+// Estimates of a step's time on the two paths, in us, from measurements at 2 to
+// 256 columns on triangles (3,997 to 249,697 nodes) and tetrahedra (30,525), most
+// within 15% of them.  Resident: a launch per column group, each the exchange of
+// border rows, the patch's shared memory accesses (a row read by fewer than 8
+// lanes conflicts with others, less so on triangles, whose neighbours lie side by
+// side) and its halo's.  Row kernels: launch and tail, then the gathers, or the
+// states' traffic when they exceed L2.
+//
+// hist: a step's states also go to a history, `mb` MB of them.  The row kernels
+// write them in whole rows.  A resident launch writes the columns of its group,
+// and its other columns of the same sectors come launches later, when these have
+// left L2: less than 128 bytes a row cost their sectors again, 16 bytes (one
+// lane) a sector each, more so the more launches there are.  Measured, us per
+// step without and with history: 249,697 nodes x 256 shots (one lane, 64
+// launches) 185 and 494 to 625, with row kernels 163 and 181; 197,377 x 256
+// (two lanes) 111 and 168, row kernels 130 and 144; 151,201 x 256 (four) 76 and
+// 99, 100 and 111; 62,641 x 256 (eight) 28.5 and 33, 43 and 48.
+double history_us(int lanes, int launches, double mb) {
+  const double per_mb = launches == 1 ? 0.1 : lanes >= 8 ? 0.07 : lanes == 4 ? 0.15
+                        : lanes == 2 ? 0.27 : std::min(1.7, 0.08 * launches);
+  return per_mb * mb;
+}
+double resident_us(const mg::DevPatches& D, const mg::ResidentShape& s, int kind, int S_pad,
+                   double mb) {
+  const bool tri = D.uniform == 3;
+  const double conflicts = s.lpr >= 8   ? 1.0
+                           : s.lpr == 4 ? (tri ? 1.15 : 1.5)
+                           : s.lpr == 2 ? (tri ? 1.15 : 2.4)
+                                        : 1.6;
   const double pairs = (double)D.max_pairs / (D.max_groups * (32 / s.lpr));
   const double group = 14.0 + pairs * (1.0 + 8.0 * conflicts) + (kind == 1 ? 6.0 : kind == 2 ? 12.0 : 0.0);
   const int launches = S_pad / (kind == 1 ? 2 * s.lpr : 4 * s.lpr);
-  return launches * (0.9 + 0.65e-3 * group * D.max_groups + 0.3e-3 * D.max_halo * 2 * s.lpr);
+  return launches * (0.9 + 0.65e-3 * group * D.max_groups + 0.3e-3 * D.max_halo * 2 * s.lpr) +
+         history_us(kind == 1 ? s.lpr / 2 : s.lpr, launches, mb);
 }
-double rows_us(const mg_mesh* M, int kind, int S_pad) {
+double rows_us(const mg_mesh* M, int kind, int S_pad, double mb) {
   const double work = (double)M->hm.rowptr.back() * S_pad, cols = (double)M->hm.n * S_pad;
   const double gathers = 4.0 + (kind == 0 ? 0.27e-6 : kind == 1 ? 0.5e-6 : 0.38e-6) * work;
   const double held = (kind == 1 ? 16.0 : 8.0) * cols;   // bytes of the states of a step
   const double moved = (kind == 0 ? 12.0 : kind == 1 ? 24.0 : 16.0) * cols;
-  if (held < 100e6) return gathers;
-  return std::max(gathers, moved / (held < 200e6 ? 3.9e6 : 3.4e6));
+  const double hist = (kind == 0 ? 0.07 : 0.01) * mb;
+  if (held < (kind == 1 ? 80e6 : 100e6)) return gathers + hist;
+  const double rate = kind == 1 ? (held < 200e6 ? 3.8e6 : 4.2e6) : held < 150e6 ? 4.1e6 : 4.5e6;
+  return std::max(gathers, moved / rate) + hist;
 }
 
 // Resident launch shape of a call that advances S_pad columns for `steps`
@@ -817,9 +840,10 @@ double rows_us(const mg_mesh* M, int kind, int S_pad) {
 // tiles of the row kernel only, for the same sums over the shots.
 // shape.lpr = 0: the row kernels are the path (nothing fits, they are estimated
 // to be faster, the kind's path asks for them, or there is no memory for the
-// tables, which they need none of; MG_PATH_RESIDENT leaves the estimate out).
+// tables, which they need none of; MG_PATH_RESIDENT leaves the estimate out,
+// but for calls that write a history).
 int resident_shape(mg_mesh* M, int kind, int S_pad, int steps, mg::DevPatches& D,
-                   mg::ResidentShape& shape) {
+                   mg::ResidentShape& shape, bool hist = false) {
   shape = mg::ResidentShape();
   const int path = M->tune[kind].path;
   if (path == MG_PATH_SHAPE || path == MG_PATH_ROWS || steps < 16 || M->hm.max_row_nnz > 256)
@@ -842,7 +866,9 @@ int resident_shape(mg_mesh* M, int kind, int S_pad, int steps, mg::DevPatches& D
     if (kind == 2) break;
   }
   if (!shape.lpr) return MG_OK;
-  if (path == MG_PATH_AUTO && resident_us(R->dev, shape, kind, S_pad) > rows_us(M, kind, S_pad)) {
+  const double mb = hist ? 4e-6 * (double)M->hm.n * S_pad : 0.0;
+  if ((path == MG_PATH_AUTO || hist) &&
+      resident_us(R->dev, shape, kind, S_pad, mb) > rows_us(M, kind, S_pad, mb)) {
     shape.lpr = 0;
     R->host.reset();
     return MG_OK;
@@ -1088,7 +1114,7 @@ int run_forward_states(mg_mesh* M, const Prep& pp, int nt, float* traces, float*
   const size_t state = (size_t)M->hm.n * pp.S_pad;
   mg::DevPatches D;
   mg::ResidentShape shape;
-  MG_TRY(resident_shape(M, 0, pp.S_pad, nt, D, shape));
+  MG_TRY(resident_shape(M, 0, pp.S_pad, nt, D, shape, true));
   if (shape.lpr) {
     const int rc = run_forward_resident(M, pp, nt, traces, 0, nullptr, seg, D, shape, st);
     if (rc != MG_ERR_UNSUPPORTED) return rc;
@@ -1971,7 +1997,7 @@ int mg_forward_jacobian_apply(mg_mesh* M, int level, const double* eps, const mg
   if (!(flags & MG_PERSISTENT)) {
     mg::DevPatches D;
     mg::ResidentShape shape;
-    MG_TRY(resident_shape(M, 1, pp.S_pad, nt, D, shape));
+    MG_TRY(resident_shape(M, 1, pp.S_pad, nt, D, shape, keep));
     if (shape.lpr) {
       const int rc = run_tangent_resident(M, pp, nt, trf, tr, keep ? seg + 2 * state : nullptr, D,
                                           shape, st);
@@ -2132,7 +2158,7 @@ int mg_jacobian_T_apply(mg_mesh* M, int level, const double* eps, const mg_shots
   mg::DevPatches Df, Da;
   mg::ResidentShape shf, sha;
   if (!(flags & MG_PERSISTENT)) {
-    MG_TRY(resident_shape(M, 0, pp.S_pad, std::min(ckpt_every, nt), Df, shf));
+    MG_TRY(resident_shape(M, 0, pp.S_pad, std::min(ckpt_every, nt), Df, shf, true));
     MG_TRY(resident_shape(M, 2, pp.S_pad, std::min(ckpt_every, nt), Da, sha));
   }
   // accumulators: one set per source tile of the untiled kernel; the tiled

@@ -411,3 +411,27 @@ def test_device_bytes_count_the_patch_tables(mg):
     m.trim()
     added = m.info()["device_bytes"] - before["device_bytes"]
     assert added >= 8 * (before["nnz"] - before["n_nodes"]) + 8 * before["n_nodes"]
+
+
+def test_narrow_history_writes_stay_with_the_row_kernels(mg):
+    """249,697 nodes hold one lane (4 shots) per row: a resident launch would write
+    a history in 16-byte pieces, so calls that keep one, and J^T's recompute, run
+    row kernels; the plain forward of few shots does not.  The same bits."""
+    w = configs.asteroid_2d(n_refine=4, S=64, nt=32)
+    a, b = _pair(mg, w)
+    a.set_kernel_path("resident", "forward")
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    s = _dev(w.wavelet(dt))
+    W = _dev(np.random.default_rng(10).standard_normal((w.shots.n_traces, w.nt)), torch.float32)
+    calls = [lambda m: mg.forward(m, eps, w.shots, s, dt),
+             lambda m: mg.forward(m, eps, w.shots, s, dt, keep_states=True),
+             lambda m: mg.jacobian_T_apply(m, 0, eps, w.shots, s, dt, W, ckpt_every=32)]
+    n = []
+    for call in calls:
+        n0 = a.launch_count()
+        x = call(a)
+        n.append(a.launch_count() - n0)
+        assert torch.equal(x, call(b))
+    assert n[0] < w.nt                  # resident: 16 launches
+    assert n[1] >= w.nt                 # a launch per step
+    assert n[2] >= 2.5 * w.nt           # recompute and reverse steps, 16 for the forward
