@@ -565,8 +565,11 @@ int mg_mesh_get_tuning(const mg_mesh* mesh, int32_t* out);
  * mg_mesh_get_gather_ring); for the forward the row kernels with 1 vector
  * per lane, and with 2 and 4 under the register cap, sweeping 4 row blocks
  * per CTA (mg_mesh_get_row_sweep); then 2, 4 and 8 shot groups on the two
- * fastest of those; and, where patches fit, the resident kernel of the kind
- * (when it wins, chosen[] still holds the fastest of the others).  The handle's L1 streaming, prefetch, wide-lane and
+ * fastest of those; the library's own row shape; and, wherever patches fit, the
+ * resident kernel of the kind.  When one of the last two wins, the kind's path
+ * (mg_mesh_get_kernel_path) is MG_PATH_ROWS or MG_PATH_RESIDENT, or MG_PATH_AUTO
+ * where that chooses the winner by itself, and chosen[] holds the fastest of the
+ * launch shapes.  The handle's L1 streaming, prefetch, wide-lane and
  * stiffness-layout switches stay as they are.  Each
  * candidate is timed as the best of three runs after the GPU has been
  * warmed up; shapes within 1% of the fastest count as equal (the earliest

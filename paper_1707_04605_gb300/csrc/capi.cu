@@ -2518,15 +2518,29 @@ int mg_autotune(mg_mesh* M, const double* eps, const mg_shots* shots, const doub
       }
     }
     pick.path = MG_PATH_SHAPE;
-    // the resident kernel, where the problem fits it, against the best of these
+    // the library's own row shape and, wherever the problem fits it, the resident
+    // kernel against the best of these; MG_PATH_AUTO where its estimate chooses the
+    // winner by itself (it chooses anew for other shot counts)
     mg::DevPatches D;
     mg::ResidentShape shape;
-    M->tune[kind] = mg_mesh::Tuning();
-    if (rc == MG_OK) rc = resident_shape(M, kind, S_pad, steps, D, shape);
-    if (rc == MG_OK && shape.lpr) {
-      float t = 0.0f;
-      rc = time_of(kind, pick, &t, MG_PATH_AUTO);
-      if (t < best) pick.path = MG_PATH_AUTO;
+    auto fits = [&](int path) {
+      M->tune[kind].path = path;
+      rc = resident_shape(M, kind, S_pad, steps, D, shape);
+      return rc == MG_OK && shape.lpr > 0;
+    };
+    float t = 0.0f;
+    if (rc == MG_OK) rc = time_of(kind, pick, &t, MG_PATH_ROWS);
+    if (rc == MG_OK && t < best * 0.99f) {
+      best = t;
+      pick.path = MG_PATH_ROWS;
+    }
+    if (rc == MG_OK && fits(MG_PATH_RESIDENT)) {
+      rc = time_of(kind, pick, &t, MG_PATH_RESIDENT);
+      if (rc == MG_OK && t < best) pick.path = MG_PATH_RESIDENT;
+    }
+    if (rc == MG_OK && pick.path != MG_PATH_SHAPE) {
+      const bool resident = fits(MG_PATH_AUTO);
+      if (rc == MG_OK && resident == (pick.path == MG_PATH_RESIDENT)) pick.path = MG_PATH_AUTO;
     }
     M->tune[kind] = pick;
   }

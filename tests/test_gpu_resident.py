@@ -435,3 +435,32 @@ def test_narrow_history_writes_stay_with_the_row_kernels(mg):
     assert n[0] < w.nt                  # resident: 16 launches
     assert n[1] >= w.nt                 # a launch per step
     assert n[2] >= 2.5 * w.nt           # recompute and reverse steps, 16 for the forward
+
+
+@pytest.mark.parametrize("make,kw", [
+    (configs.asteroid_2d, dict(n_refine=3, S=128, nt=96)),     # the resident kernels
+    (configs.ellipsoid_3d, dict(n_refine=2, S=32, nt=64))])    # no patch fits
+def test_a_tuned_handle_is_no_slower_than_an_untuned_one(mg, make, kw):
+    """The default path and the library's own row shape are candidates: the tuned
+    call takes at most 5% more than that of a new handle (three runs of each, the
+    fastest; candidates within 1% count as equal), and gives the same bits."""
+    w = make(**kw)
+    a, b = (mg.mesh_from_workload(w) for _ in range(2))
+    dt, eps = oracle_dt(w), _dev(w.eps)
+    s = _dev(w.wavelet(dt))
+    v = _dev(np.random.default_rng(11).standard_normal(w.mesh.n_cells[0]))
+    a.autotune(eps, w.shots, s, dt, steps=w.nt, level=0)
+    for call in (lambda m: mg.forward(m, eps, w.shots, s, dt),
+                 lambda m: mg.jacobian_apply(m, 0, eps, w.shots, s, dt, v)):
+        best, out = {}, {}
+        for rep in range(4):
+            for name, m in (("tuned", a), ("new", b)):
+                e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+                e0.record()
+                out[name] = call(m)
+                e1.record()
+                torch.cuda.synchronize()
+                if rep:
+                    best[name] = min(best.get(name, 1e9), e0.elapsed_time(e1))
+        assert torch.equal(out["tuned"], out["new"])
+        assert best["tuned"] < 1.05 * best["new"], (best, a.tuning())
