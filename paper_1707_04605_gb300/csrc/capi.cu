@@ -177,7 +177,7 @@ struct mg_mesh {
   Buf trf;                                // forward traces of the fused forward + tangent
   Buf tune_scratch;                       // autotuner inputs/outputs
   std::vector<mg::FluxBuffer> flux_scratch;   // work buffers of the flux path's calls
-  std::mutex flux_mu;                     // guards them and the packed geometry
+  mutable std::mutex flux_mu;             // guards them and the packed geometry
   Buf flux_cell, flux_ptr, flux_inc, flux_pinc;      // its packed geometry
   std::array<Buf, 13> flux_tab;           // and patch tables
   mg::DevFluxPatches flux_patches{};
@@ -1309,8 +1309,9 @@ int mg_mesh_trim(mg_mesh* M) {
     b->p = nullptr;
     b->bytes = 0;
   }
-  for (mg::FluxBuffer& b : M->flux_scratch) cudaFree(b.p);
-  M->flux_scratch.clear();
+  std::vector<mg::FluxBuffer> flux;   // a flux call of another thread may be taking or leaving them
+  mg::mesh_take_scratch(M, flux);
+  for (mg::FluxBuffer& b : flux) cudaFree(b.p);
   M->ev_valid = false;
   M->ck_valid = false;  M->ck_gen++;
   M->seg_full = false;
@@ -1689,14 +1690,19 @@ int mg_mesh_get_info(const mg_mesh* M, mg_mesh_info_t* info) {
                       &M->wav_h, &M->wavf, &M->coef, &M->tcoef, &M->mass, &M->scal, &M->stA,
                       &M->stB, &M->stC, &M->stD, &M->out_h, &M->w_h, &M->v_h, &M->g_h, &M->ev,
                       &M->G, &M->ckpt, &M->seg, &M->gfine, &M->step_base, &M->tr, &M->trf,
-                      &M->xbuf, &M->flux_cell, &M->flux_ptr, &M->flux_inc, &M->flux_pinc};
+                      &M->xbuf};
   for (const Buf* b : all) bytes += (int64_t)b->bytes;
   for (const auto& kv : M->auto_ellc) bytes += (int64_t)kv.second.bytes;
-  for (const Buf& b : M->flux_tab) bytes += (int64_t)b.bytes;
   for (const auto& kv : M->patches)
     for (const auto& g : kv.second.groups)
       for (const Buf& b : g.second.buf) bytes += (int64_t)b.bytes;
-  for (const mg::FluxBuffer& b : M->flux_scratch) bytes += (int64_t)b.bytes;
+  {
+    std::lock_guard<std::mutex> lock(M->flux_mu);
+    for (const Buf* b : {&M->flux_cell, &M->flux_ptr, &M->flux_inc, &M->flux_pinc})
+      bytes += (int64_t)b->bytes;
+    for (const Buf& b : M->flux_tab) bytes += (int64_t)b.bytes;
+    for (const mg::FluxBuffer& b : M->flux_scratch) bytes += (int64_t)b.bytes;
+  }
   info->device_bytes = bytes;
   return MG_OK;
 }

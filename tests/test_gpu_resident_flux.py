@@ -102,3 +102,40 @@ def test_a_large_call_does_not_wait_for_other_streams(mg):
     assert not done.query()
     assert torch.equal(jv, ref)
     torch.cuda.synchronize()
+
+
+def test_trim_and_info_beside_a_call_of_another_thread(mg):
+    """Flux calls of several threads on one handle (each with its own stream and
+    work buffers) while the handle's kept buffers are counted and given back."""
+    import threading
+
+    import torch
+
+    w = configs.asteroid_2d(n_refine=1, S=10, nt=12)
+    m = mg.mesh_from_workload(w)
+    eps = cu(w.eps)
+    dt = 0.5 * mg.cfl_dt(m, eps)
+    s = cu(w.wavelet(dt))
+    ref = mg.forward_pml(m, eps, w.shots, s, dt, allow_cfl=True)
+    torch.cuda.synchronize()
+    wrong, left = [], [3]
+
+    def calls():
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(40):
+                    if not torch.equal(mg.forward_pml(m, eps, w.shots, s, dt, allow_cfl=True), ref):
+                        wrong.append(1)
+        except Exception as e:
+            wrong.append(e)
+        left[0] -= 1
+
+    threads = [threading.Thread(target=calls) for _ in range(left[0])]
+    for t in threads:
+        t.start()
+    while left[0] > 0:
+        assert m.info()["device_bytes"] > 0
+        m.trim()
+    for t in threads:
+        t.join()
+    assert not wrong
