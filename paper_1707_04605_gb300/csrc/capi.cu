@@ -136,6 +136,7 @@ struct mg_mesh {
   int64_t cstride = 0;                    // entries per slice in it
   bool chunked_ell = false;
   std::map<int, Buf> auto_ellc;           // the same for the default launch shapes, by chunk
+  int auto_w = 0;                         // and the widest slice, once one of them is built
   int wu = 0;
   bool uniform_ell = false;
   int cache_hints = 1;                    // kept history: L2 evict-first on last reads
@@ -530,6 +531,7 @@ int ensure_auto_entries(mg_mesh* M, int kind, int cols, cudaStream_t st) {
   int w = 0;
   for (int32_t x : M->hm.slice_w) w = std::max(w, (int)x);
   const int64_t stride = (int64_t)(w + chunk - 1) / chunk * mg::kSliceH * chunk;
+  M->auto_w = w;
   if (ensure(b, (size_t)M->hm.n_slices * stride * sizeof(int2)) != MG_OK)
     return MG_OK;   // no memory: the entries as they are
   M->launches += 1;
@@ -541,11 +543,9 @@ void use_auto_entries(mg_mesh* M, const RowShape& r, int kind, int cols, mg::Dev
   const int chunk = mg::rows_lanes(cols, r.batch, kind == 2 ? r.most_cols : 512);
   auto it = M->auto_ellc.find(chunk);
   if (it == M->auto_ellc.end() || !it->second.p) return;
-  int w = 0;
-  for (int32_t x : M->hm.slice_w) w = std::max(w, (int)x);
   K.ellc = P<const int2>(it->second);
   K.cchunk = chunk;
-  K.cstride = (int64_t)(w + chunk - 1) / chunk * mg::kSliceH * chunk;
+  K.cstride = (int64_t)(M->auto_w + chunk - 1) / chunk * mg::kSliceH * chunk;
 }
 
 int do_step(mg_mesh* M, const mg::StepArgs& a, int S_pad, cudaStream_t st) {
