@@ -11,7 +11,7 @@
 //
 // Bound by shared memory bandwidth: a float4 of a row takes 41 reads and writes
 // of 16 bytes per 4 columns (6 neighbours, self, p_{l-1}, result, entries,
-// coefficients), 77% of the data pipe's peak measured on 413-row patches.
+// coefficients), 75% of the L1 data pipe's peak measured on 413-row patches.
 // Against one launch per step: 62,641 nodes, 128 shots 28.1 -> 13.9 us per step
 // (19.2 with the best row shape); 15,769 nodes, 37 shots 6.4 -> 2.7; 4,225
 // nodes, 1 shot 3.8 -> 1.3; 30,525 nodes of tetrahedra, 24 shots 10.8 -> 5.3.
