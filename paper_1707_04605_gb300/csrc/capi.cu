@@ -792,8 +792,10 @@ int upload_groups(PatchGroups& R) {
 // within 15% of them.  Resident: a launch per column group, each the exchange of
 // border rows, the patch's shared memory accesses (a row read by fewer than 8
 // lanes conflicts with others, less so on triangles, whose neighbours lie side by
-// side) and its halo's.  Row kernels: launch and tail, then the gathers, or the
-// states' traffic when they exceed L2.
+// side) and its halo's; where many narrow launches follow one another (large
+// patches) also their table fills, over the steps of a launch.  Row kernels:
+// launch and tail, then the gathers (fewer than 16 columns run one float4 per
+// lane without the register cap), or the states' traffic when they exceed L2.
 //
 // hist: a step's states also go to a history, `mb` MB of them.  The row kernels
 // write them in whole rows.  A resident launch writes the columns of its group,
@@ -803,14 +805,17 @@ int upload_groups(PatchGroups& R) {
 // step without and with history: 249,697 nodes x 256 shots (one lane, 64
 // launches) 185 and 494 to 625, with row kernels 163 and 181; 197,377 x 256
 // (two lanes) 111 and 168, row kernels 130 and 144; 151,201 x 256 (four) 76 and
-// 99, 100 and 111; 62,641 x 256 (eight) 28.5 and 33, 43 and 48.
+// 99, 100 and 111; 62,641 x 256 (eight) 28.5 and 33, 43 and 48.  The row kernels'
+// rows of 64 and 128 bytes cost more than wider ones: 120,601 x 16 8.1 and 10.0,
+// x 32 10.8 and 12.9.
 double history_us(int lanes, int launches, double mb) {
   const double per_mb = launches == 1 ? 0.1 : lanes >= 8 ? 0.07 : lanes == 4 ? 0.15
-                        : lanes == 2 ? 0.27 : std::min(1.7, 0.08 * launches);
+                        : lanes == 2 ? std::min(0.28, 0.08 * launches)
+                                     : std::min(1.7, 0.08 * launches);
   return per_mb * mb;
 }
 double resident_us(const mg::DevPatches& D, const mg::ResidentShape& s, int kind, int S_pad,
-                   double mb) {
+                   int steps, double mb) {
   const bool tri = D.uniform == 3;
   const double conflicts = s.lpr >= 8   ? 1.0
                            : s.lpr == 4 ? (tri ? 1.15 : 1.5)
@@ -819,16 +824,21 @@ double resident_us(const mg::DevPatches& D, const mg::ResidentShape& s, int kind
   const double pairs = (double)D.max_pairs / (D.max_groups * (32 / s.lpr));
   const double group = 14.0 + pairs * (1.0 + 8.0 * conflicts) + (kind == 1 ? 6.0 : kind == 2 ? 12.0 : 0.0);
   const int launches = S_pad / (kind == 1 ? 2 * s.lpr : 4 * s.lpr);
-  return launches * (0.9 + 0.65e-3 * group * D.max_groups + 0.3e-3 * D.max_halo * 2 * s.lpr) +
+  const double fill = s.lpr <= 2 ? 12.0 / steps : 0.0;
+  return launches * (0.9 + 0.65e-3 * group * D.max_groups + 0.3e-3 * D.max_halo * 2 * s.lpr + fill) +
          history_us(kind == 1 ? s.lpr / 2 : s.lpr, launches, mb);
 }
 double rows_us(const mg_mesh* M, int kind, int S_pad, double mb) {
   const double work = (double)M->hm.rowptr.back() * S_pad, cols = (double)M->hm.n * S_pad;
-  const double gathers = 4.0 + (kind == 0 ? 0.27e-6 : kind == 1 ? 0.5e-6 : 0.38e-6) * work;
+  const bool tri = M->hm.rowptr.back() < 8 * M->hm.n;
+  const double gathers = kind == 0   ? 4.0 + (S_pad < 16 ? 0.4e-6 : 0.27e-6) * work
+                         : kind == 2 ? 4.0 + 0.38e-6 * work
+                         : tri       ? 4.5 + 0.54e-6 * work
+                                     : 4.0 + 0.5e-6 * work;
   const double held = (kind == 1 ? 16.0 : 8.0) * cols;   // bytes of the states of a step
   const double moved = (kind == 0 ? 12.0 : kind == 1 ? 24.0 : 16.0) * cols;
-  const double hist = (kind == 0 ? 0.07 : 0.01) * mb;
-  if (held < (kind == 1 ? 80e6 : 100e6)) return gathers + hist;
+  const double hist = (kind == 1 ? 0.02 : S_pad == 16 ? 0.2 : S_pad == 32 ? 0.14 : 0.07) * mb;
+  if (held < (kind == 1 ? 65e6 : 100e6)) return gathers + hist;
   const double rate = kind == 1 ? (held < 200e6 ? 3.8e6 : 4.2e6) : held < 150e6 ? 4.1e6 : 4.5e6;
   return std::max(gathers, moved / rate) + hist;
 }
@@ -868,7 +878,7 @@ int resident_shape(mg_mesh* M, int kind, int S_pad, int steps, mg::DevPatches& D
   if (!shape.lpr) return MG_OK;
   const double mb = hist ? 4e-6 * (double)M->hm.n * S_pad : 0.0;
   if ((path == MG_PATH_AUTO || hist) &&
-      resident_us(R->dev, shape, kind, S_pad, mb) > rows_us(M, kind, S_pad, mb)) {
+      resident_us(R->dev, shape, kind, S_pad, steps, mb) > rows_us(M, kind, S_pad, mb)) {
     shape.lpr = 0;
     R->host.reset();
     return MG_OK;
