@@ -919,12 +919,8 @@ int poison(mg_mesh* M, float* x, int64_t n, bool reused, cudaStream_t st) {
 int note_kept(mg_mesh* M, cudaStream_t st) {
   if (!M->errbuf.p) return MG_OK;
   int* w = P<int>(M->errbuf);
-  if (M->status_clear)
-    MG_CU(cudaMemcpyAsync(w + kWordKept, w + kWordStatus, sizeof(int), cudaMemcpyDeviceToDevice,
-                          st));
-  else
-    MG_CU(cudaMemsetAsync(w + kWordKept, 0, sizeof(int), st));
-  return MG_OK;
+  M->launches += 1;
+  return mg::launch_note_kept(M->status_clear ? w + kWordStatus : nullptr, w + kWordKept, st);
 }
 
 mg::ResidentArgs resident_args(mg_mesh* M, const Prep& pp, int nt, const mg::DevPatches& D) {

@@ -9,6 +9,8 @@
 namespace mg {
 namespace {
 
+__global__ void k_note_kept(const int* status, int* kept) { *kept = status ? *status : 0; }
+
 // (a may be status: every block finds it set, whoever comes first)
 __global__ void k_poison(float* x, int64_t n, const int* a, const int* b, int* status,
                          int* count) {
@@ -62,6 +64,11 @@ int launch_resident_step(const ResidentArgs& a, const ResidentShape& s, cudaStre
     case 32: return launch_lpr<32, false>(a, s, st);
   }
   return MG_ERR_ARG;
+}
+
+int launch_note_kept(const int* status, int* kept, cudaStream_t st) {
+  k_note_kept<<<1, 1, 0, st>>>(status, kept);
+  return check_launch();
 }
 
 int launch_poison(float* x, int64_t n, const int* a, const int* b, int* status, int* count,
