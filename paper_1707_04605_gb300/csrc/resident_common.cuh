@@ -159,7 +159,10 @@ __device__ __forceinline__ Patch patch_tables(const DevPatches& D, unsigned char
 // compute, store, the neighbour's copy) is then the longer one.  Measured, us
 // per step with 1, 1.3, 1.6, 2 times the share: 104 groups (20% border) 14.7,
 // 14.6, 13.9, 14.3; 53 groups (40%) 2.67, 2.85, 2.92, 2.94; 50 groups of a
-// tetrahedral patch (70%) 5.3, 7.4, 9.4, 9.4.
+// tetrahedral patch (70%) 5.3, 7.4, 9.4, 9.4.  Around a third, forward and tangent
+// of 64 shots with once and 1.6 times the share: 42% border 2.3, 4.2 and 2.2,
+// 8.3; 37% 2.4, 4.8 and 2.6, 5.3; 34% 2.7, 5.7 and 2.7, 6.4; 31% 3.2, 7.2 and
+// 2.9, 6.8; 22% (32 shots) 3.2, 7.2 and 2.9, 6.7.
 __device__ __forceinline__ int border_warps_of(int gb, int ng, int warps) {
   if (ng <= warps) return max(gb, 1);
   const int share = gb * warps / ng;
